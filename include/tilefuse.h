@@ -104,8 +104,8 @@ typedef struct tf_blob_header {
 } tf_blob_header;
 
 /* Bytes of the packed blob, or 0 if the shape is illegal.
- * Legal: bits in {4, 8}; 128 <= K <= TF_MAX_DIM; 8 <= N <= TF_MAX_DIM; N % 8 == 0; K % group_size == 0;
- * group_size % 128 == 0, or, for bits == 4, group_size 64 or 32 (the tile then carries two or four
+ * Legal: bits in {4, 8}; 128 <= K <= TF_MAX_DIM; 8 <= N <= TF_MAX_DIM; N % 8 == 0; K % 128 == 0;
+ * K % group_size == 0; group_size % 128 == 0, or, for bits == 4, group_size 64 or 32 (the tile then carries two or four
  * scale and zero-point blocks, group after group along k: 4416 or 4736 bytes per tile). */
 size_t tf_packed_size(int bits, int K, int N, int group_size);
 
@@ -338,7 +338,7 @@ tf_status tf_pack_awq_device(const uint32_t* qweight, const uint16_t* scales_fp1
  * GEMM arm of the layout ablation (Section 5.5): the fused W4A16 GEMM computed from the AWQ arrays as given, with no
  * offline pre-tiling -- the arrays are re-tiled into scratch memory on every call (tf_pack_awq_device) and multiplied
  * by the pre-tiled GEMM.  The difference to tf_gemm_w4a16 on an offline blob is the cost the offline pre-tiling of
- * Section 4.2 removes.  Arguments as tf_gemv_awq_raw, 1 <= M <= 4096, group_size 32, 64 or a multiple of 128;
+ * Section 4.2 removes.  Arguments as tf_gemv_awq_raw, 1 <= M <= 4096, K % 128 == 0, group_size 32, 64 or a multiple of 128;
  *   workspace   device, at least tf_gemm_awq_raw_workspace_size(M, K, N, group_size) bytes (the GEMM's workspace,
  *               then the re-tiled blob); its first TF_WORKSPACE_ZERO_BYTES must be zero before first use and are left
  *               zero; tf_device_status reads its status word.

@@ -23,6 +23,7 @@ bool legal_shape(int bits, int K, int N, int g) {
     if (bits != 4 && bits != 8) return false;
     if (K < tf::kTileK || K > TF_MAX_DIM || N < 8 || N > TF_MAX_DIM) return false;
     if (N % 8 != 0) return false;
+    if (K % tf::kTileK != 0) return false;         // also for group sizes below the tile: rows behind the last whole tile would be in none
     if (g <= 0 || K % g != 0) return false;
     if (g % tf::kTileK == 0) return true;
     return bits == 4 && (g == 64 || g == 32);      // several groups inside a tile: the 4-bit format only

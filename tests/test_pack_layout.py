@@ -1,4 +1,6 @@
 """tf_pack_awq / tf_pack_w8 on the host: header, determinism, and layout read back == oracle unpack."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -94,6 +96,23 @@ def test_group_sizes_that_are_not_legal():
     assert tf.tf_packed_size(4, 1024, 64, 16) == 0 and tf.tf_packed_size(4, 1024, 64, 48) == 0
     assert tf.tf_packed_size(8, 1024, 64, 64) == 0           # below the tile: the 4-bit format only
     assert tf.tf_packed_size(4, 1024, 64, 64) > 0 and tf.tf_packed_size(4, 1024, 64, 32) > 0
+
+
+@pytest.mark.parametrize("K,g", [(192, 64), (160, 32), (4096 + 64, 64), (32768 - 32, 32)])
+def test_k_must_be_whole_tiles_whatever_the_group_size(K, g):
+    """A K that is whole groups but not whole 128-row tiles has no blob: its last rows would be in no tile."""
+    L, ok, N = tf.lib(), ctypes.c_void_p(0x1000), 64
+    assert tf.tf_packed_size(4, K, N, g) == 0
+    with pytest.raises(tf.TileFuseError) as e:
+        tf.tf_pack_awq(np.zeros((K, N // 8), np.uint32), np.zeros((K // g, N), np.float16), np.zeros((K // g, N // 8), np.uint32), K, N, g)
+    assert e.value.status == 2
+    # ... and every call on such a shape says so, before any CUDA call
+    assert L.tf_pack_awq_device(ok, ok, ok, K, N, g, ok, 1 << 30, None) == 2
+    assert L.tf_unpack_w4(ok, ok, ok, ok, K, N, g, None) == 2
+    assert L.tf_gemv_w4a16_grouped(ok, ok, ok, 1, K, N, g, ok, 1 << 30, None) == 2
+    assert L.tf_gemm_w4a16_grouped(ok, ok, ok, 1, K, N, g, ok, 1 << 30, None) == 2
+    assert L.tf_gemm_awq_raw(ok, ok, ok, ok, ok, 1, K, N, g, ok, 1 << 30, None) == 2
+    assert tf.tf_gemm_awq_raw_workspace_size(1, K, N, g) == 0
 
 
 def test_blob_is_tile_major_and_contiguous_per_strip():
