@@ -118,20 +118,19 @@ PyObject* call(PyObject* self, PyObject* const* args, Py_ssize_t nargs, PyObject
         given[at] = args[nargs + k];
     }
     Arg x[kMaxArgs];
-    for (int i = 0; i < c.count; ++i) {
-        if (given[i] == nullptr) return PyErr_Format(PyExc_TypeError, "%s() missing required argument: '%s'", c.name, c.names[i]);
-        if (!(c.kinds[i] == 't' ? convert_tensor(given[i], &x[i]) : convert_int(given[i], &x[i]))) return nullptr;
-    }
-    tf_status status;
+    void* stream = nullptr;
     try {
-        void* stream = nullptr;
+        for (int i = 0; i < c.count; ++i) {
+            if (given[i] == nullptr) return PyErr_Format(PyExc_TypeError, "%s() missing required argument: '%s'", c.name, c.names[i]);
+            if (!(c.kinds[i] == 't' ? convert_tensor(given[i], &x[i]) : convert_int(given[i], &x[i]))) return nullptr;
+        }
         if (!convert_stream(given[c.count], &stream)) return nullptr;
-        PyThreadState* released = PyEval_SaveThread();
-        status = c.make(x, stream);
-        PyEval_RestoreThread(released);
-    } catch (const std::exception& e) {          // torch has no current stream to give (no device)
+    } catch (const std::exception& e) {          // torch: a tensor without memory of its own (under vmap), no device to ask for a stream
         return PyErr_Format(PyExc_RuntimeError, "%s(): %.500s", c.name, e.what());
     }
+    PyThreadState* released = PyEval_SaveThread();
+    const tf_status status = c.make(x, stream);  // C calls, which do not throw
+    PyEval_RestoreThread(released);
     if (status != TF_OK) {
         PyObject* r = PyObject_CallFunction(g_raise, "si", c.name, static_cast<int>(status));
         Py_XDECREF(r);

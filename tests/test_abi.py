@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -111,3 +113,28 @@ def test_device_calls_check_their_arguments_before_the_library_is_called():
         with pytest.raises(tf.TileFuseError) as e:
             call(None, a=None, y=None, M=1, K=128, N=8, workspace=None, stream=Stream)
         assert e.value.status == 1
+
+
+def test_a_tensor_without_memory_is_an_exception_not_an_abort():
+    """torch throws when such a tensor (here one under vmap) is asked for its address; no C++ exception may leave the binding."""
+    code = """
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+from paper_2606_11357_b200 import binding as tf
+class Stream:
+    cuda_stream = 0
+raised = []
+def f(v):
+    for _ in range(2):                                          # the call that loads the native module, and the next one
+        try:
+            tf.tf_gemv_w4a16(v, v, v, 1, 128, 8, v, Stream)
+        except RuntimeError as e:
+            raised.append(str(e))
+    return v
+with FakeTensorMode():                                          # a CUDA tensor on a machine without a GPU
+    torch.vmap(f)(torch.empty(2, 16, dtype=torch.uint8, device="cuda"))
+assert len(raised) == 2 and all("tf_gemv_w4a16" in r and "storage" in r for r in raised), raised
+print("both raised")
+"""
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and "both raised" in res.stdout, (res.returncode, res.stderr[-2000:])
