@@ -120,6 +120,9 @@ def _native_calls() -> dict:
     if not os.path.exists(_NATIVE_PATH):
         raise ImportError(f"{_NATIVE_PATH} is missing: build it with `python -m paper_2606_11357_b200.build` "
                           "(there is no fallback path)")
+    from . import build
+    if not build.native_is_current():
+        raise ImportError(f"{_NATIVE_PATH} was built for another torch or Python: build it again with `python -m paper_2606_11357_b200.build`")
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
     loader.exec_module(module)
     calls = module.calls(_check)

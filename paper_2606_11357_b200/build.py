@@ -5,6 +5,7 @@ import os
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
+from importlib.metadata import version
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
@@ -44,6 +45,19 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _native_target() -> str:
+    """What the binding's CPython module is built for: it uses torch's C++ interface, which changes with every release, and Python's."""
+    return f"tilefuse native for torch {version('torch')}, {sys.implementation.cache_tag}"
+
+
+def native_is_current() -> bool:
+    """The module carries its target as a string: no file beside it can get lost or be about another build."""
+    if not os.path.exists(NATIVE):
+        return False
+    with open(NATIVE, "rb") as f:
+        return _native_target().encode() + b"\0" in f.read()
+
+
 def _compile_native() -> None:
     """The binding's CPython module: host code only, against the headers of Python and of torch."""
     import sysconfig
@@ -53,7 +67,8 @@ def _compile_native() -> None:
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     include = [sysconfig.get_paths()["include"], os.path.join(torch, "include"),
                os.path.join(torch, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
-    cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden", os.path.join(CSRC, "native.cpp"), "-o", NATIVE,
+    cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden", f'-DTF_NATIVE_TARGET="{_native_target()}"',
+           os.path.join(CSRC, "native.cpp"), "-o", NATIVE,
            *[a for d in include for a in ("-isystem", d)], "-L" + PKG, "-l:libtilefuse.so", "-Wl,-rpath,$ORIGIN",
            "-L" + os.path.join(torch, "lib"), "-ltorch_python", "-lc10_cuda", "-lc10", "-ltorch_cpu"]
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -64,8 +79,15 @@ def _compile_native() -> None:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every source for sm_100a and link the shared library; returns its path."""
     newest = _deps_mtime()
-    if not force and all(os.path.exists(p) and os.path.getmtime(p) >= newest for p in (LIB, NATIVE)):
-        return LIB
+    fresh = [not force and os.path.exists(p) and os.path.getmtime(p) >= newest for p in (LIB, NATIVE)]
+    if not fresh[0]:
+        _compile_library(verbose)
+    if not (all(fresh) and native_is_current()):
+        _compile_native()
+    return LIB
+
+
+def _compile_library(verbose: bool) -> None:
     os.makedirs(OBJ, exist_ok=True)
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as pool:
         objs = list(pool.map(lambda s: _compile(s, verbose), SOURCES))
@@ -74,8 +96,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
-    _compile_native()
-    return LIB
 
 
 if __name__ == "__main__":

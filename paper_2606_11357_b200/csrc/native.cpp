@@ -169,6 +169,11 @@ PyMethodDef g_calls_def = {"calls", calls, METH_O, nullptr};
 PyMODINIT_FUNC PyInit__native(void) {
     PyObject* m = PyModule_Create(&g_module);
     if (m == nullptr) return nullptr;
+    // the torch and the Python this file was compiled against; the build looks for it in the module before it is loaded
+    if (PyModule_AddStringConstant(m, "TARGET", TF_NATIVE_TARGET) != 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
     PyObject* f = PyCFunction_NewEx(&g_calls_def, nullptr, nullptr);
     if (f == nullptr || PyModule_AddObject(m, "calls", f) != 0) {
         Py_XDECREF(f);

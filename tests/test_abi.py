@@ -138,3 +138,20 @@ print("both raised")
 """
     res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and "both raised" in res.stdout, (res.returncode, res.stderr[-2000:])
+
+
+def test_native_module_of_another_torch_is_built_again_and_not_loaded(monkeypatch):
+    """torch's C++ interface changes with its releases: a module built for another one is stale whatever its date."""
+    compiled = []
+    monkeypatch.setattr(tfbuild, "_compile_native", lambda: compiled.append("native"))
+    monkeypatch.setattr(tfbuild, "_compile_library", lambda verbose: compiled.append("library"))
+    tfbuild.build()
+    assert tfbuild.native_is_current() and compiled == []
+    for name in ("2.11", "99.0.0"):                             # (the installed version's beginning is another version too)
+        monkeypatch.setattr(tfbuild, "version", lambda package: name)
+        assert not tfbuild.native_is_current()
+        tfbuild.build()
+        assert compiled == ["native"]
+        compiled.clear()
+    with pytest.raises(ImportError, match="another torch"):
+        tf._native_calls()
