@@ -957,6 +957,68 @@ static int max_resident_clusters(int csize, bool full) {
     return entry > 0 ? entry : 0;
 }
 
+// The part of a plan that follows from its form (whole SM or half): consumer warps, ring, piece table, shared memory.
+static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool full) {
+    const int mt = M <= 8 ? 1 : 2;
+    p.full = full;
+    // whole-SM integer path: about 66 KB of tiles in the consumer warps' hands (16 warps on 4-bit tiles, 8 on int8 tiles)
+    // and the rest of the ring in flight.  Measured alone, one token: 4096x32768 4-bit 20.7 us half SM, 20.7 / 18.8 /
+    // 18.1 whole SM with 8 / 12 / 16 warps; 4096x14336 int8 15.8 us half SM, 12.7 / 13.3 / 14.6 whole SM with 8 / 12 / 16.
+    p.consumers = p.i8 && p.full ? gemv_i8_full_consumers(bits) : gemv_max_consumers(mt, p.full);
+    // Floating-point path up to 8 tokens: 12 warps only for long ranges of 4-bit tiles.  Eight have fewer partial sums to add up
+    // at the end of a strip and less of the ring in their hands: 4 tokens 4096x4096 5.54 us against 5.83 with 12, x6144 7.19 and
+    // 7.50, x8192 7.90 and 8.00, then x9472 7.68 and 7.57, x28672 16.35 and 15.75; int8 8 tokens 4096x4096 6.65 and 6.90, x9472
+    // 9.79 and 10.24, x28672 21.5 and 22.3.  (10, 11 and 14 warps are slower than 8, 12 and 16 everywhere, 14336x4096 11.1 us
+    // against 10.6: with a multiple of the tiles of a chunk a warp always works on the same place of a stage, and a stage is
+    // freed by warps that are about equally far.)
+    if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < kGemvFpTwelveWarpsFromTiles)) p.consumers = 8;
+    if (tiles_per_cta < p.consumers) p.consumers = tiles_per_cta < 4 ? 4 : tiles_per_cta;
+    p.threads = 32 * (p.consumers + 2);          // + producer warp + reducer warp
+    const int kr = gemv_chunk_tiles(bits);
+    // a stage: one bulk copy of kR packed tiles, padded, and on the floating-point path their activations
+    p.stage_bytes = p.i8 ? kGemvStageBytes : (kr * tile_bytes(bits, p.groups) + 127) / 128 * 128;
+    const int act_stage_bytes = p.i8 ? 0 : kr * gemv_act_tile_bytes(mt);
+    // cluster mode: one slot per CTA of the cluster for the rows of real tokens (two token rows = 512 bytes)
+    p.xslot_bytes = p.cluster > 1 ? ((M + 1) / 2) * 512 : 0;
+    // two buffers for the consumer warps' partial sums where the whole SM is taken (a boundary between strips then
+    // costs a fast warp nothing; measured below), one in the half-SM form, where the second would cost a ring stage
+    p.nred = p.full ? 2 : 1;
+    const int base = 1024 /*alignment slack*/ + kGemvBarrierBytes + p.nred * p.consumers * (p.i8 ? 2 : 8 * mt) * kTileN * 4 +
+                     (p.cluster * p.xslot_bytes + 1023) / 1024 * 1024;
+    int fixed = base + (p.i8 ? p.consumers * 1024 : 0);
+    int stages = (gemv_smem_budget(mt, p.full) - fixed) / (p.stage_bytes + act_stage_bytes);
+    if (stages > kGemvMaxStages) stages = kGemvMaxStages;
+    // no more stages than the range has chunks
+    const int chunks = (tiles_per_cta + kr - 1) / kr + 2;
+    if (stages > chunks) stages = chunks;
+    // whole-SM integer path: a ring deeper than eight stages was slower (1x4096x32768 4-bit: 17.0 / 16.9 / 17.5 us with
+    // 6 / 8 / 10 stages; int8 1x4096x14336: 12.8 / 12.5 / 12.7 us with 6 / 8 / 11)
+    if (p.i8 && p.full && stages > kGemvI8FullMaxStages) stages = kGemvI8FullMaxStages;
+    // floating-point path up to 8 tokens on 4-bit tiles: five stages (three in the hands of the 12 consumer warps, two in
+    // flight).  Measured at 4 tokens with 4 / 5 / 6 / 7 / 9 stages: 4096x14336 12.2 / 11.6 / 11.7 / 11.9 / 12.3 us,
+    // 4096x32768 20.9 / 19.8 / 19.9 / 20.1 / 20.5 us; int8 tiles (six stages in the warps' hands) want the deep ring:
+    // 4096x14336 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us.  (Why a deeper ring is slower on 4-bit tiles was not established;
+    // the consumers, not HBM, set the pace of this path.)
+    if (!p.i8 && mt == 1 && bits == 4 && stages > kGemvFpW4MaxStages) stages = kGemvFpW4MaxStages;
+    // Integer path: where a range passes over the same k-tiles more than once and K is a multiple of 128 x consumer
+    // warps, every warp meets the same k-tiles on each pass and keeps the activation pieces it has prepared (one table
+    // entry per k-tile instead of one scratch entry per warp), if that costs the ring no stage.
+    p.piece_tab = 0;
+    // (4-bit weights only: on int8 tiles, whole SM, the table was the slower form, 13.1 against 12.5 us on 1x4096x14336)
+    if (p.i8 && bits == 4 && tiles_per_cta >= p.ktiles + p.consumers && p.ktiles % p.consumers == 0) {
+        const int table = (p.ktiles * kGemvPieceEntryBytes * M + 1023) / 1024 * 1024;
+        int with = (gemv_smem_budget(mt, p.full) - (base + table)) / p.stage_bytes;
+        if (with > kGemvMaxStages) with = kGemvMaxStages;
+        if (with > chunks) with = chunks;
+        if (with >= stages) {
+            p.piece_tab = p.ktiles;
+            fixed = base + table;
+        }
+    }
+    p.stages = stages;
+    p.smem_bytes = fixed + p.stages * (p.stage_bytes + act_stage_bytes);
+}
+
 // Launch geometry.  Global mode: one persistent CTA per SM (fewer when there are fewer tiles than SMs), all tiles
 // cut into equal ranges; a strip cut between CTAs is summed through the workspace.  Cluster mode: clusters of 2, 4
 // or 8 CTAs, each cluster owning whole strips and cutting its tiles into equal ranges among its CTAs; a cut strip
@@ -1029,71 +1091,17 @@ GemvPlan plan_gemv(int bits, int M, int K, int N, int sm_count, int groups) {
         p.nclusters = active;
         if (mt == 1 && p.grid < sm_count) p.grid = sm_count;
     }
-    // The floating-point path is bound by instruction issue in its consumer warps: it takes the whole SM (12 consumer
-    // warps, deeper ring).  The integer path of 1 and 2 tokens needs a fraction of the instructions; its short ranges
-    // gain more from the next GEMV's CTAs sitting beside this one's with their rings already full, long ones
-    // amortise the start of the kernel and take the whole SM too.
-    const bool i8_path = M <= kGemvI8MaxM && groups == 1;     // several groups per tile: floating-point path only
-    const bool kept = bits == 4 && M == 1 && p.ktiles % gemv_max_consumers(1, false) == 0 && tiles_per_cta >= p.ktiles + gemv_max_consumers(1, false);
-    p.full = mt == 2 || !i8_path ||
-             tiles_per_cta * tile_bytes(bits, groups) >= (bits == 8 ? kGemvFullFromBytesI8W8 : kept ? kGemvFullFromBytesI8W4Kept : kGemvFullFromBytesI8W4);
-    p.i8 = i8_path && p.cluster == 1;
-    // whole-SM integer path: about 66 KB of tiles in the consumer warps' hands (16 warps on 4-bit tiles, 8 on int8 tiles)
-    // and the rest of the ring in flight.  Measured alone, one token: 4096x32768 4-bit 20.7 us half SM, 20.7 / 18.8 /
-    // 18.1 whole SM with 8 / 12 / 16 warps; 4096x14336 int8 15.8 us half SM, 12.7 / 13.3 / 14.6 whole SM with 8 / 12 / 16.
-    p.consumers = p.i8 && p.full ? gemv_i8_full_consumers(bits) : gemv_max_consumers(mt, p.full);
-    // Floating-point path up to 8 tokens: 12 warps only for long ranges of 4-bit tiles.  Eight have fewer partial sums to add up
-    // at the end of a strip and less of the ring in their hands: 4 tokens 4096x4096 5.54 us against 5.83 with 12, x6144 7.19 and
-    // 7.50, x8192 7.90 and 8.00, then x9472 7.68 and 7.57, x28672 16.35 and 15.75; int8 8 tokens 4096x4096 6.65 and 6.90, x9472
-    // 9.79 and 10.24, x28672 21.5 and 22.3.  (10, 11 and 14 warps are slower than 8, 12 and 16 everywhere, 14336x4096 11.1 us
-    // against 10.6: with a multiple of the tiles of a chunk a warp always works on the same place of a stage, and a stage is
-    // freed by warps that are about equally far.)
-    if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < kGemvFpTwelveWarpsFromTiles)) p.consumers = 8;
-    if (tiles_per_cta < p.consumers) p.consumers = tiles_per_cta < 4 ? 4 : tiles_per_cta;
-    p.threads = 32 * (p.consumers + 2);          // + producer warp + reducer warp
-    const int kr = gemv_chunk_tiles(bits);
-    // a stage: one bulk copy of kR packed tiles, padded, and on the floating-point path their activations
-    p.stage_bytes = p.i8 ? kGemvStageBytes : (kr * tile_bytes(bits, groups) + 127) / 128 * 128;
-    const int act_stage_bytes = p.i8 ? 0 : kr * gemv_act_tile_bytes(mt);
-    // cluster mode: one slot per CTA of the cluster for the rows of real tokens (two token rows = 512 bytes)
-    p.xslot_bytes = p.cluster > 1 ? ((M + 1) / 2) * 512 : 0;
-    // two buffers for the consumer warps' partial sums where the whole SM is taken (a boundary between strips then
-    // costs a fast warp nothing; measured below), one in the half-SM form, where the second would cost a ring stage
-    p.nred = p.full ? 2 : 1;
-    const int base = 1024 /*alignment slack*/ + kGemvBarrierBytes + p.nred * p.consumers * (p.i8 ? 2 : 8 * mt) * kTileN * 4 +
-                     (p.cluster * p.xslot_bytes + 1023) / 1024 * 1024;
-    int fixed = base + (p.i8 ? p.consumers * 1024 : 0);
-    int stages = (gemv_smem_budget(mt, p.full) - fixed) / (p.stage_bytes + act_stage_bytes);
-    if (stages > kGemvMaxStages) stages = kGemvMaxStages;
-    // no more stages than the range has chunks
-    const int chunks = (tiles_per_cta + kr - 1) / kr + 2;
-    if (stages > chunks) stages = chunks;
-    // whole-SM integer path: a ring deeper than eight stages was slower (1x4096x32768 4-bit: 17.0 / 16.9 / 17.5 us with
-    // 6 / 8 / 10 stages; int8 1x4096x14336: 12.8 / 12.5 / 12.7 us with 6 / 8 / 11)
-    if (p.i8 && p.full && stages > kGemvI8FullMaxStages) stages = kGemvI8FullMaxStages;
-    // floating-point path up to 8 tokens on 4-bit tiles: five stages (three in the hands of the 12 consumer warps, two in
-    // flight).  Measured at 4 tokens with 4 / 5 / 6 / 7 / 9 stages: 4096x14336 12.2 / 11.6 / 11.7 / 11.9 / 12.3 us,
-    // 4096x32768 20.9 / 19.8 / 19.9 / 20.1 / 20.5 us; int8 tiles (six stages in the warps' hands) want the deep ring:
-    // 4096x14336 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us.  (Why a deeper ring is slower on 4-bit tiles was not established;
-    // the consumers, not HBM, set the pace of this path.)
-    if (!p.i8 && mt == 1 && bits == 4 && stages > kGemvFpW4MaxStages) stages = kGemvFpW4MaxStages;
-    // Integer path: where a range passes over the same k-tiles more than once and K is a multiple of 128 x consumer
-    // warps, every warp meets the same k-tiles on each pass and keeps the activation pieces it has prepared (one table
-    // entry per k-tile instead of one scratch entry per warp), if that costs the ring no stage.
-    p.piece_tab = 0;
-    // (4-bit weights only: on int8 tiles, whole SM, the table was the slower form, 13.1 against 12.5 us on 1x4096x14336)
-    if (p.i8 && bits == 4 && tiles_per_cta >= p.ktiles + p.consumers && p.ktiles % p.consumers == 0) {
-        const int table = (p.ktiles * kGemvPieceEntryBytes * M + 1023) / 1024 * 1024;
-        int with = (gemv_smem_budget(mt, p.full) - (base + table)) / p.stage_bytes;
-        if (with > kGemvMaxStages) with = kGemvMaxStages;
-        if (with > chunks) with = chunks;
-        if (with >= stages) {
-            p.piece_tab = p.ktiles;
-            fixed = base + table;
-        }
+    p.i8 = M <= kGemvI8MaxM && groups == 1 && p.cluster == 1;     // several groups per tile: floating-point path only
+    // The floating-point path and 9..16 tokens take the whole SM: they are bound by what their consumer warps do, and only one
+    // kernel's consumers work at a time.  The integer path of 1 and 2 tokens needs a fraction of the instructions; its short
+    // ranges gain more from the next GEMV's CTAs sitting beside this one's with their rings already full, long ones amortise
+    // the start of the kernel and take the whole SM too.  Where the line lies depends on whether the half-SM form keeps its
+    // activation pieces, so that form is laid out first.
+    lay_out_gemv(p, bits, M, tiles_per_cta, !p.i8);
+    if (!p.full) {
+        const int whole_from = bits == 8 ? kGemvFullFromBytesI8W8 : p.piece_tab > 0 ? kGemvFullFromBytesI8W4Kept : kGemvFullFromBytesI8W4;
+        if (tiles_per_cta * tile_bytes(bits, groups) >= whole_from) lay_out_gemv(p, bits, M, tiles_per_cta, true);
     }
-    p.stages = stages;
-    p.smem_bytes = fixed + p.stages * (p.stage_bytes + act_stage_bytes);
     return p;
 }
 

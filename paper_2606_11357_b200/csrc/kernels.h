@@ -47,10 +47,17 @@ constexpr int kGemvPieceEntryBytes = 512;
 // their rings full.
 constexpr int kGemvFullFromBytesI8W4 = TF_I8_FULL_BYTES_W4;
 constexpr int kGemvFullFromBytesI8W8 = TF_I8_FULL_BYTES_W8;
-// One token and 4-bit tiles whose activation pieces are kept: a tile costs a half-SM CTA so little that its short start and the
-// neighbour's full ring win up to longer ranges (1x4096x20480 10.7 us half SM, 11.6 whole; x28672 13.3 and 13.5; x32768
-// 14.6 and 14.8), and a chain that stays on half SMs has no change of form to pay for: the four GEMVs of a layer with
-// 4096x28672 among them 36.0 -> 34.7 us.
+// 4-bit tiles, the half-SM form without / with its activation pieces kept (piece table).  Figures: us per call in a chain of one
+// shape, one token, half SM / whole SM.
+// Without the table a tile costs a half-SM warp its preparation as well, and eight warps fall behind sixteen: 3584x24576 (303 KB)
+// 12.75 / 11.93, 5120x16384 (291 KB) 12.30 / 11.26, x20480 14.87 / 13.46, 7168x16384 15.41 / 13.45, 9216x12288 15.22 / 13.44.  (In such
+// a chain the forms cross near 235 KB, 3584x18944 9.80 / 9.74, 8192x10240 12.12 / 11.23; the line is at 288 KB, since a pass that goes
+// from half-SM calls to a whole-SM one pays for the change, about 1 us.)
+// With it a tile costs so little that the short start and the neighbour's full ring win: 3072x32768 (349 KB) 12.57 / 13.38,
+// 4096x20480 (287 KB) 11.07 / 11.59, x28672 (403 KB) 13.87 / 14.04; then the two are level: x30720 (432 KB) 14.82 / 14.77, x32768
+// (461 KB) 15.38 / 15.44.  And a pass that stays on half SMs changes no form: the four GEMVs of a layer with 4096x28672 among
+// them 36.0 -> 34.7 us.  The table fits for K of 1024 to 4096 (multiples of 1024) at one token; at two tokens for 1024 and 2048, whose
+// ranges stay below 288 KB (without it 4096x20480 13.62 / 12.13, 3072x26624 13.60 / 12.67).
 constexpr int kGemvFullFromBytesI8W4Kept = 448 * 1024;
 __host__ __device__ constexpr int gemv_i8_full_consumers(int bits) { return bits == 8 ? 8 : 16; }
 constexpr int kGemvI8FullMaxStages = 8;

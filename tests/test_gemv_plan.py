@@ -71,6 +71,32 @@ def test_plan_of_the_benchmark_shapes_on_a_b200():
     assert p["nclusters"] == 128                                         # 128 CTAs x 16 tiles: ranges line up with the strips
 
 
+@pytest.mark.parametrize("M", [1, 2])
+def test_form_of_the_integer_path_follows_the_piece_table(M):
+    """Long ranges of 4-bit tiles stay on half an SM only where the activation pieces are kept there, which is a matter of whether the
+    table fits: K of 1024, 2048, 3072 and 4096 at one token, 1024 and 2048 at two.  Without it, from 288 KB on: the whole SM."""
+    kept_from_288 = set()
+    for K in range(128, 32768 + 1, 128):
+        for N in range(512, 32768 + 1, 512):
+            p = tf.tf_gemv_plan(4, M, K, N, 148)
+            packed = -(-(K // 128 * N // 64) // p["nclusters"]) * 4256   # packed bytes of a CTA's range
+            if p["full"]:
+                assert packed >= 288 * 1024
+            elif packed >= 288 * 1024:
+                assert p["i8"] == 2 and packed < 448 * 1024
+                kept_from_288.add(K)
+            if not p["full"] and p["i8"] == 2:
+                assert p["stages"] == 5 and K in ((1024, 2048, 3072, 4096) if M == 1 else (1024, 2048))
+    assert kept_from_288 == ({3072, 4096} if M == 1 else set())          # (shorter K: 32768 columns are less than 288 KB)
+
+
+@pytest.mark.parametrize("K,N,full,i8", [(3072, 32768, 0, 2), (4096, 28672, 0, 2), (4096, 32768, 1, 2), (3584, 28672, 1, 1),
+                                         (5120, 20480, 1, 1), (6144, 16384, 1, 2), (7168, 16384, 1, 1), (8192, 14336, 1, 2), (9216, 12288, 1, 1)])
+def test_form_and_table_of_long_ranges_at_one_token(K, N, full, i8):
+    p = tf.tf_gemv_plan(4, 1, K, N, 148)
+    assert (p["full"], p["i8"]) == (full, i8)
+
+
 @pytest.mark.parametrize("K,N,ctas", [(128, 8, 1), (128, 9472, 148), (512, 4096, 64), (896, 1024, 16), (512, 9536, 75), (1024, 1024, 16)])
 @pytest.mark.parametrize("M", [1, 8])
 def test_strips_shorter_than_a_round_are_not_put_one_after_the_other(M, K, N, ctas):
