@@ -300,6 +300,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                    int nstages, int stage_bytes, int csize, int nclusters, int xslot_bytes, int nred, int piece_tab,
                    uint8_t* __restrict__ workspace, uint32_t debug) {
     static_assert(G == 1 || (BITS == 4 && !I8 && !CL && FULL), "several groups per tile: 4-bit, floating-point path, whole SM");
+    static_assert((FULL || I8) && (!CL || MT == 2) && (I8 != 2 || BITS == 4), "forms that plan_gemv never chooses");
     constexpr int kTileBytes = tile_bytes(BITS, G);
     constexpr int kWeightBytes = BITS == 4 ? kW4WeightBytes : kW8WeightBytes;
     constexpr int kR = gemv_chunk_tiles(BITS);            // tiles per bulk copy / ring stage
@@ -921,38 +922,54 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     }
 }
 
-// How many clusters of `csize` CTAs the device can hold at once, for half-SM CTAs (two per SM) or whole-SM ones
-// (asked once per device).  0 if the question fails: cluster mode is then not used.
-static int max_resident_clusters(int csize, bool full) {
-    static std::atomic<int> cached[kGemvMaxDevices][2][4];   // [device][full][log2 csize], 0 = not asked yet, -1 = failed
+// Function attributes belong to one device: set once per device and kernel instantiation.  The flag is atomic: two
+// host threads may both find it unset and both set the attributes, which is harmless.
+template <int BITS, int MT, bool FULL, bool CL, int I8, int G = 1>
+static cudaError_t configure_one() {
+    static std::atomic<bool> configured_on[kGemvMaxDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+    const bool seen = dev >= 0 && dev < kGemvMaxDevices;
+    if (seen && configured_on[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(gemv_stream_kernel<BITS, MT, FULL, CL, I8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         FULL ? gemv_smem_budget(MT, FULL) : kGemvSoloSmemBytes);
+    if (e != cudaSuccess) return e;
+    // Always the largest shared-memory carve-out: a GEMV whose ring happens to be a little smaller would
+    // otherwise ask for a smaller split of the SM's memory, and an SM changes its split only when idle, so
+    // consecutive GEMVs of different shapes could not share an SM.
+    e = cudaFuncSetAttribute(gemv_stream_kernel<BITS, MT, FULL, CL, I8, G>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    if (seen) configured_on[dev].store(true, std::memory_order_release);
+    return cudaSuccess;
+}
+
+// How many clusters of `csize` CTAs the device can hold at once: of the kernel that is launched as clusters, at its block size
+// and at the most shared memory that it may ask for (asked once per device).  0 if the question fails: cluster mode is then
+// not used.
+template <int BITS>
+static int max_resident_clusters(int csize) {
+    static std::atomic<int> cached[kGemvMaxDevices][4];      // [device][log2 csize], 0 = not asked yet, -1 = failed
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kGemvMaxDevices) return 0;
     const int slot = csize == 2 ? 1 : csize == 4 ? 2 : 3;
-    int entry = cached[dev][full ? 1 : 0][slot].load(std::memory_order_relaxed);
+    int entry = cached[dev][slot].load(std::memory_order_relaxed);
     if (entry == 0) {                           // two host threads may both ask: same answer, harmless
         int n = 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(csize * 64, 1, 1);
-        cfg.blockDim = dim3(gemv_max_threads(1, full), 1, 1);
-        cfg.dynamicSmemBytes = gemv_smem_budget(1, full);
+        cfg.blockDim = dim3(gemv_max_threads(2, true), 1, 1);
+        cfg.dynamicSmemBytes = gemv_smem_budget(2, true);
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t e;
-        if (full) {
-            e = cudaFuncSetAttribute(gemv_stream_kernel<4, 1, true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     gemv_smem_budget(1, true));
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemv_stream_kernel<4, 1, true, true, false>, &cfg);
-        } else {
-            e = cudaFuncSetAttribute(gemv_stream_kernel<4, 1, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     gemv_smem_budget(1, false));
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemv_stream_kernel<4, 1, false, true, false>, &cfg);
-        }
+        cudaError_t e = configure_one<BITS, 2, true, true, 0>();
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemv_stream_kernel<BITS, 2, true, true, 0>, &cfg);
         if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
         entry = n > 0 ? n : -1;
-        cached[dev][full ? 1 : 0][slot].store(entry, std::memory_order_relaxed);
+        cached[dev][slot].store(entry, std::memory_order_relaxed);
     }
     return entry > 0 ? entry : 0;
 }
@@ -1063,34 +1080,31 @@ GemvPlan plan_gemv(int bits, int M, int K, int N, int sm_count, int groups) {
         }
     }
     p.cluster = 1;
-    p.nclusters = 0;
-    int best_t = 0;
-    for (int c = 2; c <= 8; c *= 2) {
-        // one CTA per SM even where two half-SM ones would fit: the other half is where the next GEMV's CTAs
-        // wait with their rings full (measured: filling both halves shortens the call and lengthens the step)
-        int maxc = max_resident_clusters(c, mt == 2);
-        if (maxc > sm_count / c) maxc = sm_count / c;
-        if (maxc < 1) continue;
-        const int j = (p.strips + maxc - 1) / maxc;                 // whole strips per cluster, at most
-        const int ncl = (p.strips + j - 1) / j;
-        const int t = (j * p.ktiles + c - 1) / c;                   // longest range of a CTA
-        if (p.cluster == 1 || t < best_t) { p.cluster = c; p.nclusters = ncl; best_t = t; }
-    }
-    // Worth it for short ranges only (there the hand-over dominates the call), only if the longest range stays
-    // within one round of the consumer warps or close to the evenly split one, and only for the whole-SM
-    // configuration of 9..16 tokens: a half-SM GEMV overlaps its start with the previous kernel's end, a cluster
-    // launch next to a plain one does not (about 2.7 us per transition, measured), and in a pass over layers of
+    p.nclusters = active;
+    // Cluster mode, for 9..16 tokens only: the half-SM form of 1 and 2 tokens overlaps its start with the previous kernel's end, a
+    // cluster launch next to a plain one does not (about 2.7 us per transition, measured), and in a pass over layers of
     // different sizes that loss is larger than what the short hand-over wins for up to 8 tokens.
-    const int one_round = gemv_max_consumers(mt, mt == 2);
-    const bool cluster_ok = mt == 2 && groups == 1;
-    if (p.cluster > 1 && cluster_ok && tiles_per_cta <= 16 && (best_t <= one_round || best_t * 10 <= tiles_per_cta * 11 + 20)) {
-        p.grid = p.nclusters * p.cluster;
-        tiles_per_cta = best_t;
-    } else {
-        p.cluster = 1;
-        p.nclusters = active;
-        if (mt == 1 && p.grid < sm_count) p.grid = sm_count;
+    if (mt == 2 && groups == 1 && tiles_per_cta <= 16) {
+        int best_c = 1, best_n = 0, best_t = 0;
+        for (int c = 2; c <= 8; c *= 2) {
+            // one CTA per SM
+            int maxc = bits == 4 ? max_resident_clusters<4>(c) : max_resident_clusters<8>(c);
+            if (maxc > sm_count / c) maxc = sm_count / c;
+            if (maxc < 1) continue;
+            const int j = (p.strips + maxc - 1) / maxc;                 // whole strips per cluster, at most
+            const int t = (j * p.ktiles + c - 1) / c;                   // longest range of a CTA
+            if (best_c == 1 || t < best_t) { best_c = c; best_n = (p.strips + j - 1) / j; best_t = t; }
+        }
+        // Worth it for short ranges only (there the hand-over dominates the call), and only if the longest range stays
+        // within one round of the consumer warps or close to the evenly split one.
+        if (best_c > 1 && (best_t <= gemv_max_consumers(mt, true) || best_t * 10 <= tiles_per_cta * 11 + 20)) {
+            p.cluster = best_c;
+            p.nclusters = best_n;
+            p.grid = best_n * best_c;
+            tiles_per_cta = best_t;
+        }
     }
+    if (mt == 1 && p.grid < sm_count) p.grid = sm_count;
     p.i8 = M <= kGemvI8MaxM && groups == 1 && p.cluster == 1;     // several groups per tile: floating-point path only
     // The floating-point path and 9..16 tokens take the whole SM: they are bound by what their consumer warps do, and only one
     // kernel's consumers work at a time.  The integer path of 1 and 2 tokens needs a fraction of the instructions; its short
@@ -1135,39 +1149,15 @@ void note_launch(cudaStream_t stream, bool whole_sm) {
 void note_whole_sm_launch(cudaStream_t stream) { note_launch(stream, true); }
 
 
-// Function attributes belong to one device: set once per device and kernel instantiation.  The flag is atomic: two
-// host threads may both find it unset and both set the attributes, which is harmless.
-template <int BITS, int MT, bool FULL, bool CL, int I8, int G = 1>
-static cudaError_t configure_one() {
-    static std::atomic<bool> configured_on[kGemvMaxDevices];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-    const bool seen = dev >= 0 && dev < kGemvMaxDevices;
-    if (seen && configured_on[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(gemv_stream_kernel<BITS, MT, FULL, CL, I8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         FULL ? gemv_smem_budget(MT, FULL) : kGemvSoloSmemBytes);
-    if (e != cudaSuccess) return e;
-    // Always the largest shared-memory carve-out: a GEMV whose ring happens to be a little smaller would
-    // otherwise ask for a smaller split of the SM's memory, and an SM changes its split only when idle, so
-    // consecutive GEMVs of different shapes could not share an SM.
-    e = cudaFuncSetAttribute(gemv_stream_kernel<BITS, MT, FULL, CL, I8, G>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    if (seen) configured_on[dev].store(true, std::memory_order_release);
-    return cudaSuccess;
-}
-
 template <int BITS>
 static cudaError_t configure_bits() {
     cudaError_t e = cudaSuccess;
     auto all = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    all(configure_one<BITS, 1, false, false, 0>()); all(configure_one<BITS, 1, true, false, 0>());
-    all(configure_one<BITS, 1, false, false, 1>());  all(configure_one<BITS, 1, true, false, 1>());
-    all(configure_one<BITS, 1, false, false, 2>());  all(configure_one<BITS, 1, true, false, 2>());
-    all(configure_one<BITS, 2, true, false, 0>());
-    all(configure_one<BITS, 1, false, true, 0>());  all(configure_one<BITS, 1, true, true, 0>());
-    all(configure_one<BITS, 2, true, true, 0>());
+    all(configure_one<BITS, 1, true, false, 0>());
+    all(configure_one<BITS, 1, false, false, 1>()); all(configure_one<BITS, 1, true, false, 1>());
+    all(configure_one<BITS, 2, true, false, 0>());  all(configure_one<BITS, 2, true, true, 0>());
     if constexpr (BITS == 4) {
+        all(configure_one<4, 1, false, false, 2>()); all(configure_one<4, 1, true, false, 2>());
         all(configure_one<4, 1, true, false, 0, 2>()); all(configure_one<4, 2, true, false, 0, 2>());
         all(configure_one<4, 1, true, false, 0, 4>()); all(configure_one<4, 2, true, false, 0, 4>());
     }
@@ -1179,7 +1169,7 @@ static cudaError_t configure_bits() {
 cudaError_t configure_gemv_kernels() {
     cudaError_t e = configure_bits<4>();
     if (e == cudaSuccess) e = configure_bits<8>();
-    for (int c = 2; c <= 8; c *= 2) { max_resident_clusters(c, false); max_resident_clusters(c, true); }
+    for (int c = 2; c <= 8; c *= 2) { max_resident_clusters<4>(c); max_resident_clusters<8>(c); }
     return e;
 }
 
@@ -1241,21 +1231,17 @@ static cudaError_t launch_bits(const GemvPlan& p, const void* blob, const void* 
                          : launch_one<4, 1, true, false, 0, 4>(p, blob, a, y, M, K, N, workspace, stream);
     }
     if (p.groups != 1) return cudaErrorInvalidValue;
-    // the cluster instructions are compiled only into the instantiations that are launched as clusters
-    if (p.cluster > 1) {
-        if (M > 8) return launch_one<BITS, 2, true, true, 0>(p, blob, a, y, M, K, N, workspace, stream);
-        return p.full ? launch_one<BITS, 1, true, true, 0>(p, blob, a, y, M, K, N, workspace, stream)
-                      : launch_one<BITS, 1, false, true, 0>(p, blob, a, y, M, K, N, workspace, stream);
+    if (M > 8)                                  // the cluster instructions are compiled only into what is launched as clusters
+        return p.cluster > 1 ? launch_one<BITS, 2, true, true, 0>(p, blob, a, y, M, K, N, workspace, stream)
+                             : launch_one<BITS, 2, true, false, 0>(p, blob, a, y, M, K, N, workspace, stream);
+    if (!p.i8) return launch_one<BITS, 1, true, false, 0>(p, blob, a, y, M, K, N, workspace, stream);
+    if constexpr (BITS == 4) {
+        if (p.piece_tab > 0)
+            return p.full ? launch_one<4, 1, true, false, 2>(p, blob, a, y, M, K, N, workspace, stream)
+                          : launch_one<4, 1, false, false, 2>(p, blob, a, y, M, K, N, workspace, stream);
     }
-    if (M > 8) return launch_one<BITS, 2, true, false, 0>(p, blob, a, y, M, K, N, workspace, stream);
-    if (p.i8 && p.piece_tab > 0)
-        return p.full ? launch_one<BITS, 1, true, false, 2>(p, blob, a, y, M, K, N, workspace, stream)
-                      : launch_one<BITS, 1, false, false, 2>(p, blob, a, y, M, K, N, workspace, stream);
-    if (p.i8)
-        return p.full ? launch_one<BITS, 1, true, false, 1>(p, blob, a, y, M, K, N, workspace, stream)
-                      : launch_one<BITS, 1, false, false, 1>(p, blob, a, y, M, K, N, workspace, stream);
-    return p.full ? launch_one<BITS, 1, true, false, 0>(p, blob, a, y, M, K, N, workspace, stream)
-                  : launch_one<BITS, 1, false, false, 0>(p, blob, a, y, M, K, N, workspace, stream);
+    return p.full ? launch_one<BITS, 1, true, false, 1>(p, blob, a, y, M, K, N, workspace, stream)
+                  : launch_one<BITS, 1, false, false, 1>(p, blob, a, y, M, K, N, workspace, stream);
 }
 
 cudaError_t launch_gemv(int bits, const GemvPlan& p, const void* blob, const void* a, void* y, int M, int K,
