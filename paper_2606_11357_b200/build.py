@@ -4,8 +4,6 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
-from concurrent.futures import ThreadPoolExecutor
-from importlib.metadata import version
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
@@ -45,9 +43,17 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _torch_version() -> str:
+    """Of the torch that is loaded, where one is (the binding asks on its first call), else of the installed one."""
+    if "torch" in sys.modules:
+        return str(sys.modules["torch"].__version__)
+    from importlib.metadata import version
+    return version("torch")
+
+
 def _native_target() -> str:
     """What the binding's CPython module is built for: it uses torch's C++ interface, which changes with every release, and Python's."""
-    return f"tilefuse native for torch {version('torch')}, {sys.implementation.cache_tag}"
+    return f"tilefuse native for torch {_torch_version()}, {sys.implementation.cache_tag}"
 
 
 def native_is_current() -> bool:
@@ -88,6 +94,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 def _compile_library(verbose: bool) -> None:
+    from concurrent.futures import ThreadPoolExecutor
     os.makedirs(OBJ, exist_ok=True)
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as pool:
         objs = list(pool.map(lambda s: _compile(s, verbose), SOURCES))

@@ -148,7 +148,7 @@ def test_native_module_of_another_torch_is_built_again_and_not_loaded(monkeypatc
     tfbuild.build()
     assert tfbuild.native_is_current() and compiled == []
     for name in ("2.11", "99.0.0"):                             # (the installed version's beginning is another version too)
-        monkeypatch.setattr(tfbuild, "version", lambda package: name)
+        monkeypatch.setattr(tfbuild, "_torch_version", lambda: name)
         assert not tfbuild.native_is_current()
         tfbuild.build()
         assert compiled == ["native"]
