@@ -11,7 +11,6 @@
 namespace {
 
 struct DeviceInfo {
-    int known;      // 1 = ok (cc 10.x), -1 = wrong architecture
     int sm_count;
 };
 // Per device: 0 = not queried yet, else (sm_count << 2) | (2 = compute capability 10.x, 1 = another architecture).
@@ -37,7 +36,6 @@ tf_status device_info(DeviceInfo* out) {
         g_devices[dev].store(word, std::memory_order_release);
     }
     if ((word & 3) != 2) return TF_ERR_ARCH;
-    out->known = 1;
     out->sm_count = word >> 2;
     return TF_OK;
 }
@@ -79,7 +77,7 @@ tf_status gemm(int bits, const void* packed, const void* a, void* y, int M, int 
     DeviceInfo dev;
     st = device_info(&dev);
     if (st != TF_OK) return st;
-    cudaError_t e = tf::launch_gemm(bits, packed, a, y, M, K, N, workspace, workspace_bytes, dev.sm_count,
+    cudaError_t e = tf::launch_gemm(bits, packed, a, y, M, K, N, workspace, dev.sm_count,
                                     static_cast<cudaStream_t>(stream), tf::groups_per_tile(group_size));
     if (e != cudaSuccess) { cudaGetLastError(); return TF_ERR_CUDA; }
     return TF_OK;

@@ -717,8 +717,7 @@ cudaError_t launch_bits(const void* blob, const void* a, void* y, int M, int K, 
 }  // namespace
 
 cudaError_t launch_gemm(int bits, const void* blob, const void* a, void* y, int M, int K, int N, void* workspace,
-                        size_t workspace_bytes, int sm_count, cudaStream_t stream, int groups) {
-    (void)workspace_bytes;
+                        int sm_count, cudaStream_t stream, int groups) {
     if (groups == 2 && bits == 4) return launch_bits<4, 2>(blob, a, y, M, K, N, workspace, sm_count, stream);
     if (groups == 4 && bits == 4) return launch_bits<4, 4>(blob, a, y, M, K, N, workspace, sm_count, stream);
     if (groups != 1) return cudaErrorInvalidValue;

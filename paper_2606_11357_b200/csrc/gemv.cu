@@ -30,7 +30,7 @@
 //
 // A range may cut a strip (64 output columns) in two.  A CTA that holds a whole strip stores y
 // directly.  Otherwise the reducer writes the fp32 partial to the workspace, and the CTA that has the strip's first tile
-// collects the partials in CTA order (see gather_partials) and stores y, so results are deterministic.  This keeps the
+// collects the partials in CTA order (see gather_partial) and stores y, so results are deterministic.  This keeps the
 // paper's rule that partial sums do not travel between workers for everything but the (at most two) cut strips of a CTA.
 #include <cuda.h>
 
@@ -146,51 +146,45 @@ __device__ __forceinline__ float4 never_plus_zero(float4 v) {
     return make_float4(__uint_as_float(x == 0u ? 0x80000000u : x), __uint_as_float(y == 0u ? 0x80000000u : y),
                        __uint_as_float(z == 0u ? 0x80000000u : z), __uint_as_float(w == 0u ? 0x80000000u : w));
 }
-// `slot` already points at this lane's first float4 of the partial of the first of `count` (<= kBatch) consecutive
-// CTAs; rows of tokens >= M are neither written nor read.  The loads of all `count` partials are issued together (one
-// trip to the L2 per turn), then the partials are added to `acc` in CTA order and their slots cleared.  Returns false
-// if the wait ran out.  Kept out of line so that the polling loop does not take part in the register allocation of the
+// `slot` already points at this lane's first float4 of the partial; rows of tokens >= M are neither written nor read.  The
+// partial is added to `acc` and its slot cleared.  Returns false if the wait ran out.  One partial per trip to the L2: with
+// four at once the finisher of a strip shared by four CTAs would wait one trip instead of three, but the gathering code
+// then needs 64 registers more and the whole step was slower (125.7 against 122.6 us; 2 MB shapes gained 0.3 us, 9 MB shapes
+// lost 1 us).  Kept out of line so that the polling loop does not take part in the register allocation of the
 // streaming kernel around it.
-template <int kVec, int kBatch>
-__device__ __noinline__ bool gather_partials(float4* slot, int count, int M, float4 (&acc)[kVec], volatile uint32_t* abort_flag, uint32_t site) {
-    constexpr int kSlotVec = kGemvSlotBytes / 16;
-    float4 v[kBatch][kVec];
+template <int kVec>
+__device__ __noinline__ bool gather_partial(float4* slot, int M, float4 (&acc)[kVec], volatile uint32_t* abort_flag, uint32_t site) {
+    float4 v[kVec];
     const long long t_begin = clock64();
     for (;;) {
         bool here = true;
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b)
+        for (int e = 0; e < kVec; ++e) {
+            v[e] = make_float4(-0.f, -0.f, -0.f, -0.f);
+            if (2 * e < M)                       // a real load on every turn of the loop, from the L2
+                asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(v[e].x), "=f"(v[e].y), "=f"(v[e].z), "=f"(v[e].w) : "l"(slot + 32 * e) : "memory");
+        }
 #pragma unroll
-            for (int e = 0; e < kVec; ++e) {
-                v[b][e] = make_float4(-0.f, -0.f, -0.f, -0.f);
-                if (b < count && 2 * e < M)                       // a real load on every turn of the loop, from the L2
-                    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                 : "=f"(v[b][e].x), "=f"(v[b][e].y), "=f"(v[b][e].z), "=f"(v[b][e].w)
-                                 : "l"(slot + b * kSlotVec + 32 * e) : "memory");
-            }
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b)
-#pragma unroll
-            for (int e = 0; e < kVec; ++e)
-                here = here && __float_as_uint(v[b][e].x) != 0u && __float_as_uint(v[b][e].y) != 0u &&
-                       __float_as_uint(v[b][e].z) != 0u && __float_as_uint(v[b][e].w) != 0u;
+        for (int e = 0; e < kVec; ++e)
+            here = here && __float_as_uint(v[e].x) != 0u && __float_as_uint(v[e].y) != 0u && __float_as_uint(v[e].z) != 0u &&
+                   __float_as_uint(v[e].w) != 0u;
         if (__all_sync(0xFFFFFFFFu, here)) break;
         if (*abort_flag != 0) return false;
         if (wait_expired(t_begin, abort_flag)) { *abort_flag = site; return false; }
     }
 #pragma unroll
-    for (int b = 0; b < kBatch; ++b)
-#pragma unroll
-        for (int e = 0; e < kVec; ++e) {
-            acc[e].x += v[b][e].x; acc[e].y += v[b][e].y; acc[e].z += v[b][e].z; acc[e].w += v[b][e].w;
-            if (b < count && 2 * e < M) __stcg(slot + b * kSlotVec + 32 * e, make_float4(0.f, 0.f, 0.f, 0.f));
-        }
+    for (int e = 0; e < kVec; ++e) {
+        acc[e].x += v[e].x; acc[e].y += v[e].y; acc[e].z += v[e].z; acc[e].w += v[e].w;
+        if (2 * e < M) __stcg(slot + 32 * e, make_float4(0.f, 0.f, 0.f, 0.f));
+    }
     return true;
 }
 
 // The same hand-over taken row pair by row pair: for float4 index e (token rows 2e, 2e + 1) the words of up to four
 // consecutive CTAs' partials are requested together, so a strip shared by many CTAs and few tokens costs one trip per
-// row pair instead of one per contributor, in 16 registers.  `slot` as above; adds to acc[e] in CTA order.
+// row pair instead of one per contributor, in 16 registers.  `slot` points at this lane's first float4 of the first of `count`
+// (<= 4) partials; adds to acc[e] in CTA order.
 template <int kVec>
 __device__ __noinline__ bool gather_rows(float4* slot, int count, int M, float4 (&acc)[kVec], volatile uint32_t* abort_flag, uint32_t site) {
     constexpr int kSlotVec = kGemvSlotBytes / 16;
@@ -444,24 +438,20 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 const bool finisher = (!CL || csize == 1) && !whole && c_first == crank;
 
                 // While the consumers still work on this segment, collect what the other contributors have dropped
-                // (in CTA order; a partial has arrived when none of its words is +0.0, see gather_partials).
+                // (in CTA order; a partial has arrived when none of its words is +0.0, see gather_partial).
                 float4 others[kVec];
 #pragma unroll
                 for (int e = 0; e < kVec; ++e) others[e] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (finisher) {
-                    // one partial per trip: with four at once the finisher of a strip shared by four CTAs would wait one
-                    // trip instead of three, but the gathering code then needs 64 registers more and the whole step was
-                    // slower (measured: 125.7 against 122.6 us), 2 MB shapes gained 0.3 us, 9 MB shapes lost 1 us
-                    constexpr int kBatch = 1;
                     const int nothers = c_last - c_first;
                     if (nothers > 1 && nothers <= 4 && (M + 1) / 2 < nothers) {
                         // more contributors than pairs of token rows: row pair by row pair, all contributors at once
                         float4* slot = reinterpret_cast<float4*>(partials + (size_t)(c_first + 1) * (kGemvMaxM * kTileN)) + lane;
                         ok = gather_rows<kVec>(slot, nothers, M, others, abort_flag, 0x450);
                     } else {
-                        for (int c = c_first + 1; c <= c_last && ok; c += kBatch) {
+                        for (int c = c_first + 1; c <= c_last && ok; ++c) {
                             float4* slot = reinterpret_cast<float4*>(partials + (size_t)c * (kGemvMaxM * kTileN)) + lane;
-                            ok = gather_partials<kVec, kBatch>(slot, min(kBatch, c_last - c + 1), M, others, abort_flag, 0x440);
+                            ok = gather_partial<kVec>(slot, M, others, abort_flag, 0x440);
                         }
                     }
                     if (!ok) break;

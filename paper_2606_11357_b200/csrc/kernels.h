@@ -65,8 +65,7 @@ constexpr int kGemvFpW4MaxStages = 5;
 constexpr int kGemvFpTwelveWarpsFromTiles = 32;
 constexpr int kGemvMaxDevices = 64;            // devices the per-device caches cover
 constexpr int kGemvMaxStages = 48;
-constexpr int kGemvBarrierBytes = 4096;       // 2 x 48 mbarriers + flags, then contributor offsets
-constexpr int kGemvMaxContrib = 320;          // CTAs that can share one strip (<= K/128 + 1 = 257)
+constexpr int kGemvBarrierBytes = 4096;       // 2 x 48 mbarriers + flags, then the chunk tags of the stages
 // A ring stage holds one bulk copy of several contiguous tiles (about 16.6 KB either way) and, on the floating-point path, their
 // activations.  (4-bit tiles, floating-point path: with two tiles per copy the one lane that issues the copies sets the pace, 4
 // tokens 4096x28672 19.0 us against 15.7 with four; with five, six or eight a stage is freed late: 16.0, 15.9, 16.5.)
@@ -82,7 +81,7 @@ constexpr int kGemvMaxGrid = 256;             // CTAs (one per SM); sizes the pa
 //   (16 tokens x 64 columns fp32) per persistent CTA | behind them the GEMM's partial tiles (written before they are
 //   read, so the GEMM may leave anything there).
 // Everything below kWorkspaceZeroBytes is zero between calls: the GEMV's hand-over of a cut strip relies on its slots
-// being all +0.0 bits (see gather_partials in gemv.cu), the GEMM on its flags.
+// being all +0.0 bits (see gather_partial in gemv.cu), the GEMM on its flags.
 constexpr int kWorkspaceHeadBytes = 20480;
 constexpr int kGemvStatusBytes = 256;         // what the GEMV itself needs cleared besides its slots
 constexpr int kGemvPartialOffset = kWorkspaceHeadBytes;
@@ -151,6 +150,6 @@ cudaError_t launch_repack_awq(const uint32_t* qweight, const uint16_t* scales, c
 // Prefill GEMM (tcgen05).  `workspace` starts with the DeviceStatus word.
 size_t gemm_workspace_bytes(int M, int K, int N);
 cudaError_t launch_gemm(int bits, const void* blob, const void* a, void* y, int M, int K, int N,
-                        void* workspace, size_t workspace_bytes, int sm_count, cudaStream_t stream, int groups = 1);
+                        void* workspace, int sm_count, cudaStream_t stream, int groups = 1);
 
 }  // namespace tf

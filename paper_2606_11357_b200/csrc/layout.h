@@ -37,7 +37,6 @@ constexpr int kW4WeightBytes = 4096;
 constexpr int kW8WeightBytes = 8192;
 constexpr int kScaleBytes = 128;
 constexpr int kZeroBytes = 32;
-constexpr int kW4TileBytes = kW4WeightBytes + kScaleBytes + kZeroBytes;   // 4256
 constexpr int kW8TileBytes = kW8WeightBytes + kScaleBytes;                // 8320
 
 // Groups per tile for a legal group size (a multiple of 128 that divides K: one; 64: two; 32: four).
