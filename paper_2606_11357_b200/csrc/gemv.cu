@@ -281,6 +281,13 @@ __device__ __noinline__ void make_pieces_call(const uint2 (&raws)[2], uint32_t* 
     make_pieces<BITS>(raws, dst, meta, M, lane);
 }
 
+// Floating-point path: token g + 8 mt, k = 16 kb + 4t .. +3 of a tile's activations in the ring.  The 16-byte units of a row are
+// permuted by the swizzle: two wavefronts for 256 bytes.
+template <int MT>
+__device__ __forceinline__ uint2 act_fragment(const uint8_t* acts, int g, int t, int kb, int mt) {
+    return *reinterpret_cast<const uint2*>(acts + (kb >> 2) * (1024 * MT) + (g + 8 * mt) * 128 + (((2 * (kb & 3) + (t >> 1)) ^ g) << 4) + (t & 1) * 8);
+}
+
 // G = groups per tile: 1 for group sizes that are multiples of 128, 2 / 4 for the 4-bit group sizes 64 / 32.
 // I8 = 0: floating-point path; 1: integer path, a consumer warp prepares the activation pieces of every tile it works
 // on; 2: integer path for ranges that pass over the same k-tiles more than once, with K a multiple of 128 times the
@@ -534,12 +541,6 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 if (m < M) araw[m] = __ldcg(reinterpret_cast<const uint2*>(base + (size_t)m * K + 4 * lane));
             }
         };
-        // Floating-point path: token g + 8 mt, k = 16 kb + 4t .. +3 of a tile's activations in the ring.  The 16-byte units of a row
-        // are permuted by the swizzle: two wavefronts for 256 bytes.  (As a lambda: without one that captures g and t here the
-        // compiler schedules the integer path differently, 1x4096x1024 4.6 against 3.7 us, 1x4096x28672 16.1 against 13.4.)
-        auto act_fragment = [&](const uint8_t* acts, int kb, int mt) {
-            return *reinterpret_cast<const uint2*>(acts + (kb >> 2) * (1024 * MT) + (g + 8 * mt) * 128 + (((2 * (kb & 3) + (t >> 1)) ^ g) << 4) + (t & 1) * 8);
-        };
         constexpr int kColWords = kGemvPieceColWords;
         // Piece table (I8 == 2): local tile j of the range finds its pieces in entry j mod piece_n, piece_n =
         // min(ntiles, ktiles); j < piece_n is the first visit of that k-tile.  ktiles is a multiple of the number of
@@ -759,7 +760,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                     for (int kb = gr * (8 / G); kb < (gr + 1) * (8 / G); ++kb) {
                         uint2 av[MT];
 #pragma unroll
-                        for (int mt = 0; mt < MT; ++mt) av[mt] = act_fragment(acts, kb, mt);
+                        for (int mt = 0; mt < MT; ++mt) av[mt] = act_fragment<MT>(acts, g, t, kb, mt);
                         uint4 wv[kVecPerKb];
 #pragma unroll
                         for (int h = 0; h < kVecPerKb; ++h)
@@ -822,21 +823,19 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
             if (!mbar_wait(seg_free0 + 8 * rb, (ru & 1) ^ 1, abort_flag, 0x300)) { aborted = true; break; }
             float* mine = red + (size_t)(rb * nconsumers + cw) * kRedWarp;      // [token][n]
             if constexpr (I8) {
-                // columns 3m .. 3m+2 are the pieces of token m, already on a common scale: add them up across the four
-                // threads of a row (fixed order) and leave tokens 0, 1 where the bf16 path has them (t = 0)
+                // columns 3m .. 3m+2 are the pieces of token m, already on a common scale: token 0 is columns 0 and 1 of thread
+                // t = 0 and column 2 of t = 1, token 1 column 3 of t = 1 and columns 4 and 5 of t = 2.  Both end where the
+                // floating-point path has them (t = 0); what the other threads add up is not used.  (No choice by t: written as
+                // nested conditions the compiler made divergent branches of them or not, depending on unrelated code around, and
+                // the branches cost 1.1 us per segment: 1x4096x1024 4.7 against 3.6 us, x28672 16.6 against 13.8; this form
+                // 3.60 and 13.52.)
 #pragma unroll
                 for (int w = 0; w < 4; ++w)
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
-                        const float c0 = acc[w][0][2 * r], c1 = acc[w][0][2 * r + 1];
-                        float tok0 = t == 0 ? c0 + c1 : t == 1 ? c0 : 0.f;
-                        float tok1 = t == 1 ? c1 : t == 2 ? c0 + c1 : 0.f;
-                        tok0 += __shfl_xor_sync(0xFFFFFFFFu, tok0, 1);
-                        tok1 += __shfl_xor_sync(0xFFFFFFFFu, tok1, 1);
-                        tok0 += __shfl_xor_sync(0xFFFFFFFFu, tok0, 2);
-                        tok1 += __shfl_xor_sync(0xFFFFFFFFu, tok1, 2);
-                        acc[w][0][2 * r] = t == 0 ? tok0 : 0.f;
-                        acc[w][0][2 * r + 1] = t == 0 ? tok1 : 0.f;
+                        const float c0 = acc[w][0][2 * r], c1 = acc[w][0][2 * r + 1], both = c0 + c1;
+                        acc[w][0][2 * r] = both + __shfl_down_sync(0xFFFFFFFFu, c0, 1);
+                        acc[w][0][2 * r + 1] = __shfl_down_sync(0xFFFFFFFFu, c1, 1) + __shfl_down_sync(0xFFFFFFFFu, both, 2);
                     }
             }
 #pragma unroll
