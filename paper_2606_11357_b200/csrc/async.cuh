@@ -47,9 +47,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return done != 0;
 }
 
-// Bounded wait.  Gives up after about a second of polling, or as soon as another thread of the CTA
-// has given up (`abort_flag[0]` != 0).  On giving up it records `site` in the flag and returns false;
-// the caller must then leave its role loop and go to the common teardown.
+// Bounded waits.  A wait gives up after about a second of polling, or as soon as another thread of the CTA has given up
+// (`abort_flag[0]` != 0).  On giving up it records `site` in the flag and returns false; the caller must then leave its role loop
+// and go to the common teardown.
+// Of the threads of a warp that poll for themselves one may see the data arrive and the next the limit run out; the first would go
+// on to a shuffle, a vote or an MMA of the whole warp and wait there, without a limit, for threads that have left.  So a
+// role of one thread waits with mbar_wait, a role of a whole warp with mbar_wait_warp (or a loop of its own around
+// wait_given_up), which decides by a vote.
 // `abort_flag` points at two words of shared memory: [0] the flag, [1] the limit of a wait in units of 1024
 // cycles, written once by the CTA's first thread from the kernel's `debug` argument (see wait_limit_kcycles).
 constexpr long long kWaitLimitCycles = 2000000000ll;
@@ -62,6 +66,12 @@ __device__ __forceinline__ uint32_t wait_limit_kcycles(uint32_t debug) {
 }
 __device__ __forceinline__ bool wait_expired(long long t_begin, volatile uint32_t* abort_flag) {
     return clock64() - t_begin > ((long long)abort_flag[1] << 10);
+}
+// One turn of a converged warp's wait that has not been met yet: whether the warp, all of it, gives up.
+__device__ __forceinline__ bool wait_given_up(long long t_begin, volatile uint32_t* abort_flag, uint32_t site) {
+    const bool expired = wait_expired(t_begin, abort_flag);
+    if (expired && *abort_flag == 0) *abort_flag = site;
+    return __any_sync(0xFFFFFFFFu, expired || *abort_flag != 0);
 }
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                           uint32_t site) {
@@ -79,18 +89,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
-// The same by a whole converged warp, which leaves it by a vote: the compiler then knows that what the loop around it
-// carries is uniform in the warp and keeps it in uniform registers, where tcgen05.mma wants its operands.
+// The same by a whole converged warp, which leaves it by a vote.  (The compiler then also knows that what the loop around it
+// carries is uniform in the warp and keeps it in uniform registers, where tcgen05.mma wants its operands.)
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
     if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
     const long long t0 = clock64();
     for (uint32_t it = 1;; ++it) {
         if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
-        if ((it & 0xFFu) == 0) {
-            const bool expired = wait_expired(t0, abort_flag);
-            if (expired && *abort_flag == 0) *abort_flag = site;
-            if (__any_sync(0xFFFFFFFFu, expired || *abort_flag != 0)) return false;
-        }
+        if ((it & 0xFFu) == 0 && wait_given_up(t0, abort_flag, site)) return false;
     }
 }
 

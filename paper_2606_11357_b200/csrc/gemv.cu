@@ -170,8 +170,7 @@ __device__ __noinline__ bool gather_partial(float4* slot, int M, float4 (&acc)[k
             here = here && __float_as_uint(v[e].x) != 0u && __float_as_uint(v[e].y) != 0u && __float_as_uint(v[e].z) != 0u &&
                    __float_as_uint(v[e].w) != 0u;
         if (__all_sync(0xFFFFFFFFu, here)) break;
-        if (*abort_flag != 0) return false;
-        if (wait_expired(t_begin, abort_flag)) { *abort_flag = site; return false; }
+        if (wait_given_up(t_begin, abort_flag, site)) return false;
     }
 #pragma unroll
     for (int e = 0; e < kVec; ++e) {
@@ -205,8 +204,7 @@ __device__ __noinline__ bool gather_rows(float4* slot, int count, int M, float4 
                 here = here && __float_as_uint(v[b].x) != 0u && __float_as_uint(v[b].y) != 0u && __float_as_uint(v[b].z) != 0u &&
                        __float_as_uint(v[b].w) != 0u;
             if (__all_sync(0xFFFFFFFFu, here)) break;
-            if (*abort_flag != 0) return false;
-            if (wait_expired(t_begin, abort_flag)) { *abort_flag = site; return false; }
+            if (wait_given_up(t_begin, abort_flag, site)) return false;
         }
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -330,7 +328,8 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     constexpr uint32_t kActStageBytes = I8 == 0 ? kR * gemv_act_tile_bytes(MT) : 0;
     uint8_t* ring = abuf + nstages * kActStageBytes;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle tells the compiler that the warp number is uniform in the warp)
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int cta = blockIdx.x;
     // "Contributor space": the CTAs that split one pool of tiles evenly among themselves.  Global mode: all CTAs
     // of the grid over all tiles.  Cluster mode: the CTAs of one cluster over the whole strips that cluster owns,
@@ -466,7 +465,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
 
                 // segment sidx goes through buffer sidx % nred, in that buffer's use number sidx / nred
                 const int rb = nred == 2 ? (sidx & 1) : 0, ru = nred == 2 ? (sidx >> 1) : sidx;
-                ok = mbar_wait(seg_full0 + 8 * rb, ru & 1, abort_flag, 0x400);
+                ok = mbar_wait_warp(seg_full0 + 8 * rb, ru & 1, abort_flag, 0x400);
                 if (!ok) break;
                 // sum = partial of warp 0 + warp 1 + ... (fixed order); rows of tokens >= M hold zeros
                 float4 sum[kVec];
@@ -584,14 +583,12 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 cg_cur = cg;
                 while (s_cur >= nstages) { s_cur -= nstages; ++use_cur; }
                 const int s = s_cur;
-                if (stage_tag[s] != (uint32_t)cg) {            // the producer has not reached this chunk yet
+                if (!__all_sync(0xFFFFFFFFu, stage_tag[s] == (uint32_t)cg)) {      // the producer has not reached this chunk yet
                     const long long t_begin = clock64();
-                    while (stage_tag[s] != (uint32_t)cg) {
-                        if (*abort_flag != 0) return false;
-                        if (wait_expired(t_begin, abort_flag)) { *abort_flag = 0x280 + s; return false; }
-                    }
+                    while (!__all_sync(0xFFFFFFFFu, stage_tag[s] == (uint32_t)cg))
+                        if (wait_given_up(t_begin, abort_flag, 0x280 + s)) return false;
                 }
-                if (!mbar_wait(full0 + 8 * s, use_cur & 1, abort_flag, 0x200 + s)) return false;
+                if (!mbar_wait_warp(full0 + 8 * s, use_cur & 1, abort_flag, 0x200 + s)) return false;
                 nx_tile = ring + (size_t)s * stage_bytes + (size_t)slot * kTileBytes;
                 nx_s = s; nx_slot = slot; nx_cl = cl;
                 if constexpr (!I8) {
@@ -820,7 +817,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
             // With two buffers a warp that is a segment ahead of the slowest warp does not wait for it: a segment's
             // partials go to buffer sidx % nred, which the reducer must have read nred segments ago.
             const int rb = nred == 2 ? (sidx & 1) : 0, ru = nred == 2 ? (sidx >> 1) : sidx;
-            if (!mbar_wait(seg_free0 + 8 * rb, (ru & 1) ^ 1, abort_flag, 0x300)) { aborted = true; break; }
+            if (!mbar_wait_warp(seg_free0 + 8 * rb, (ru & 1) ^ 1, abort_flag, 0x300)) { aborted = true; break; }
             float* mine = red + (size_t)(rb * nconsumers + cw) * kRedWarp;      // [token][n]
             if constexpr (I8) {
                 // columns 3m .. 3m+2 are the pieces of token m, already on a common scale: token 0 is columns 0 and 1 of thread

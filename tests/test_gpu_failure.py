@@ -57,6 +57,31 @@ def test_bounded_wait_runs_out_and_the_library_recovers(kind, bits, M, K, N):
     gu.check_against_oracle(p, gu.bits_of(y))
 
 
+# (the last two: a strip shared by four CTAs, hand-over through the workspace)
+@pytest.mark.parametrize("kind,bits,M,K,N", [c for c in CASES if c[0] == "gemv"] + [("gemv", 4, 1, 4096, 1024), ("gemv", 4, 6, 4096, 1024)])
+def test_waits_that_run_out_while_the_data_arrives(kind, bits, M, K, N):
+    """Limits of half a microsecond and up with the producers at work: waits run out at the moment in which what they wait for
+    comes in.  A warp must leave such a wait as a whole, whichever of its threads saw what; the call returns, with or
+    without TF_ERR_TIMEOUT, and the next one is right."""
+    p = wl.make_w4(M, K, N, seed=3200 + M) if bits == 4 else wl.make_w8(M, K, N, seed=3200 + M)
+    blob = torch.from_numpy(gu.pack(p)).cuda()
+    a = gu.to_device_bf16(p.a_bf16)
+    y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    op = (0 if kind == "gemv" else 2) + (1 if bits == 8 else 0)
+    ws = torch.zeros(tf.tf_workspace_size(op, M, K, N), dtype=torch.uint8, device="cuda")
+    fn = getattr(tf, f"tf_{kind}_w{bits}a16")
+    for limit in (1, 2, 3, 4, 6, 8, 16, 64):
+        tf.tf_debug_inject(limit, False)
+        for _ in range(4):
+            fn(blob, a, y, M, K, N, ws)
+            assert tf.tf_device_status(ws) in (0, TF_ERR_TIMEOUT)
+            ws.zero_()
+    tf.tf_debug_inject(0, False)
+    fn(blob, a, y, M, K, N, ws)
+    assert tf.tf_device_status(ws) == 0
+    gu.check_against_oracle(p, gu.bits_of(y))
+
+
 def test_short_limit_alone_changes_nothing():
     """With the producer at work a millisecond is ample: the shortened limit by itself must not trip any wait."""
     p = wl.make_w4(4, 4096, 4096, seed=3100)
