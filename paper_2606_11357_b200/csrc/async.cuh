@@ -90,14 +90,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 
 // The same by a whole converged warp, which leaves it by a vote.  (The compiler then also knows that what the loop around it
-// carries is uniform in the warp and keeps it in uniform registers, where tcgen05.mma wants its operands.)
+// carries is uniform in the warp and keeps it in uniform registers, where tcgen05.mma wants its operands.
+// The limit is looked at on every turn: looked at on every 256th, with a counter, the GEMM's dequant warps spilled, 2048x4096x14336
+// 187.9 us against 185.9.)
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
     if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
     const long long t0 = clock64();
-    for (uint32_t it = 1;; ++it) {
-        if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
-        if ((it & 0xFFu) == 0 && wait_given_up(t0, abort_flag, site)) return false;
-    }
+    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)))
+        if (wait_given_up(t0, abort_flag, site)) return false;
+    return true;
 }
 
 // ---- programmatic dependent launch -------------------------------------------------------------------

@@ -460,7 +460,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
             share.tbuf = drain_buf + (warp - kFirstDequant) * kDrainWarpBytes;
             auto do_duty = [&](int sidx) -> bool {
                 const int acc = sidx % kAccs;
-                if (!mbar_wait(smem_u32(&bars->acc_full[acc]), sidx / kAccs & 1, abort_flag, 0x520)) return false;
+                if (!mbar_wait_warp(smem_u32(&bars->acc_full[acc]), sidx / kAccs & 1, abort_flag, 0x520)) return false;
                 tc_fence_after();
                 int dtile, dkt0, dlen;
                 segs.get(sidx, dtile, dkt0, dlen);
@@ -482,9 +482,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                             uint32_t f = 1;
                             if (mine) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(f) : "l"(flag) : "memory");
                             if (__all_sync(0xFFFFFFFFu, f != 0)) break;
-                            const bool expired = wait_expired(t_begin, abort_flag);
-                            if (expired && *abort_flag == 0) *abort_flag = 0x610;
-                            if (__any_sync(0xFFFFFFFFu, expired || *abort_flag != 0)) return false;
+                            if (wait_given_up(t_begin, abort_flag, 0x610)) return false;
                         }
                         if (mine) *flag = 0;                            // zero for the next call
                     }
@@ -510,7 +508,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                         ws += kGroups / kChunk;
                         if (ws >= wp_stages) { ws -= wp_stages; wparity ^= 1u; }
                     };
-                    ok = mbar_wait(smem_u32(&bars->wp_full[ws]), wparity, abort_flag, 0x500 + ws);
+                    ok = mbar_wait_warp(smem_u32(&bars->wp_full[ws]), wparity, abort_flag, 0x500 + ws);
                     if (!ok) break;
                     if (T + group % kChunk >= len) {          // a chunk of one k-tile, and it is the other group's
                         release_stage();
@@ -578,7 +576,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                         if (step == 3) release_stage();       // the packed stage has been read
                         if (step == 0) {
                             // the MMAs that read this operand stage last have run
-                            ok = mbar_wait(smem_u32(&bars->op_done[group]), done_parity, abort_flag, 0x510 + group);
+                            ok = mbar_wait_warp(smem_u32(&bars->op_done[group]), done_parity, abort_flag, 0x510 + group);
                             if (!ok) break;
                             done_parity ^= 1u;
                             tc_fence_after();

@@ -57,8 +57,9 @@ def test_bounded_wait_runs_out_and_the_library_recovers(kind, bits, M, K, N):
     gu.check_against_oracle(p, gu.bits_of(y))
 
 
-# (the last two: a strip shared by four CTAs, hand-over through the workspace)
-@pytest.mark.parametrize("kind,bits,M,K,N", [c for c in CASES if c[0] == "gemv"] + [("gemv", 4, 1, 4096, 1024), ("gemv", 4, 6, 4096, 1024)])
+# (the last four: a strip shared by four CTAs, hand-over through the workspace, and GEMM tiles cut between CTAs)
+@pytest.mark.parametrize("kind,bits,M,K,N", CASES + [("gemv", 4, 1, 4096, 1024), ("gemv", 4, 6, 4096, 1024), ("gemm", 4, 77, 4096, 1016),
+                                                   ("gemm", 8, 260, 1024, 1096)])
 def test_waits_that_run_out_while_the_data_arrives(kind, bits, M, K, N):
     """Limits of half a microsecond and up with the producers at work: waits run out at the moment in which what they wait for
     comes in.  A warp must leave such a wait as a whole, whichever of its threads saw what; the call returns, with or
