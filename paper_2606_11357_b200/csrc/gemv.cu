@@ -74,21 +74,14 @@ __device__ __forceinline__ void mma_u8s8_16832_first(int d[4], uint32_t a0, uint
 constexpr int kIntAsFloatBias = 0x4B400000;
 constexpr float kIntAsFloatBiasValue = 12582912.0f;
 
-// Even split of `total` tiles over `grid` CTAs.  The products fit 32 bits (at most 256 x 512 tiles, K and N <= 32768,
-// times at most 257 CTAs), and a 32-bit division is a fraction of the instructions of a 64-bit one.  These sit between
-// the start of a CTA and its first weight copy, in the reducer's bookkeeping and in the cluster-mode finish; k32 chooses
-// the width per kernel instantiation and function, by measurement (the compiler schedules the kernels differently).  Both in 32
-// bits for 9..16 tokens; up to 8 tokens only the start (4 tokens 4096x6144 7.22 -> 7.14 us, 14336x4096 10.58 -> 10.43; the owner
-// too: 7.04 and 10.36, but 4096x2048 5.01 -> 5.21); integer path only the owner (4096x6144 6.09 -> 5.90, 4096x28672 13.35 -> 13.16).
-template <bool k32>
+// Even split of `total` tiles over `grid` CTAs.  32-bit: the products stay below 2^26 (at most 256 x 512 tiles, K and N <= 32768,
+// times at most 257), and a 64-bit division is several times the instructions.  These sit between the start of a CTA and its
+// first weight copy, in the reducer's bookkeeping and in the cluster-mode finish.
 __device__ __forceinline__ int range_start(int cta, int total, int grid) {
-    if constexpr (k32) return static_cast<int>((static_cast<uint32_t>(cta) * static_cast<uint32_t>(total)) / static_cast<uint32_t>(grid));
-    else return static_cast<int>((static_cast<long long>(cta) * total) / grid);
+    return static_cast<int>((static_cast<uint32_t>(cta) * static_cast<uint32_t>(total)) / static_cast<uint32_t>(grid));
 }
-template <bool k32>
 __device__ __forceinline__ int range_owner(int tile, int total, int grid) {
-    if constexpr (k32) return static_cast<int>(((static_cast<uint32_t>(tile) + 1u) * static_cast<uint32_t>(grid) - 1u) / static_cast<uint32_t>(total));
-    else return static_cast<int>(((static_cast<long long>(tile) + 1) * grid - 1) / total);
+    return static_cast<int>(((static_cast<uint32_t>(tile) + 1u) * static_cast<uint32_t>(grid) - 1u) / static_cast<uint32_t>(total));
 }
 
 // The chunks of a tile range [t0, t0 + ntiles): up to kR consecutive tiles of one strip each.  Tiles are stored
@@ -339,12 +332,12 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     int cn = nclusters, crank = cta, cbase = 0, ctiles = total_tiles;
     if (CL && csize > 1) {
         const int q = cta / csize, strips = total_tiles / ktiles;
-        const int s0 = range_start<I8 == 0>(q, strips, nclusters), s1 = range_start<I8 == 0>(q + 1, strips, nclusters);
+        const int s0 = range_start(q, strips, nclusters), s1 = range_start(q + 1, strips, nclusters);
         cn = csize; crank = cta - q * csize; cbase = s0 * ktiles; ctiles = (s1 - s0) * ktiles;
     }
     const bool idle = crank >= cn;
-    const int t0 = idle ? 0 : cbase + range_start<I8 == 0>(crank, ctiles, cn);
-    const int ntiles = idle ? 0 : cbase + range_start<I8 == 0>(crank + 1, ctiles, cn) - t0;
+    const int t0 = idle ? 0 : cbase + range_start(crank, ctiles, cn);
+    const int ntiles = idle ? 0 : cbase + range_start(crank + 1, ctiles, cn) - t0;
     int fin_strip = -1, fin_first = 0;          // cluster mode: the strip this CTA finishes after the cluster barrier
 
     DeviceStatus* status = reinterpret_cast<DeviceStatus*>(workspace);
@@ -437,8 +430,8 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 const int strip = tile0 / ktiles, T0 = tile0 - strip * ktiles;
                 const int seg_len = min(ntiles - i, ktiles - T0);
                 const bool whole = seg_len == ktiles;
-                const int c_first = range_owner<I8 != 0 || MT == 2>(strip * ktiles - cbase, ctiles, cn);
-                const int c_last = range_owner<I8 != 0 || MT == 2>(strip * ktiles + ktiles - 1 - cbase, ctiles, cn);
+                const int c_first = range_owner(strip * ktiles - cbase, ctiles, cn);
+                const int c_last = range_owner(strip * ktiles + ktiles - 1 - cbase, ctiles, cn);
                 // Global mode, cut strip: the CTA that holds the strip's first tile finishes it.  Its part of the strip
                 // is the tail of its range; for every other contributor the strip is the head of the range, done early.
                 const bool finisher = (!CL || csize == 1) && !whole && c_first == crank;
@@ -870,7 +863,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
             const bool some_empty = ctiles < cn;
 #pragma unroll 2
             for (int c = fin_first; c <= crank; ++c) {                     // rank order, as in global mode
-                if (some_empty && range_start<I8 == 0>(c + 1, ctiles, cn) == range_start<I8 == 0>(c, ctiles, cn)) continue;   // empty range: no partial
+                if (some_empty && range_start(c + 1, ctiles, cn) == range_start(c, ctiles, cn)) continue;   // empty range: no partial
                 const float4* src = reinterpret_cast<const float4*>(xred + (size_t)c * xslot_bytes) + lane;
 #pragma unroll
                 for (int e = 0; e < kVec; ++e)
