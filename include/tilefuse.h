@@ -246,7 +246,7 @@ tf_status tf_gemv_w8a16(const void* packed, const void* a_bf16, void* y_bf16,
  * Work is split evenly over the persistent CTAs in units of (output tile, 128-deep k-tile): an
  * output tile whose K range is cut between CTAs is summed in fp32 through the workspace, in CTA
  * order, by the CTA that has the tile's last k-tile, so results do not depend on timing.
- * Workspace: tf_workspace_size() bytes (tens of MB: fp32 tile slots per CTA).  Its first
+ * Workspace: tf_workspace_size() bytes (3.7 to 22 MB: one fp32 tile slot per CTA).  Its first
  * TF_WORKSPACE_ZERO_BYTES bytes (status word, flags, the GEMV's slots) must be zero before the first
  * call that uses it; every call leaves them zero again unless it reports an error there.  One
  * workspace per stream (it may be the one the GEMV calls of that stream use): calls that run

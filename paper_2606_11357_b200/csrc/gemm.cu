@@ -625,7 +625,7 @@ static int gemm_token_tile(int M) { return M > 128 ? 256 : M > 64 ? 128 : M > 32
 
 size_t gemm_workspace_bytes(int M, int K, int N) {
     (void)K; (void)N;
-    return (size_t)kGemmPartialOffset + (size_t)kGemmMaxGrid * 2 * kBN * gemm_token_tile(M) * 4;   // (half of it is used)
+    return (size_t)kGemmPartialOffset + (size_t)kGemmMaxGrid * kBN * gemm_token_tile(M) * 4;      // one slot per CTA
 }
 
 namespace {

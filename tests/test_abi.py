@@ -92,6 +92,13 @@ def test_compute_calls_validate_before_touching_the_gpu():
         assert len(L.tf_status_string(code)) > 0
 
 
+@pytest.mark.parametrize("M,tokens", [(1, 32), (32, 32), (33, 64), (64, 64), (65, 128), (128, 128), (129, 256), (4096, 256)])
+def test_gemm_workspace_is_one_slot_of_partial_sums_per_cta(M, tokens):
+    """Behind the zeroed part: fp32 sums of one tile (128 columns x the widest token tile of the call's class) for each of 160 CTAs."""
+    for op in (tf.TF_OP_GEMM_W4A16, tf.TF_OP_GEMM_W8A16):
+        assert tf.tf_workspace_size(op, M, 4096, 14336) == 1069056 + 160 * 128 * tokens * 4
+
+
 def test_device_calls_check_their_arguments_before_the_library_is_called():
     """The natively marshalled calls: positional and keyword arguments, wrong buffers, and a status that is an error."""
     import torch
