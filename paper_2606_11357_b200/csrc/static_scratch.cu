@@ -30,8 +30,8 @@ static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBy
 
 struct PerDevice {
     std::atomic<int> state;   // 0 = not set up, 1 = ready, -1 = wrong architecture; published after the fields below
-    int sm_count;
-    void* scratch;            // device address of g_static_scratch on this device
+    std::atomic<int> sm_count;
+    std::atomic<void*> scratch;      // device address of g_static_scratch on this device
 };
 PerDevice g_dev[64];
 
@@ -62,8 +62,8 @@ tf_status setup_current_device(PerDevice** out) {
                 return TF_ERR_CUDA;
             }
             if (tf::configure_gemv_kernels() != cudaSuccess) { cudaGetLastError(); return TF_ERR_CUDA; }
-            d.scratch = ptr;
-            d.sm_count = sms;
+            d.scratch.store(ptr, std::memory_order_relaxed);
+            d.sm_count.store(sms, std::memory_order_relaxed);
             state = 1;
         }
         d.state.store(state, std::memory_order_release);
@@ -88,11 +88,12 @@ tf_status tf_gemv_w4a16_static(const void* packed, const void* a_bf16, void* y_b
     tf_status st = setup_current_device(&dev);
     if (st != TF_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // status word and arrival counters must start at zero; the partial sums are always written before read
-    if (cudaMemsetAsync(dev->scratch, 0, tf::kGemvStatusBytes, stream) != cudaSuccess) { cudaGetLastError(); return TF_ERR_CUDA; }
-    const int ctas = dev->sm_count < kStaticMaxGrid ? dev->sm_count : kStaticMaxGrid;
+    void* const scratch = dev->scratch.load(std::memory_order_relaxed);
+    // the status word is this call's; the partial-sum slots are zero at load and again after every call that completes
+    if (cudaMemsetAsync(scratch, 0, tf::kGemvStatusBytes, stream) != cudaSuccess) { cudaGetLastError(); return TF_ERR_CUDA; }
+    const int sm_count = dev->sm_count.load(std::memory_order_relaxed), ctas = sm_count < kStaticMaxGrid ? sm_count : kStaticMaxGrid;
     const tf::GemvPlan plan = tf::plan_gemv(4, M, K, N, ctas);
-    if (tf::launch_gemv(4, plan, packed, a_bf16, y_bf16, M, K, N, dev->scratch, stream) != cudaSuccess) {
+    if (tf::launch_gemv(4, plan, packed, a_bf16, y_bf16, M, K, N, scratch, stream) != cudaSuccess) {
         cudaGetLastError();
         return TF_ERR_CUDA;
     }
