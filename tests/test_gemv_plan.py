@@ -58,7 +58,7 @@ def test_plan_of_the_benchmark_shapes_on_a_b200():
     p = tf.tf_gemv_plan(4, 1, 4096, 32768, 148)
     assert (p["full"], p["consumers"], p["i8"]) == (1, 16, 2)            # 111 tiles over 32 k-tiles: a warp keeps the pieces it has prepared
     p = tf.tf_gemv_plan(8, 1, 4096, 14336, 148)
-    assert (p["full"], p["consumers"], p["i8"]) == (1, 8, 1)             # int8, whole SM: a table would cost a ring stage
+    assert (p["full"], p["consumers"], p["i8"]) == (1, 8, 1)             # int8 tiles: no table (it was the slower form)
     # the decode step's shapes take half an SM; 48 tiles over 32 k-tiles keep their pieces, 24 over 112 and 16 over 32 have none to keep
     assert [tf.tf_gemv_plan(4, 1, K, N, 148)["i8"] for (K, N) in ((4096, 14336), (14336, 4096), (4096, 4096))] == [2, 1, 1]
     for (K, N) in ((4096, 14336), (14336, 4096), (4096, 4096)):

@@ -110,7 +110,7 @@ def test_group_size_mismatch_is_detected_on_the_device():
                                                    ("gemv", 4, 1536, 328, 1069056), ("gemv", 3, 14336, 4096, 1069056), ("gemm", 300, 2048, 1096, 1069056),
                                                    ("gemm", 512, 4096, 640, 1069056)])
 def test_workspace_head_is_left_zero(kind, M, K, N, zero_bytes):
-    """The status word, the arrival counters and the GEMV's partial-sum slots must be zero again after a call, so the
+    """The status word, the GEMM's flags and the GEMV's partial-sum slots must be zero again after a call, so the
     same workspace serves the next call without being cleared."""
     p = wl.make_w4(M, K, N, seed=900 + M)
     blob = torch.from_numpy(gu.pack(p)).cuda()
@@ -259,7 +259,7 @@ def test_gemv_on_two_streams_with_their_own_workspaces():
 
 def test_gemv_and_gemm_share_one_workspace():
     """One workspace of the largest size serves every call of a stream, in any order: the GEMV's partial sums of cut
-    strips and the GEMM's arrival counters must not use the same bytes, and both leave the head of it zero."""
+    strips and the GEMM's flags must not use the same bytes, and both leave the head of it zero."""
     Mv, Mm, K, N = 4, 160, 4096, 4096                       # both shapes cut strips / tiles between CTAs
     pv = wl.make_w4(Mv, K, N, seed=1201)
     pm = wl.make_w4(Mm, K, N, seed=1202)
