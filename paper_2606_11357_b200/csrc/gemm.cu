@@ -27,8 +27,8 @@
 // Work split: whole tiles, or the sequence of (output tile, k-tile) units cut into equal contiguous ranges, one per CTA
 // (split_gemm).  A CTA that computes part of a tile whose last k-tile is another CTA's does that first and writes its fp32 sums
 // to the workspace; the owner of the last k-tile adds them to its own in CTA order (deterministic) and stores y.
-// What bounds it: with 256 tokens the tensor pipe (1060 cycles per k-tile, 1024 of them MMA), the clock being held down by the
-// power limit (1.4 to 1.6 GHz); up to 128 tokens the issue slots of the dequant warps and the waits of the warp that issues
+// What bounds it: with 256 tokens the tensor pipe, 73 % active over a launch (inside a tile a k-tile takes 1060 cycles, 1024 of them
+// MMA; start, drains and cuts bring it to about 1400), at a clock that the power limit holds down in a loop (1.4 to 1.6 GHz); up to 128 tokens the issue slots of the dequant warps and the waits of the warp that issues
 // the MMAs (0.43 to 0.6 us per k-tile), for short calls the 4 to 5 us around them.  Before (eight dequant warps on one k-tile at
 // a time, a packed ring of 26 KB, partial sums through an arrival counter): 0.61 to 0.83 us per k-tile; 32x4096x18944 24.1 ->
 // 20.2 us, 96x2944x11016 18.9 -> 15.0, 297x2944x11016 33.5 -> 25.5, W8 1024x4096x4096 32.9 -> 29.6, 512x4096x4096 31.1 -> 24.3.

@@ -962,9 +962,9 @@ static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool f
     // 18.1 whole SM with 8 / 12 / 16 warps; 4096x14336 int8 15.8 us half SM, 12.7 / 13.3 / 14.6 whole SM with 8 / 12 / 16.
     p.consumers = p.i8 && p.full ? gemv_i8_full_consumers(bits) : gemv_max_consumers(mt, p.full);
     // Floating-point path up to 8 tokens: 12 warps only for long ranges of 4-bit tiles.  Eight have fewer partial sums to add up
-    // at the end of a strip and less of the ring in their hands: 4 tokens 4096x4096 5.54 us against 5.83 with 12, x6144 7.19 and
-    // 7.50, x8192 7.90 and 8.00, then x9472 7.68 and 7.57, x28672 16.35 and 15.75; int8 8 tokens 4096x4096 6.65 and 6.90, x9472
-    // 9.79 and 10.24, x28672 21.5 and 22.3.  (10, 11 and 14 warps are slower than 8, 12 and 16 everywhere, 14336x4096 11.1 us
+    // at the end of a strip and less of the ring in their hands: 4 tokens 4096x4096 5.29 us against 5.59 with 12, x6144 6.82 and
+    // 7.04, x8192 7.55 either way, then x9472 7.37 and 7.33, x14336 9.81 and 9.94, x28672 16.39 and 15.81; int8 8 tokens 4096x4096
+    // 6.42 and 6.71, x9472 9.76 and 10.21, x28672 22.1 and 23.1.  (10, 11 and 14 warps are slower than 8, 12 and 16 everywhere, 14336x4096 11.1 us
     // against 10.6: with a multiple of the tiles of a chunk a warp always works on the same place of a stage, and a stage is
     // freed by warps that are about equally far.)
     if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < kGemvFpTwelveWarpsFromTiles)) p.consumers = 8;
@@ -990,9 +990,9 @@ static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool f
     // whole-SM integer path: a ring deeper than eight stages was slower (1x4096x32768 4-bit: 17.0 / 16.9 / 17.5 us with
     // 6 / 8 / 10 stages; int8 1x4096x14336: 12.8 / 12.5 / 12.7 us with 6 / 8 / 11)
     if (p.i8 && p.full && stages > kGemvI8FullMaxStages) stages = kGemvI8FullMaxStages;
-    // floating-point path up to 8 tokens on 4-bit tiles: five stages (three in the hands of the 12 consumer warps, two in
-    // flight).  Measured at 4 tokens with 4 / 5 / 6 / 7 / 9 stages: 4096x14336 12.2 / 11.6 / 11.7 / 11.9 / 12.3 us,
-    // 4096x32768 20.9 / 19.8 / 19.9 / 20.1 / 20.5 us; int8 tiles (six stages in the warps' hands) want the deep ring:
+    // floating-point path up to 8 tokens on 4-bit tiles: five stages (two in the hands of 8 consumer warps, three in those of 12, the
+    // others in flight).  Measured, with 12 warps, at 4 tokens with 4 / 5 / 6 / 7 / 9 stages: 4096x14336 12.2 / 11.6 / 11.7 / 11.9 / 12.3 us,
+    // 4096x32768 20.9 / 19.8 / 19.9 / 20.1 / 20.5 us; int8 tiles (four or six stages in the warps' hands) want the deep ring:
     // 4096x14336 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us.  (Why a deeper ring is slower on 4-bit tiles was not established;
     // the consumers, not HBM, set the pace of this path.)
     if (!p.i8 && mt == 1 && bits == 4 && stages > kGemvFpW4MaxStages) stages = kGemvFpW4MaxStages;

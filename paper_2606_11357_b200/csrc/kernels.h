@@ -24,10 +24,10 @@ namespace tf {
 //     preparing them per tile.
 //   floating-point path up to 8 tokens: the whole SM and 8 consumer warps, 12 for long ranges of 4-bit tiles; on 4-bit tiles
 //     a ring of five stages (two or three in the warps' hands; deeper was measured slower), on int8 tiles the deepest that fits.
-//     A consumer warp of the floating-point path is bound by instruction issue (about 20 issue cycles per packed
-//     word of 8 weights, measured on registers alone), and since a GEMV may not read its activations before the
-//     kernel ahead of it has completed, only one kernel's consumers work on an SM at a time: three warps per
-//     scheduler beat two warps plus a waiting neighbour (decode step of the benchmark: 133 against 140 us).
+//     A consumer warp of this path needs about 20 issue cycles per packed word of 8 weights (measured on registers alone), and
+//     since a GEMV may not read its activations before the kernel ahead of it has completed, only one kernel's consumers
+//     work on an SM at a time: room for a waiting neighbour is worth less than a deep ring and, on long ranges, a third
+//     warp per scheduler.
 //   9..16 tokens: twice the MMA work per tile and the whole SM, but 8 consumer warps: every tile a warp is working on is a
 //     tile that is not in flight, and 12 warps do not fit the register file.
 __host__ __device__ constexpr int gemv_max_consumers(int mt, bool full, bool i8 = false) { return mt == 1 ? (full ? (i8 ? 16 : 12) : 8) : 8; }
@@ -49,15 +49,15 @@ constexpr int kGemvFullFromBytesI8W4 = TF_I8_FULL_BYTES_W4;
 constexpr int kGemvFullFromBytesI8W8 = TF_I8_FULL_BYTES_W8;
 // 4-bit tiles, the half-SM form without / with its activation pieces kept (piece table).  Figures: us per call in a chain of one
 // shape, one token, half SM / whole SM.
-// Without the table a tile costs a half-SM warp its preparation as well, and eight warps fall behind sixteen: 3584x24576 (303 KB)
-// 12.75 / 11.93, 5120x16384 (291 KB) 12.30 / 11.26, x20480 14.87 / 13.46, 7168x16384 15.41 / 13.45, 9216x12288 15.22 / 13.44.  (In such
-// a chain the forms cross near 235 KB, 3584x18944 9.80 / 9.74, 8192x10240 12.12 / 11.23; the line is at 288 KB, since a pass that goes
-// from half-SM calls to a whole-SM one pays for the change, about 1 us.)
-// With it a tile costs so little that the short start and the neighbour's full ring win: 3072x32768 (349 KB) 12.57 / 13.38,
-// 4096x20480 (287 KB) 11.07 / 11.59, x28672 (403 KB) 13.87 / 14.04; then the two are level: x30720 (432 KB) 14.82 / 14.77, x32768
-// (461 KB) 15.38 / 15.44.  And a pass that stays on half SMs changes no form: the four GEMVs of a layer with 4096x28672 among
-// them 36.0 -> 34.7 us.  The table fits for K of 1024 to 4096 (multiples of 1024) at one token; at two tokens for 1024 and 2048, whose
-// ranges stay below 288 KB (without it 4096x20480 13.62 / 12.13, 3072x26624 13.60 / 12.67).
+// Without the table a tile costs a half-SM warp its preparation as well, and eight warps fall behind sixteen: 3584x18944 (233 KB)
+// 8.79 / 8.91, 5120x13824 (245 KB) 9.64 / 9.36, 5120x16384 (291 KB) 10.86 / 10.24, x20480 (362 KB) 13.26 / 12.22, 7168x16384
+// 13.75 / 12.78.  The forms cross near 240 KB in such a chain; the line is at 288 KB because a pass that goes from half-SM calls
+// to a whole-SM one pays about 1 us for the change (5120x20480 among three half-SM calls, 36.75 / 36.5).
+// With it a tile costs so little that the short start and the neighbour's full ring win: 3072x32768 (349 KB) 11.84 / 11.90,
+// 4096x20480 (291 KB) 10.47 / 10.87, x28672 (403 KB) 13.22 / 13.45, x30720 (432 KB) 14.04 / 14.20.  4096x32768 (461 KB), 14.69 / 14.83,
+// is the longest range that keeps its pieces; there the forms are within 1 %, and it stays on the other side.  The table fits for
+// K of 1024 to 4096 (multiples of 1024) at one token; at two tokens for 1024 and 2048, whose ranges stay below 288 KB (without
+// it 4096x20480 11.89 / 11.33, 3072x26624 11.90 / 11.25).
 constexpr int kGemvFullFromBytesI8W4Kept = 448 * 1024;
 __host__ __device__ constexpr int gemv_i8_full_consumers(int bits) { return bits == 8 ? 8 : 16; }
 constexpr int kGemvI8FullMaxStages = 8;
