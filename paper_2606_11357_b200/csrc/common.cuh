@@ -17,53 +17,42 @@ struct DeviceStatus {
     uint32_t pad[2];
 };
 
-// ---- 4-bit codes -> bf16 --------------------------------------------------------------
-// bf16 0x4300 is 128.0 with a unit in the last place of 1, so OR-ing a 4-bit code into the
-// mantissa gives exactly 128 + q.  Register i of a packed word sits in nibbles i and i+4.
-// Written as one three-input logic op (a & b) | c with mask and magic held in registers; left to
-// the compiler it becomes two two-input ops because each may carry only one immediate.
-__device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
+// ---- codes -> bf16 ------------------------------------------------------------------------
+// A bf16 whose upper eight bits are zero is its lower eight bits times 2^-133 (subnormal up to 127, and the first normal binade
+// continues the line to 255), so a masked code already is a number and one fused multiply-add by a power of two takes it to
+// its place and subtracts the zero point: exactly (q - z) / 64, the 64 being what the largest power of two that bf16 holds,
+// 2^127, leaves over (kCodeUnit; whoever adds the products up multiplies by it, exactly).  Register i of a packed word sits in
+// nibbles i and i + 4; registers 1 and 3 stay sixteen times too large under their mask and get a smaller power of two.
+// Nine instructions per packed word, five of them on the integer pipe, which takes two cycles for each and bounds every loop that
+// unpacks.  (With the code OR-ed into the bf16 128.0 and a subtraction it was eleven and seven: GEMV 4 tokens 4096x28672 15.8 us,
+// now 14.9; 16 tokens 20.2 and 19.4; 6 tokens, group 64, 7424x18440 18.3 and 17.4; int8, 8 tokens, 4096x14336 13.4 and 12.5; GEMM
+// 77x2944x11016, group 32, 16.0 and 15.4, int8 1024x4096x4096 29.6 and 28.9.)  Results do not change: everything is scaled by a
+// power of two, which shows only where sums come within 2^-110 of zero or 2^118 of infinity.
+constexpr float kCodeUnit = 64.f;
+__device__ __forceinline__ uint32_t bf16x2_fma(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t d;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
-__device__ __forceinline__ uint32_t w4_reg_biased(uint32_t word, int i) {
-    uint32_t mask, magic;
-    asm("mov.b32 %0, 0x000F000F;" : "=r"(mask));      // opaque to constant folding on purpose
-    asm("mov.b32 %0, 0x43004300;" : "=r"(magic));
-    return and_or(word >> (4 * i), mask, magic);
+constexpr uint32_t kCodeScale = 0x7F007F00u, kCodeScale16 = 0x7D007D00u;       // 2^127, 2^123
+constexpr uint32_t kMinusCodeScale = 0xFF00FF00u, kMinusCodeScale16 = 0xFD00FD00u;
+__device__ __forceinline__ uint32_t w4_masked(uint32_t word, int i) { return (i & 2 ? word >> 8 : word) & (i & 1 ? 0x00F000F0u : 0x000F000Fu); }
+// Register i of a packed word: (q + minus_zero * 64) / 64 in both halves.
+__device__ __forceinline__ uint32_t w4_reg(uint32_t word, int i, uint32_t minus_zero) {
+    return bf16x2_fma(w4_masked(word, i), i & 1 ? kCodeScale16 : kCodeScale, minus_zero);
 }
-
-__device__ __forceinline__ uint32_t bf16x2_sub(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
+// The zero points of a lane's rows 16 i + g and 16 i + g + 8: -z / 64, each in both halves of a register.
+__device__ __forceinline__ void w4_minus_zero(uint32_t zword, int i, uint32_t& row_g, uint32_t& row_g8) {
+    const uint32_t pair = bf16x2_fma(w4_masked(zword, i), i & 1 ? kMinusCodeScale16 : kMinusCodeScale, 0x80008000u);
+    row_g = __byte_perm(pair, 0, 0x1010);
+    row_g8 = __byte_perm(pair, 0, 0x3232);
 }
-
-// The 8 zero points of a lane: pair i = (128 + z[16i+g], 128 + z[16i+g+8]) as bf16x2, then
-// each half duplicated so it can be subtracted from a (k, k+1) register of that row.
-__device__ __forceinline__ void w4_zero_regs(uint32_t zword, uint32_t zrow_g[4], uint32_t zrow_g8[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        uint32_t pair = w4_reg_biased(zword, i);
-        zrow_g[i] = __byte_perm(pair, 0, 0x1010);
-        zrow_g8[i] = __byte_perm(pair, 0, 0x3232);
-    }
-}
-
-// ---- int8 -> bf16 ---------------------------------------------------------------------
-// Four int8 in a word -> two bf16x2 registers (bytes 0,1 and bytes 2,3), exactly.  A byte is its low seven bits minus 128
-// times its sign bit; OR-ed into the bf16 0x4300 (128.0, unit in the last place 1) the low bits give 128 + low, the sign bit, which
-// falls on the lowest exponent bit, gives 128 or 256, and the difference is the byte.  Eight instructions per word; through the
-// fp32 mantissa (one byte permute and one subtraction per byte) it took eleven.
+// Four int8 in a word -> two bf16x2 registers (bytes 0, 1 and bytes 2, 3), exactly a byte / 64: the byte plus 128, without a
+// sign, then the same multiply-add with -128.  Five instructions per word (through the fraction of 128.0 it took eight).
 __device__ __forceinline__ void w8_word_to_regs(uint32_t word, uint32_t& lo, uint32_t& hi) {
-    uint32_t low, sign, magic;
-    asm("mov.b32 %0, 0x007F007F;" : "=r"(low));       // opaque to constant folding, see w4_reg_biased
-    asm("mov.b32 %0, 0x00800080;" : "=r"(sign));
-    asm("mov.b32 %0, 0x43004300;" : "=r"(magic));
-    const uint32_t a = __byte_perm(word, 0, 0x4140), b = __byte_perm(word, 0, 0x4342);
-    lo = bf16x2_sub(and_or(a, low, magic), and_or(a, sign, magic));
-    hi = bf16x2_sub(and_or(b, low, magic), and_or(b, sign, magic));
+    const uint32_t u = word ^ 0x80808080u;
+    lo = bf16x2_fma(__byte_perm(u, 0, 0x4140), kCodeScale, 0xC000C000u);       // -2
+    hi = bf16x2_fma(__byte_perm(u, 0, 0x4342), kCodeScale, 0xC000C000u);
 }
 
 // ---- warp MMA: D(16x8, fp32) += A(16x16, bf16) . B(16x8, bf16) ---------------------------

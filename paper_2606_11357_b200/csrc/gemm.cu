@@ -163,7 +163,7 @@ struct DrainShare {
         const int n8 = n0 + 8 * (lane & 3), tl = lane >> 2, tok = token0 + tl;
         uint32_t m[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) m[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
+        for (int i = 0; i < 4; ++i) m[i] = pack_bf16(kCodeUnit * v[2 * i], kCodeUnit * v[2 * i + 1]);      // the operand holds weights in 64ths
         stmatrix_x4_trans(smem_u32(tbuf) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane & 7) >> 1)) & 3) * 16, m);
         __syncwarp();
         const uint4 d = *reinterpret_cast<const uint4*>(tbuf + tl * 64 + (((lane & 3) ^ (tl >> 1)) & 3) * 16);
@@ -534,11 +534,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                         if (BITS == 4) {
                             const uint32_t zword = *(reinterpret_cast<const uint32_t*>(tile_smem + w4_zero_offset(G, gr)) + g);
 #pragma unroll
-                            for (int b = 0; b < 2; ++b) {
-                                const uint32_t pair = w4_reg_biased(zword, w0 + b);   // (128 + z[row g], 128 + z[row g+8])
-                                zg[b] = __byte_perm(pair, 0, 0x1010);
-                                zg8[b] = __byte_perm(pair, 0, 0x3232);
-                            }
+                            for (int b = 0; b < 2; ++b) w4_minus_zero(q & 1 ? zword >> 8 : zword, b, zg[b], zg8[b]);
                         }
                     };
                     // four steps of 32 k (two k-blocks, half of a 32-column quarter of the stage each)
@@ -553,10 +549,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                                 const uint32_t xs[2] = {x.x, x.y};
 #pragma unroll
                                 for (int b = 0; b < 2; ++b) {
-                                    op[b][4 * kb + 0] = times_scale(bf16x2_sub(w4_reg_biased(xs[b], 0), zg[b]), s_g[b], l_g[b]);     // row g,   k 0,1
-                                    op[b][4 * kb + 1] = times_scale(bf16x2_sub(w4_reg_biased(xs[b], 2), zg[b]), s_g[b], l_g[b]);     // row g,   k 2,3
-                                    op[b][4 * kb + 2] = times_scale(bf16x2_sub(w4_reg_biased(xs[b], 1), zg8[b]), s_g8[b], l_g8[b]);  // row g+8, k 0,1
-                                    op[b][4 * kb + 3] = times_scale(bf16x2_sub(w4_reg_biased(xs[b], 3), zg8[b]), s_g8[b], l_g8[b]);  // row g+8, k 2,3
+                                    op[b][4 * kb + 0] = times_scale(w4_reg(xs[b], 0, zg[b]), s_g[b], l_g[b]);     // row g,   k 0,1
+                                    op[b][4 * kb + 1] = times_scale(w4_reg(xs[b], 2, zg[b]), s_g[b], l_g[b]);     // row g,   k 2,3
+                                    op[b][4 * kb + 2] = times_scale(w4_reg(xs[b], 1, zg8[b]), s_g8[b], l_g8[b]);  // row g+8, k 0,1
+                                    op[b][4 * kb + 3] = times_scale(w4_reg(xs[b], 3, zg8[b]), s_g8[b], l_g8[b]);  // row g+8, k 2,3
                                 }
                             } else {
                                 const uint4 x = *reinterpret_cast<const uint4*>(tile_smem + (((2 * step + kb) * 2 + (q & 1)) * 32 + lane) * 16);

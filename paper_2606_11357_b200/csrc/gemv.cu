@@ -737,7 +737,9 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                         if (BITS == 4) zword = *(reinterpret_cast<const uint32_t*>(tile + w4_zero_offset(G, gr)) + g);
                     }
                     uint32_t zg[4], zg8[4];
-                    if (BITS == 4) w4_zero_regs(zword, zg, zg8);
+                    if (BITS == 4)
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) w4_minus_zero(zword, w, zg[w], zg8[w]);
                     float gacc[4][MT][4];
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
@@ -761,10 +763,10 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                             if (BITS == 4) {
                                 const uint4 v = wv[0];
                                 const uint32_t x = w == 0 ? v.x : w == 1 ? v.y : w == 2 ? v.z : v.w;
-                                r0 = bf16x2_sub(w4_reg_biased(x, 0), zg[w]);
-                                r1 = bf16x2_sub(w4_reg_biased(x, 1), zg8[w]);
-                                r2 = bf16x2_sub(w4_reg_biased(x, 2), zg[w]);
-                                r3 = bf16x2_sub(w4_reg_biased(x, 3), zg8[w]);
+                                r0 = w4_reg(x, 0, zg[w]);
+                                r1 = w4_reg(x, 1, zg8[w]);
+                                r2 = w4_reg(x, 2, zg[w]);
+                                r3 = w4_reg(x, 3, zg8[w]);
                             } else {
                                 const uint4 v = wv[(w >> 1) % kVecPerKb];
                                 w8_word_to_regs((w & 1) ? v.z : v.x, r0, r1);
@@ -834,10 +836,12 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 for (int mt = 0; mt < MT; ++mt) {
                     const int tok = 8 * mt + 2 * t;
                     if (I8 && t != 0) continue;                 // integer path: tokens 0 and 1 sit in the t = 0 threads, the buffer has two rows
-                    mine[tok * kTileN + 16 * w + g] = acc[w][mt][0];
-                    mine[(tok + 1) * kTileN + 16 * w + g] = acc[w][mt][1];
-                    mine[tok * kTileN + 16 * w + g + 8] = acc[w][mt][2];
-                    mine[(tok + 1) * kTileN + 16 * w + g + 8] = acc[w][mt][3];
+                    // (the floating-point path multiplies with codes in 64ths)
+                    constexpr float kUnit = I8 ? 1.f : kCodeUnit;
+                    mine[tok * kTileN + 16 * w + g] = kUnit * acc[w][mt][0];
+                    mine[(tok + 1) * kTileN + 16 * w + g] = kUnit * acc[w][mt][1];
+                    mine[tok * kTileN + 16 * w + g + 8] = kUnit * acc[w][mt][2];
+                    mine[(tok + 1) * kTileN + 16 * w + g + 8] = kUnit * acc[w][mt][3];
                 }
             __syncwarp();
             if (lane == 0) mbar_arrive(seg_full0 + 8 * rb);

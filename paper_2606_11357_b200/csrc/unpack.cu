@@ -1,13 +1,13 @@
 // Blob -> plain arrays, on the GPU, through the same unpack helpers the GEMV / GEMM use
 // (the "unpacking" step of Section 4.3).  Bit-exact by construction of the helpers: the values
-// 128 + q (4-bit) and q (int8) are exact in bf16 and are turned back into integers here.
+// q / 64 are exact in bf16 and are turned back into integers here.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace tf {
 
-__device__ __forceinline__ int bf16_bits_to_int(uint32_t bits16) {
-    return (int)__uint_as_float(bits16 << 16);
+__device__ __forceinline__ int code_of_bf16(uint32_t bits16) {
+    return (int)(kCodeUnit * __uint_as_float(bits16 << 16));
 }
 
 // One thread per packed word (W4) / per pair of words (W8): thread id -> (strip, ktile, kb, lane, w).
@@ -32,7 +32,7 @@ __global__ void unpack_kernel(const uint8_t* __restrict__ blob, uint8_t* __restr
     if (BITS == 4) {
         const uint32_t x = reinterpret_cast<const uint32_t*>(tile)[(kb * 32 + lane) * 4 + w];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) r[i] = bf16x2_sub(w4_reg_biased(x, i), 0x43004300u);   // exact q
+        for (int i = 0; i < 4; ++i) r[i] = w4_reg(x, i, 0u);                               // exact q / 64
     } else {
         const uint32_t* v = reinterpret_cast<const uint32_t*>(tile) + ((kb * 2 + (w >> 1)) * 32 + lane) * 4 + 2 * (w & 1);
         w8_word_to_regs(v[0], r[0], r[1]);
@@ -45,7 +45,7 @@ __global__ void unpack_kernel(const uint8_t* __restrict__ blob, uint8_t* __restr
             for (int el = 0; el < 2; ++el) {
                 const int k = k0 + 16 * kb + 4 * t + 2 * (i >> 1) + el;
                 const int n = n0 + 16 * w + g + 8 * (i & 1);
-                const int val = bf16_bits_to_int(el ? (r[i] >> 16) : (r[i] & 0xFFFFu));
+                const int val = code_of_bf16(el ? (r[i] >> 16) : (r[i] & 0xFFFFu));
                 if (n < N) q[(size_t)k * N + n] = (uint8_t)val;
             }
     }
@@ -58,7 +58,8 @@ __global__ void unpack_kernel(const uint8_t* __restrict__ blob, uint8_t* __restr
         uint32_t zg[4], zg8[4];
         if (BITS == 4) {
             const uint32_t zword = reinterpret_cast<const uint32_t*>(tile + w4_zero_offset(G, gr))[g];
-            w4_zero_regs(zword, zg, zg8);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w4_minus_zero(zword, i, zg[i], zg8[i]);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -66,8 +67,7 @@ __global__ void unpack_kernel(const uint8_t* __restrict__ blob, uint8_t* __restr
             if (n >= N) continue;
             if (s != nullptr) s[(size_t)grp * N + n] = sc[2 * w + h];
             if (BITS == 4 && z != nullptr) {
-                const uint32_t pair = h ? zg8[0 + w] : zg[0 + w];     // (128 + z) duplicated
-                z[(size_t)grp * N + n] = (uint8_t)(bf16_bits_to_int(pair & 0xFFFFu) - 128);
+                z[(size_t)grp * N + n] = (uint8_t)-code_of_bf16((h ? zg8[w] : zg[w]) & 0xFFFFu);
             }
         }
     }
@@ -119,16 +119,16 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict_
         if (BITS == 4) {
             const uint32_t x = reinterpret_cast<const uint32_t*>(tile)[(kb * 32 + lane) * 4 + w];
             const uint32_t zword = reinterpret_cast<const uint32_t*>(tile + w4_zero_offset(G, gr))[g];
-            const uint32_t pair = w4_reg_biased(zword, w);                         // (128 + z[row g], 128 + z[row g+8])
-            const uint32_t zg = __byte_perm(pair, 0, 0x1010), zg8 = __byte_perm(pair, 0, 0x3232);
+            uint32_t zg, zg8;
+            w4_minus_zero(zword, w, zg, zg8);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) r[i] = bf16x2_sub(w4_reg_biased(x, i), (i & 1) ? zg8 : zg);   // exact q - z
+            for (int i = 0; i < 4; ++i) r[i] = w4_reg(x, i, (i & 1) ? zg8 : zg);              // exact (q - z) / 64
         } else {
             const uint32_t* v = reinterpret_cast<const uint32_t*>(tile) + ((kb * 2 + (w >> 1)) * 32 + lane) * 4 + 2 * (w & 1);
             w8_word_to_regs(v[0], r[0], r[1]);
             w8_word_to_regs(v[1], r[2], r[3]);
         }
-        const float s_g = fp16_bits_to_float(scales[g * 8 + 2 * w]), s_g8 = fp16_bits_to_float(scales[g * 8 + 2 * w + 1]);
+        const float s_g = kCodeUnit * fp16_bits_to_float(scales[g * 8 + 2 * w]), s_g8 = kCodeUnit * fp16_bits_to_float(scales[g * 8 + 2 * w + 1]);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
