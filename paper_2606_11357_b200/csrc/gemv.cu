@@ -27,10 +27,17 @@
 //   reducer warp  : when the consumers finish the tiles of one strip inside this CTA's range they drop
 //                   their fp32 partials into shared memory and move on; the reducer adds them up (fixed
 //                   order), rounds to bf16 and stores y, so the consumers never wait at a strip boundary.
+//   The last segment of a range is on the way of the whole call, and nobody has tiles left: there the consumer warps add up a
+//   slice each (two token rows), and those of the CTA that puts a cut strip together fetch the same slice of the others' sums, asked
+//   for before they wait for their own.  From the last consumer to the end of the kernel it took 2.2 us (4 tokens, 14336x4096)
+//   when the one reducer warp did it, one contributor after the other, and takes 1.0 now.  us per call, before -> after: 16 tokens 14336x4096 12.8 -> 11.0, 4096x6144 8.7 -> 7.1, 4 tokens 4096x4096 5.1 -> 4.5, 14336x4096 9.8 -> 9.0, 6 tokens, group 64,
+//   7424x18440 17.4 -> 16.4, 1 and 16 tokens 32768x1024 10.1 -> 7.2 and 14.1 -> 9.3.  The integer path has one slice; its reducer
+//   does the same, as it has time to look for the others' sums while the consumers work (by a consumer warp: 1 token 14336x4096 8.4
+//   us, by the reducer 8.2).
 //
 // A range may cut a strip (64 output columns) in two.  A CTA that holds a whole strip stores y
-// directly.  Otherwise the reducer writes the fp32 partial to the workspace, and the CTA that has the strip's first tile
-// collects the partials in CTA order (see gather_partial) and stores y, so results are deterministic.  This keeps the
+// directly.  Otherwise its fp32 partial goes to the workspace, and the CTA that has the strip's first tile
+// collects the partials in CTA order (see Gather) and stores y, so results are deterministic.  This keeps the
 // paper's rule that partial sums do not travel between workers for everything but the (at most two) cut strips of a CTA.
 #include <cuda.h>
 
@@ -109,24 +116,19 @@ struct ChunkWalk {
     }
 };
 
-// fp32 [token][64 n] tile held as float4 per lane (element 4 (lane + 32 e)) -> bf16 -> y; rows >= M and columns >= N
-// are not written (N % 8 == 0: a group of 4 columns is in or out)
-template <int kVec>
-__device__ __forceinline__ void store_strip(__nv_bfloat16* y, const float4 (&tot)[kVec], int strip, int M, int N, int lane) {
-#pragma unroll
-    for (int e = 0; e < kVec; ++e) {
-        const int idx = 4 * (lane + 32 * e);
-        const int m = idx / kTileN, n = strip * kTileN + (idx % kTileN);
-        if (m < M && n < N) {
-            uint2 o;
-            o.x = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(tot[e].x)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(tot[e].y)) << 16);
-            o.y = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(tot[e].z)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(tot[e].w)) << 16);
-            *reinterpret_cast<uint2*>(y + (size_t)m * N + n) = o;
-        }
+// A strip's sums are an fp32 tile [token][64 n]; slice e of it is the token rows 2e and 2e + 1, a float4 per lane (row 2e + lane / 16,
+// columns 4 (lane % 16) .. + 3).  A slice rounded to bf16 -> y; rows >= M and columns >= N are not written (N % 8 == 0: a
+// group of 4 columns is in or out).
+__device__ __forceinline__ void store_slice(__nv_bfloat16* y, float4 v, int e, int strip, int M, int N, int lane) {
+    const int m = 2 * e + (lane >> 4), n = strip * kTileN + 4 * (lane & 15);
+    if (m < M && n < N) {
+        uint2 o;
+        o.x = pack_bf16(v.x, v.y);
+        o.y = pack_bf16(v.z, v.w);
+        *reinterpret_cast<uint2*>(y + (size_t)m * N + n) = o;
     }
 }
+__device__ __forceinline__ void add_to(float4& a, float4 v) { a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w; }
 
 // Hand-over of a cut strip without a fence or a counter.  The partial-sum slots of a workspace are all +0.0 bits
 // between calls.  A contributor stores its sums with every +0.0 replaced by -0.0 (the same number), so a word that is
@@ -139,78 +141,41 @@ __device__ __forceinline__ float4 never_plus_zero(float4 v) {
     return make_float4(__uint_as_float(x == 0u ? 0x80000000u : x), __uint_as_float(y == 0u ? 0x80000000u : y),
                        __uint_as_float(z == 0u ? 0x80000000u : z), __uint_as_float(w == 0u ? 0x80000000u : w));
 }
-// `slot` already points at this lane's first float4 of the partial; rows of tokens >= M are neither written nor read.  The
-// partial is added to `acc` and its slot cleared.  Returns false if the wait ran out.  One partial per trip to the L2: with
-// four at once the finisher of a strip shared by four CTAs would wait one trip instead of three, but the gathering code
-// then needs 64 registers more and the whole step was slower (125.7 against 122.6 us; 2 MB shapes gained 0.3 us, 9 MB shapes
-// lost 1 us).  Kept out of line so that the polling loop does not take part in the register allocation of the
-// streaming kernel around it.
-template <int kVec>
-__device__ __noinline__ bool gather_partial(float4* slot, int M, float4 (&acc)[kVec], volatile uint32_t* abort_flag, uint32_t site) {
-    float4 v[kVec];
-    const long long t_begin = clock64();
-    for (;;) {
-        bool here = true;
-#pragma unroll
-        for (int e = 0; e < kVec; ++e) {
-            v[e] = make_float4(-0.f, -0.f, -0.f, -0.f);
-            if (2 * e < M)                       // a real load on every turn of the loop, from the L2
-                asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(v[e].x), "=f"(v[e].y), "=f"(v[e].z), "=f"(v[e].w) : "l"(slot + 32 * e) : "memory");
-        }
-#pragma unroll
-        for (int e = 0; e < kVec; ++e)
-            here = here && __float_as_uint(v[e].x) != 0u && __float_as_uint(v[e].y) != 0u && __float_as_uint(v[e].z) != 0u &&
-                   __float_as_uint(v[e].w) != 0u;
-        if (__all_sync(0xFFFFFFFFu, here)) break;
-        if (wait_given_up(t_begin, abort_flag, site)) return false;
-    }
-#pragma unroll
-    for (int e = 0; e < kVec; ++e) {
-        acc[e].x += v[e].x; acc[e].y += v[e].y; acc[e].z += v[e].z; acc[e].w += v[e].w;
-        if (2 * e < M) __stcg(slot + 32 * e, make_float4(0.f, 0.f, 0.f, 0.f));
-    }
-    return true;
-}
-
-// The same hand-over taken row pair by row pair: for float4 index e (token rows 2e, 2e + 1) the words of up to four
-// consecutive CTAs' partials are requested together, so a strip shared by many CTAs and few tokens costs one trip per
-// row pair instead of one per contributor, in 16 registers.  `slot` points at this lane's first float4 of the first of `count`
-// (<= 4) partials; adds to acc[e] in CTA order.
-template <int kVec>
-__device__ __noinline__ bool gather_rows(float4* slot, int count, int M, float4 (&acc)[kVec], volatile uint32_t* abort_flag, uint32_t site) {
-    constexpr int kSlotVec = kGemvSlotBytes / 16;
-    const long long t_begin = clock64();
-    for (int e = 0; e < kVec && 2 * e < M; ++e) {
-        float4 v[4];
-        for (;;) {
-            bool here = true;
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                v[b] = make_float4(-0.f, -0.f, -0.f, -0.f);
-                if (b < count)
-                    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                 : "=f"(v[b].x), "=f"(v[b].y), "=f"(v[b].z), "=f"(v[b].w) : "l"(slot + b * kSlotVec + 32 * e) : "memory");
-            }
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-                here = here && __float_as_uint(v[b].x) != 0u && __float_as_uint(v[b].y) != 0u && __float_as_uint(v[b].z) != 0u &&
-                       __float_as_uint(v[b].w) != 0u;
-            if (__all_sync(0xFFFFFFFFu, here)) break;
-            if (wait_given_up(t_begin, abort_flag, site)) return false;
-        }
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+// This lane's float4 of the other contributors' slots (kGemvSlotBytes apart, in CTA order): asked for four contributors at a time,
+// one trip to the L2 for all of them, added up in CTA order when all have arrived, and their slots cleared.
+struct Gather {
+    static constexpr int kSlotVec = kGemvSlotBytes / 16;
+    float4* slot;
+    int count;                 // contributors still missing
+    float4 sum, v[4];
+    __device__ __forceinline__ Gather(float4* slot_, int count_) : slot(slot_), count(count_), sum(make_float4(0.f, 0.f, 0.f, 0.f)) {}
+    __device__ __forceinline__ void ask() {
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            a.x += v[b].x; a.y += v[b].y; a.z += v[b].z; a.w += v[b].w;
-            if (b < count) __stcg(slot + b * kSlotVec + 32 * e, make_float4(0.f, 0.f, 0.f, 0.f));
+            v[b] = make_float4(-0.f, -0.f, -0.f, -0.f);
+            if (b < count)                       // a real load every time, from the L2
+                asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(v[b].x), "=f"(v[b].y), "=f"(v[b].z), "=f"(v[b].w) : "l"(slot + b * kSlotVec) : "memory");
         }
-#pragma unroll
-        for (int k = 0; k < kVec; ++k)
-            if (k == e) { acc[k].x += a.x; acc[k].y += a.y; acc[k].z += a.z; acc[k].w += a.w; }
     }
-    return true;
-}
+    // What was asked for, if all of it has arrived (whole warp).
+    __device__ __forceinline__ bool take() {
+        bool here = true;
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            here = here && __float_as_uint(v[b].x) != 0u && __float_as_uint(v[b].y) != 0u && __float_as_uint(v[b].z) != 0u &&
+                   __float_as_uint(v[b].w) != 0u;
+        if (!__all_sync(0xFFFFFFFFu, here)) return false;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            add_to(sum, v[b]);
+            if (b < count) __stcg(slot + b * kSlotVec, make_float4(0.f, 0.f, 0.f, 0.f));
+        }
+        slot += 4 * kSlotVec;
+        count -= 4;
+        return true;
+    }
+};
 
 }  // namespace
 
@@ -287,7 +252,7 @@ __device__ __forceinline__ uint2 act_fragment(const uint8_t* acts, int g, int t,
 struct NoActMap {};
 template <int I8> using GemvActMap = std::conditional_t<I8 == 0, CUtensorMap, NoActMap>;      // floating-point path: [K / 64][M][64] activations
 template <int BITS, int MT, bool FULL, bool CL, int I8, int G = 1>
-__global__ void __launch_bounds__(gemv_max_threads(MT, FULL, I8 != 0), FULL ? 1 : 2)
+__global__ void __launch_bounds__(gemv_max_threads(BITS, MT, FULL, I8 != 0), FULL ? 1 : 2)
 gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t* __restrict__ blob, const __nv_bfloat16* __restrict__ a_glob, __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int total_tiles,
                    int nstages, int stage_bytes, int csize, int nclusters, int xslot_bytes, int nred, int piece_tab,
                    uint8_t* __restrict__ workspace, uint32_t debug) {
@@ -315,7 +280,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     uint8_t* xred = smem + kGemvBarrierBytes + nred * nconsumers * kRedWarp * 4;
     // pscr: integer path.  [consumers][1 KB], a warp's activation pieces of the tile it works on; or
     // [piece_tab][kGemvPieceEntryBytes per token], the pieces of every k-tile of the CTA's range
-    uint32_t* pscr = reinterpret_cast<uint32_t*>(xred + ((CL && csize > 1 ? csize * xslot_bytes : 0) + 1023) / 1024 * 1024);
+    uint32_t* pscr = reinterpret_cast<uint32_t*>(xred + ((CL ? csize * xslot_bytes : 0) + 1023) / 1024 * 1024);
     // abuf [stages][kR][gemv_act_tile_bytes(MT)]: floating-point path, the activations of the tiles in the ring
     uint8_t* abuf = reinterpret_cast<uint8_t*>(pscr) + (I8 == 2 ? (piece_tab * kGemvPieceEntryBytes * M + 1023) / 1024 * 1024 : I8 == 1 ? nconsumers * 1024 : 0);
     constexpr uint32_t kActStageBytes = I8 == 0 ? kR * gemv_act_tile_bytes(MT) : 0;
@@ -330,7 +295,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     // In global mode `nclusters` carries the number of CTAs that take part (the first ones of the grid); the rest
     // of the grid has no tiles and only keeps one CTA of this kernel on every SM (see plan_gemv).
     int cn = nclusters, crank = cta, cbase = 0, ctiles = total_tiles;
-    if (CL && csize > 1) {
+    if (CL) {
         const int q = cta / csize, strips = total_tiles / ktiles;
         const int s0 = range_start(q, strips, nclusters), s1 = range_start(q + 1, strips, nclusters);
         cn = csize; crank = cta - q * csize; cbase = s0 * ktiles; ctiles = (s1 - s0) * ktiles;
@@ -338,7 +303,6 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     const bool idle = crank >= cn;
     const int t0 = idle ? 0 : cbase + range_start(crank, ctiles, cn);
     const int ntiles = idle ? 0 : cbase + range_start(crank + 1, ctiles, cn) - t0;
-    int fin_strip = -1, fin_first = 0;          // cluster mode: the strip this CTA finishes after the cluster barrier
 
     DeviceStatus* status = reinterpret_cast<DeviceStatus*>(workspace);
     float* partials = reinterpret_cast<float*>(workspace + kGemvPartialOffset);
@@ -371,6 +335,64 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     // workspace, thread 0 before it writes the status word.  (What keeps two half-SM CTAs of one GEMV off the same
     // SM when they come in behind a whole-SM kernel is decided at launch: see launch_one.)
     grid_launch_dependents();
+
+    // The sums of slice e of a cut strip, to the CTA that puts it together.  Cluster mode: to that CTA's shared memory (`to`; maybe this
+    // one's), where it adds the slots up in rank order after the cluster barrier at the end of the kernel.  Global mode: to this
+    // CTA's slot of the workspace, with no fence and no counter: the data says by itself that it has arrived.
+    constexpr int kVec = (I8 ? 2 : kTok) / 2;             // slices of a strip
+    auto hand_over = [&](float4 v, int e, int to) {
+        if (CL) {
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(map_to_cta(smem_u32(xred + (size_t)crank * xslot_bytes), (uint32_t)to) + (32 * e + lane) * 16),
+                         "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+        } else {
+            __stcg(reinterpret_cast<float4*>(partials + (size_t)crank * (kGemvMaxM * kTileN)) + 32 * e + lane, never_plus_zero(v));
+        }
+    };
+
+    // The last segment of the range: its strip, and who has the strip's first and last tile.  Global mode: the CTA that holds the
+    // strip's first tile puts a cut strip together.  Its part of the strip is the tail of its range; for every other contributor
+    // the strip is the head of the range, done early, or all of it.
+    struct Last { int strip, first, last; bool whole; };
+    auto last_segment = [&]() {
+        Last l;
+        l.strip = (t0 + max(ntiles, 1) - 1) / ktiles;
+        l.whole = t0 <= l.strip * ktiles && t0 + ntiles == (l.strip + 1) * ktiles;
+        l.first = range_owner(l.strip * ktiles - cbase, ctiles, cn);
+        l.last = range_owner(l.strip * ktiles + ktiles - 1 - cbase, ctiles, cn);
+        return l;
+    };
+    // One warp's part in it: slice e, from buffer rb in its use ru.  What other CTAs hold of a cut strip is asked for before the wait
+    // for this CTA's own sums, by a warp that has nothing else to do (`poll`) again and again.
+    auto finish = [&](const Last& l, int e, int rb, int ru, bool poll) {
+        const bool finisher = !CL && !l.whole && l.first == crank;
+        Gather others(reinterpret_cast<float4*>(partials + (size_t)(crank + 1) * (kGemvMaxM * kTileN)) + 32 * e + lane, finisher ? l.last - crank : 0);
+        const uint32_t bar = seg_full0 + 8 * rb;
+        if (others.count > 0) others.ask();
+        if (poll) {
+            const long long t_begin = clock64();
+            while (others.count > 0) {
+                const bool taken = others.take();
+                if (!taken && __all_sync(0xFFFFFFFFu, mbar_test(bar, ru & 1))) break;
+                if (!taken && wait_given_up(t_begin, abort_flag, 0x430)) return;
+                if (others.count > 0) others.ask();
+            }
+        }
+        if (!mbar_wait_warp(bar, ru & 1, abort_flag, 0x410)) return;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4* src = reinterpret_cast<const float4*>(red + (size_t)rb * nconsumers * kRedWarp) + 32 * e + lane;
+#pragma unroll 4
+        for (int w = 0; w < nconsumers; ++w) add_to(sum, src[w * (kRedWarp / 4)]);         // fixed order: warp 0 + warp 1 + ...
+        if (!l.whole && !finisher) {
+            hand_over(sum, e, l.last);
+            return;
+        }
+        const long long t_begin = clock64();
+        while (others.count > 0)
+            if (!others.take() && wait_given_up(t_begin, abort_flag, 0x440)) return;
+            else if (others.count > 0) others.ask();
+        add_to(sum, others.sum);                            // fixed order: the other contributors in CTA order, then this CTA
+        store_slice(y, sum, e, l.strip, M, N, lane);
+    };
 
     if (warp == 0) {
         // ---------------- producer: stream this CTA's contiguous tile range through the ring --------------
@@ -418,99 +440,45 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
             }
         }
     } else if (warp == 1) {
-        // ---------------- reducer: one strip segment at a time, behind the consumers ------------------------
-        // Lane l owns output elements 4(l + 32e) .. +3 of the [token][64 n] tile (e < kVec), as float4.
+        // ---------------- reducer: one strip segment at a time, behind the consumers, but for the last one ------------------
+        // (The consumer warps put the last segment of the range together themselves: they have nothing else to do then.)
         if (header_ok) {
-            constexpr int kVec = kTok * kTileN / 128;  // float4 per lane
             int sidx = 0, i = 0;
-            bool ok = true;
+            const Last last = I8 ? last_segment() : Last();
             grid_dependency_wait();                    // y and the partial sums belong to earlier kernels until now
-            while (i < ntiles && ok) {
-                const int tile0 = t0 + i;
-                const int strip = tile0 / ktiles, T0 = tile0 - strip * ktiles;
-                const int seg_len = min(ntiles - i, ktiles - T0);
-                const bool whole = seg_len == ktiles;
-                const int c_first = range_owner(strip * ktiles - cbase, ctiles, cn);
-                const int c_last = range_owner(strip * ktiles + ktiles - 1 - cbase, ctiles, cn);
-                // Global mode, cut strip: the CTA that holds the strip's first tile finishes it.  Its part of the strip
-                // is the tail of its range; for every other contributor the strip is the head of the range, done early.
-                const bool finisher = (!CL || csize == 1) && !whole && c_first == crank;
-
-                // While the consumers still work on this segment, collect what the other contributors have dropped
-                // (in CTA order; a partial has arrived when none of its words is +0.0, see gather_partial).
-                float4 others[kVec];
-#pragma unroll
-                for (int e = 0; e < kVec; ++e) others[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (finisher) {
-                    const int nothers = c_last - c_first;
-                    if (nothers > 1 && nothers <= 4 && (M + 1) / 2 < nothers) {
-                        // more contributors than pairs of token rows: row pair by row pair, all contributors at once
-                        float4* slot = reinterpret_cast<float4*>(partials + (size_t)(c_first + 1) * (kGemvMaxM * kTileN)) + lane;
-                        ok = gather_rows<kVec>(slot, nothers, M, others, abort_flag, 0x450);
-                    } else {
-                        for (int c = c_first + 1; c <= c_last && ok; ++c) {
-                            float4* slot = reinterpret_cast<float4*>(partials + (size_t)c * (kGemvMaxM * kTileN)) + lane;
-                            ok = gather_partial<kVec>(slot, M, others, abort_flag, 0x440);
-                        }
-                    }
-                    if (!ok) break;
-                }
-
+            while (i + ktiles - (t0 + i) % ktiles < ntiles) {
+                const int strip = (t0 + i) / ktiles, seg_len = ktiles - (t0 + i) % ktiles;
                 // segment sidx goes through buffer sidx % nred, in that buffer's use number sidx / nred
                 const int rb = nred == 2 ? (sidx & 1) : 0, ru = nred == 2 ? (sidx >> 1) : sidx;
-                ok = mbar_wait_warp(seg_full0 + 8 * rb, ru & 1, abort_flag, 0x400);
-                if (!ok) break;
-                // sum = partial of warp 0 + warp 1 + ... (fixed order); rows of tokens >= M hold zeros
+                if (!mbar_wait_warp(seg_full0 + 8 * rb, ru & 1, abort_flag, 0x400)) break;
                 float4 sum[kVec];
 #pragma unroll
                 for (int e = 0; e < kVec; ++e) sum[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                // (the integer path has at most two tokens, one row pair: a quarter of the loads and additions of this
-                // loop, which for the last segment of a range is the tail of the kernel; a run-time bound on the row
-                // pairs for the other paths made them slower: 36.7 against 35.7 us over the four shapes at 4 tokens)
-                // Four warps' loads in flight at a time: this loop is the tail of every CTA (the last segment's sum sits
-                // between the last consumer warp and the store), and rolled up it cost the decode step 1.8 us (115.7 ->
-                // 113.9; unrolled by 2: 115.3, by 8: 114.7).
-                constexpr int kVecUsed = I8 ? 1 : kVec;
+                // partial of warp 0 + warp 1 + ... (fixed order); rows of tokens >= M hold zeros.  (A run-time bound on the row pairs made
+                // this slower: 36.7 against 35.7 us over four shapes at 4 tokens.)
 #pragma unroll 4
                 for (int w = 0; w < nconsumers; ++w) {
                     const float4* src = reinterpret_cast<const float4*>(red + (size_t)(rb * nconsumers + w) * kRedWarp) + lane;
 #pragma unroll
-                    for (int e = 0; e < kVecUsed; ++e) {
-                        const float4 v = src[32 * e];
-                        sum[e].x += v.x; sum[e].y += v.y; sum[e].z += v.z; sum[e].w += v.w;
-                    }
+                    for (int e = 0; e < kVec; ++e) add_to(sum[e], src[32 * e]);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(seg_free0 + 8 * rb);         // consumers may reuse the buffer
 
-                if (whole || finisher) {
-                    // fixed order: the other contributors in CTA order, then this CTA
+                // A segment that ends its strip is the whole strip or, for the first one, its end: then the sums go to the CTA that
+                // puts the strip together.
+                if (seg_len == ktiles) {
 #pragma unroll
-                    for (int e = 0; e < kVec; ++e) {
-                        sum[e].x += others[e].x; sum[e].y += others[e].y; sum[e].z += others[e].z; sum[e].w += others[e].w;
-                    }
-                    store_strip<kVec>(y, sum, strip, M, N, lane);
-                } else if (CL && csize > 1) {
-                    // cluster mode: hand the partial to the CTA that holds the strip's last tile (maybe this one);
-                    // it adds the slots up in rank order after the cluster barrier at the end of the kernel
-                    const uint32_t remote = map_to_cta(smem_u32(xred + (size_t)crank * xslot_bytes), (uint32_t)c_last);
-#pragma unroll
-                    for (int e = 0; e < kVec; ++e)
-                        if (2 * e < M)
-                            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote + (lane + 32 * e) * 16),
-                                         "f"(sum[e].x), "f"(sum[e].y), "f"(sum[e].z), "f"(sum[e].w) : "memory");
-                    if (c_last == crank) { fin_strip = strip; fin_first = c_first; }
+                    for (int e = 0; e < kVec; ++e) store_slice(y, sum[e], e, strip, M, N, lane);
                 } else {
-                    // Drop this CTA's partial for the finisher and go on: no fence, no counter.  The data says by itself
-                    // that it has arrived: the slot is all +0.0 between calls and no word stored here is +0.0.
-                    float4* mine = reinterpret_cast<float4*>(partials + (size_t)crank * (kGemvMaxM * kTileN)) + lane;
 #pragma unroll
                     for (int e = 0; e < kVec; ++e)
-                        if (2 * e < M) __stcg(mine + 32 * e, never_plus_zero(sum[e]));
+                        if (2 * e < M) hand_over(sum[e], e, crank);
                 }
                 i += seg_len;
                 ++sidx;
             }
+            if (I8 && i < ntiles) finish(last, 0, nred == 2 ? (sidx & 1) : 0, nred == 2 ? (sidx >> 1) : sidx, true);
         }
     } else if (header_ok) {
         // ---------------- consumers ---------------------------------------------------------------------------
@@ -541,6 +509,11 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
         const int piece_n = min(ntiles, ktiles);
         const int T_first = t0 % ktiles;                // k-tile index of the range's first tile
         int piece_e = cw;                               // entry of this warp's next tile (cw < piece_n whenever it has one)
+        // (worked out here, ahead of the wait, or at the end where that costs the tile loop registers: 16 tokens 14336x4096 11.04 us at the
+        // end, 11.22 here; 10 tokens, group 64, 7424x18440 21.6 and 21.0; 4 tokens 4096x4096 4.57 and 4.50)
+        constexpr bool kLastAtEnd = MT == 2 && G == 1;
+        Last last;
+        if (!I8 && !kLastAtEnd) last = last_segment();
         // Everything above touches registers and this CTA's shared memory only; from here on the warp reads activations, or
         // waits for them in the ring (the limit of that wait must not run while earlier kernels do).
         grid_dependency_wait();                         // the activations belong to earlier kernels until now
@@ -847,36 +820,34 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
             if (lane == 0) mbar_arrive(seg_full0 + 8 * rb);
             chunk_base += (seg_len + kR - 1) / kR;
             i += seg_len;
-            ++sidx;
+            if (i < ntiles) { ++sidx; continue; }
+
+            // ---- the last segment: put together by these warps, a slice each, on the integer path (one slice) by the reducer ----
+            if (kLastAtEnd) last = last_segment();
+            if (!I8)
+                for (int e = cw; e < kVec && 2 * e < M; e += nconsumers) finish(last, e, rb, ru, false);
         }
     }
 
-    // ---------------- cluster mode: finish the strip whose last tile this CTA holds -----------------------------
+    // ---------------- cluster mode: put together the strip whose last tile this CTA holds ------------------------
     __syncthreads();
-    if (CL && csize > 1) {
+    if (CL) {
         // Every CTA of the cluster gets here (all waits above are bounded).  After the barrier the partials the
         // other CTAs stored into this CTA's slots are visible, and nobody touches another CTA's memory again.
+        const int strip = t0 / ktiles, head = t0 - strip * ktiles;              // cut before this CTA, ended by it
+        const bool mine = ntiles > 0 && head > 0 && head + ntiles >= ktiles;
+        const int first = range_owner(strip * ktiles - cbase, ctiles, cn);
+        const bool some_empty = ctiles < cn;            // a range can be empty only where the cluster has fewer tiles than CTAs
         cluster_sync_all();
-        if (warp == 1 && fin_strip >= 0 && header_ok && *abort_flag == 0) {
-            constexpr int kVec = kTok * kTileN / 128;
-            float4 tot[kVec];
-#pragma unroll
-            for (int e = 0; e < kVec; ++e) tot[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            // (a range can be empty only where the cluster has fewer tiles than CTAs: the divisions of
-            // range_start stay out of this loop, which is the tail of the kernel, in every other case)
-            const bool some_empty = ctiles < cn;
+        if (mine && warp >= 2 && header_ok && *abort_flag == 0)
+        for (int e = warp - 2; e < kVec && 2 * e < M; e += nconsumers) {
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 2
-            for (int c = fin_first; c <= crank; ++c) {                     // rank order, as in global mode
+            for (int c = first; c <= crank; ++c) {                             // rank order, as in global mode
                 if (some_empty && range_start(c + 1, ctiles, cn) == range_start(c, ctiles, cn)) continue;   // empty range: no partial
-                const float4* src = reinterpret_cast<const float4*>(xred + (size_t)c * xslot_bytes) + lane;
-#pragma unroll
-                for (int e = 0; e < kVec; ++e)
-                    if (2 * e < M) {
-                        const float4 v = src[32 * e];
-                        tot[e].x += v.x; tot[e].y += v.y; tot[e].z += v.z; tot[e].w += v.w;
-                    }
+                add_to(sum, reinterpret_cast<const float4*>(xred + (size_t)c * xslot_bytes)[32 * e + lane]);
             }
-            store_strip<kVec>(y, tot, fin_strip, M, N, lane);
+            store_slice(y, sum, e, strip, M, N, lane);
         }
     }
 
@@ -941,7 +912,7 @@ static int max_resident_clusters(int csize) {
         int n = 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(csize * 64, 1, 1);
-        cfg.blockDim = dim3(gemv_max_threads(2, true), 1, 1);
+        cfg.blockDim = dim3(gemv_max_threads(BITS, 2, true, false), 1, 1);
         cfg.dynamicSmemBytes = gemv_smem_budget(2, true);
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -30,8 +30,11 @@ namespace tf {
 //     warp per scheduler.
 //   9..16 tokens: twice the MMA work per tile and the whole SM, but 8 consumer warps: every tile a warp is working on is a
 //     tile that is not in flight, and 12 warps do not fit the register file.
-__host__ __device__ constexpr int gemv_max_consumers(int mt, bool full, bool i8 = false) { return mt == 1 ? (full ? (i8 ? 16 : 12) : 8) : 8; }
-__host__ __device__ constexpr int gemv_max_threads(int mt, bool full, bool i8 = false) { return 32 * (gemv_max_consumers(mt, full, i8) + 2); }   // + producer + reducer
+__host__ __device__ constexpr int gemv_i8_full_consumers(int bits) { return bits == 8 ? 8 : 16; }
+__host__ __device__ constexpr int gemv_max_consumers(int mt, bool full) { return mt == 1 ? (full ? 12 : 8) : 8; }      // floating-point path, half-SM form
+__host__ __device__ constexpr int gemv_max_threads(int bits, int mt, bool full, bool i8) {
+    return 32 * ((i8 && full ? gemv_i8_full_consumers(bits) : gemv_max_consumers(mt, full)) + 2);      // + producer + reducer
+}
 __host__ __device__ constexpr int gemv_smem_budget(int mt, bool full) { return (mt == 1 && !full ? 110 : 220) * 1024; }
 // Shared memory a half-SM CTA asks for when two of its kind must not share an SM: with 228 KB per SM and 1 KB reserved
 // per CTA, two of these do not fit (2 x 115 KB), one beside a plain half-SM CTA (at most 110 KB) does.
@@ -59,7 +62,6 @@ constexpr int kGemvFullFromBytesI8W8 = TF_I8_FULL_BYTES_W8;
 // K of 1024 to 4096 (multiples of 1024) at one token; at two tokens for 1024 and 2048, whose ranges stay below 288 KB (without
 // it 4096x20480 11.89 / 11.33, 3072x26624 11.90 / 11.25).
 constexpr int kGemvFullFromBytesI8W4Kept = 448 * 1024;
-__host__ __device__ constexpr int gemv_i8_full_consumers(int bits) { return bits == 8 ? 8 : 16; }
 constexpr int kGemvI8FullMaxStages = 8;
 constexpr int kGemvFpW4MaxStages = 5;
 constexpr int kGemvFpTwelveWarpsFromTiles = 32;
@@ -81,7 +83,7 @@ constexpr int kGemvMaxGrid = 256;             // CTAs (one per SM); sizes the pa
 //   (16 tokens x 64 columns fp32) per persistent CTA | behind them the GEMM's partial tiles (written before they are
 //   read, so the GEMM may leave anything there).
 // Everything below kWorkspaceZeroBytes is zero between calls: the GEMV's hand-over of a cut strip relies on its slots
-// being all +0.0 bits (see gather_partial in gemv.cu), the GEMM on its flags.
+// being all +0.0 bits (see Gather in gemv.cu), the GEMM on its flags.
 constexpr int kWorkspaceHeadBytes = 20480;
 constexpr int kGemvStatusBytes = 256;         // what the GEMV itself needs cleared besides its slots
 constexpr int kGemvPartialOffset = kWorkspaceHeadBytes;
