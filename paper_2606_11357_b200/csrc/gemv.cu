@@ -56,22 +56,22 @@ namespace {
 // Integer warp MMA: D(16x8, s32) += A(16x32, s8) . B(32x8, s8).  Thread (g, t): a0 = row g, k 4t..4t+3; a1 = row g+8;
 // a2, a3 = the same rows, k + 16; b0 = column g, k 4t..4t+3; b1 = k + 16; d = rows g, g+8 x columns 2t, 2t+1.
 __device__ __forceinline__ void mma_s8_16832(int d[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 // The same with D = A . B + c in every element (no accumulator to set first).
 __device__ __forceinline__ void mma_s8_16832_first(int d[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, int c) {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
                  : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c));
 }
 
 // The same shapes with unsigned bytes in the 16-row operand (4-bit codes 0..15 as they come out of a packed word).
 __device__ __forceinline__ void mma_u8s8_16832(int d[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 __device__ __forceinline__ void mma_u8s8_16832_first(int d[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, int c) {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
                  : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c));
 }
 
@@ -182,28 +182,24 @@ struct Gather {
 // Integer path: the activation pieces of one k-tile (up to two tokens), from the raw bf16 of lane L (k = 4L .. 4L+3).
 // dst: [column][kGemvPieceColWords] piece words, the word of lane L at (L & 3) * 8 + (L >> 2), so that a thread of the
 // MMA phase finds the eight k-blocks of its column and k quarter in two 16-byte loads (columns 36 words apart fall
-// into different banks); meta: [column] {2^(emax-148) 256^j, sum of the piece over the tile} in 8-byte entries, a
-// thread's two columns = one 16-byte load (with 4-byte entries and an 8-byte load the same kernel ran 12 % slower:
-// measured, cause not established).
+// into different banks).  unit[m]: 2^(emax - 148), what the integers of token m are multiples of.
+// KEEP (pieces that serve several tiles): also meta: [column] {unit 256^j, sum of the piece over the tile} in 8-byte entries, a thread's two
+// columns = one 16-byte load (with 4-byte entries and an 8-byte load the same kernel ran 12 % slower: measured, cause not established).
 constexpr int kGemvPieceColWords = 36;
-template <int BITS>
-__device__ __forceinline__ void make_pieces(const uint2 (&raws)[2], uint32_t* dst, uint2* meta, int M, int lane) {
+template <int BITS, bool KEEP>
+__device__ __forceinline__ void make_pieces(const uint2 (&raws)[2], uint32_t* dst, uint2* meta, float (&unit)[2], int M, int lane) {
     constexpr int kColWords = kGemvPieceColWords;
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
         if (m < M) {
-            const uint2 raw = raws[m];
-            const uint32_t x0 = raw.x, x1 = raw.y;
-            uint32_t e = max(max((x0 << 17) >> 24, (x0 << 1) >> 24), max((x1 << 17) >> 24, (x1 << 1) >> 24));
-            e = __reduce_max_sync(0xFFFFFFFFu, e);
-            e = max(e, 22u);                                  // keeps both powers of two normal numbers
+            const uint32_t x0 = raws[m].x, x1 = raws[m].y;
+            const uint32_t pair = __vmaxu2(x0 & 0x7FFF7FFFu, x1 & 0x7FFF7FFFu);
+            const uint32_t e = max(__reduce_max_sync(0xFFFFFFFFu, max(pair >> 16, pair & 0xFFFFu)) >> 7, 22u);      // at least 22: keeps both powers of two normal numbers
             const float mult = __uint_as_float((275u - e) << 23);          // 2^(148 - emax)
-            // v + 0x808080 has the bytes p0 + 128, p1 + 128, p2 + 128 of the balanced split
-            uint32_t v[4];
-            v[0] = (uint32_t)__float2int_rn(__uint_as_float(x0 << 16) * mult) + 0x808080u;
-            v[1] = (uint32_t)__float2int_rn(__uint_as_float(x0 & 0xFFFF0000u) * mult) + 0x808080u;
-            v[2] = (uint32_t)__float2int_rn(__uint_as_float(x1 << 16) * mult) + 0x808080u;
-            v[3] = (uint32_t)__float2int_rn(__uint_as_float(x1 & 0xFFFF0000u) * mult) + 0x808080u;
+            // rint(a mult) = v in the low bits of 1.5 * 2^23 + a mult (no conversion unit), and on to v + 0x808080, whose bytes are p0 + 128,
+            // p1 + 128, p2 + 128 of the balanced split (what is left above them is not used)
+            const auto biased = [&](uint32_t bits) { return __float_as_uint(fmaf(__uint_as_float(bits), mult, kIntAsFloatBiasValue)) + (0x808080u - 0x400000u); };
+            const uint32_t v[4] = {biased(x0 << 16), biased(x0 & 0xFFFF0000u), biased(x1 << 16), biased(x1 & 0xFFFF0000u)};
             // 4 x 3 byte transpose: one word per piece, bytes in the k order of the weight operand's bytes
             // (int8: k, k+1, k+2, k+3; 4-bit: k, k+2, k+1, k+3, the order of a packed word's nibble pairs)
             const uint32_t ab01 = __byte_perm(v[0], v[1], 0x5140), ab2 = __byte_perm(v[0], v[1], 0x0062);
@@ -212,19 +208,20 @@ __device__ __forceinline__ void make_pieces(const uint2 (&raws)[2], uint32_t* ds
             word[0] = __byte_perm(ab01, cd01, BITS == 8 ? 0x5410 : 0x5140) ^ 0x80808080u;
             word[1] = __byte_perm(ab01, cd01, BITS == 8 ? 0x7632 : 0x7362) ^ 0x80808080u;
             word[2] = __byte_perm(ab2, cd2, BITS == 8 ? 0x5410 : 0x5140) ^ 0x80808080u;
-            // 2^(emax - 148); an Inf or NaN among the 128 activations makes this token's outputs NaN
-            const float se = e == 255u ? __uint_as_float(0x7FC00000u) : __uint_as_float((e - 21u) << 23);
+            // an Inf or NaN among the 128 activations makes this token's outputs NaN
+            unit[m] = e == 255u ? __uint_as_float(0x7FC00000u) : __uint_as_float((e - 21u) << 23);
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const int c = 3 * m + j;
                 dst[c * kColWords + (lane & 3) * 8 + (lane >> 2)] = word[j];
-                int psum = 0;                           // 4-bit: sum of the piece over the tile's 128 k, for the zero point
-                if constexpr (BITS == 4) psum = __reduce_add_sync(0xFFFFFFFFu, __dp4a((int)word[j], 0x01010101, 0));
-                if (lane == 0) meta[c] = make_uint2(__float_as_uint(se * (j == 0 ? 1.f : j == 1 ? 256.f : 65536.f)), (uint32_t)psum);
+                if constexpr (KEEP) {
+                    const int psum = __reduce_add_sync(0xFFFFFFFFu, __dp4a((int)word[j], 0x01010101, 0));
+                    if (lane == 0) meta[c] = make_uint2(__float_as_uint(unit[m] * (j == 0 ? 1.f : j == 1 ? 256.f : 65536.f)), (uint32_t)psum);
+                }
             }
         }
     }
-    if (lane == 0) {                                    // columns without a token contribute nothing
+    if (KEEP && lane == 0) {                            // columns without a token contribute nothing
 #pragma unroll
         for (int c = 3; c < 8; ++c)
             if (c >= 3 * M) meta[c] = make_uint2(0u, 0u);
@@ -234,7 +231,8 @@ __device__ __forceinline__ void make_pieces(const uint2 (&raws)[2], uint32_t* ds
 // loop's register allocation.
 template <int BITS>
 __device__ __noinline__ void make_pieces_call(const uint2 (&raws)[2], uint32_t* dst, uint2* meta, int M, int lane) {
-    make_pieces<BITS>(raws, dst, meta, M, lane);
+    float unit[2];
+    make_pieces<BITS, true>(raws, dst, meta, unit, M, lane);
 }
 
 // Floating-point path: token g + 8 mt, k = 16 kb + 4t .. +3 of a tile's activations in the ring.  The 16-byte units of a row are
@@ -311,9 +309,31 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
 
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kGemvMaxStages);
     const uint32_t seg_full0 = smem_u32(bars + 2 * kGemvMaxStages), seg_free0 = seg_full0 + 16;
+    // Integer path: the lane that issues the weight copies initialises the barriers of the ring itself, while the header of the blob is on
+    // its way, and issues the first chunk ahead of the barrier that the others meet at (packed weights are constants; 1 token 4096x4096
+    // 4.24 -> 4.00 us.  On the floating-point path it changed nothing.)
+    ChunkWalk early(t0, I8 != 0 ? ntiles : 0, ktiles, blob + kHeaderBytes, kTileBytes);
+    int issued = 0;                                     // chunks
+    auto issue_weights = [&](ChunkWalk& walk, int c) {
+        int tiles_here, T;
+        const uint8_t* src;
+        walk.next(kR, tiles_here, T, src);
+        stage_tag[c] = (uint32_t)c;
+        mbar_arrive_expect_tx(full0 + 8 * c, (uint32_t)tiles_here * kTileBytes + kActStageBytes);
+        bulk_copy_g2s(smem_u32(ring + (size_t)c * stage_bytes), src, (uint32_t)tiles_here * kTileBytes, full0 + 8 * c);
+    };
+    if (I8 != 0 && threadIdx.x == 0) {
+        for (int s = 0; s < nstages; ++s) {
+            mbar_init(full0 + 8 * s, 1);
+            mbar_init(empty0 + 8 * s, kR);
+            stage_tag[s] = 0xFFFFFFFFu;
+        }
+        mbar_init_fence();
+        if (header_ok && (debug & kDebugDropWeights) == 0 && !early.done()) issue_weights(early, issued++);
+    }
     // One thread per ring stage, one more for the rest: the set-up sits between the start of a CTA and its first
     // weight copy (one thread doing all of it in turn cost the decode step 1.7 us).
-    if (threadIdx.x < (unsigned)nstages) {
+    if (I8 == 0 && threadIdx.x < (unsigned)nstages) {
         const int s = threadIdx.x;
         mbar_init(full0 + 8 * s, 1);
         mbar_init(empty0 + 8 * s, kR);           // every tile of a chunk is released by its consumer warp
@@ -401,18 +421,11 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
         // with consumer warps that never idle.  The packed weights are constants: the first ring fill of them does not
         // wait for the kernels before this one and is on its way while they finish.
         if (lane == 0 && header_ok && (debug & kDebugDropWeights) == 0) {
-            ChunkWalk walk(t0, ntiles, ktiles, blob + kHeaderBytes, kTileBytes);
+            ChunkWalk walk = I8 != 0 ? early : ChunkWalk(t0, ntiles, ktiles, blob + kHeaderBytes, kTileBytes);
             // first ring fill, weights only: they are constants, so they may be fetched before the dependency wait
             if constexpr (I8 == 0) prefetch_tensormap(&act_map);
-            int cg = 0;
-            for (; cg < nstages && !walk.done(); ++cg) {
-                int tiles_here, T;
-                const uint8_t* src;
-                walk.next(kR, tiles_here, T, src);
-                stage_tag[cg] = (uint32_t)cg;
-                mbar_arrive_expect_tx(full0 + 8 * cg, (uint32_t)tiles_here * kTileBytes + kActStageBytes);
-                bulk_copy_g2s(smem_u32(ring + (size_t)cg * stage_bytes), src, (uint32_t)tiles_here * kTileBytes, full0 + 8 * cg);
-            }
+            int cg = issued;
+            for (; cg < nstages && !walk.done(); ++cg) issue_weights(walk, cg);
             if constexpr (I8 == 0) {                             // the activations of that first fill
                 grid_dependency_wait();
                 ChunkWalk first(t0, ntiles, ktiles, blob, kTileBytes);
@@ -518,6 +531,9 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
         // waits for them in the ring (the limit of that wait must not run while earlier kernels do).
         grid_dependency_wait();                         // the activations belong to earlier kernels until now
         if (I8 != 0 && cw < ntiles) load_araw(a_glob + (size_t)T_act * kTileK);
+        // powers of 256 by which the pieces of this thread's columns 2t and 2t + 1 count (0: a column without a token)
+        const float pow_x = t == 0 ? 1.f : t == 1 ? 65536.f : t == 2 && M == 2 ? 256.f : 0.f;
+        const float pow_y = t == 0 ? 256.f : M == 1 ? 0.f : t == 1 ? 1.f : t == 2 ? 65536.f : 0.f;
         int T0 = T_first;                               // k-tile index at which the current segment starts (0 after the first)
         int j = cw;                                     // this warp's next tile, as a local index of the CTA's range
         while (i < ntiles && !aborted) {
@@ -549,12 +565,16 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 cg_cur = cg;
                 while (s_cur >= nstages) { s_cur -= nstages; ++use_cur; }
                 const int s = s_cur;
-                if (!__all_sync(0xFFFFFFFFu, stage_tag[s] == (uint32_t)cg)) {      // the producer has not reached this chunk yet
+                // (the tag and then the barrier, both asked for before either answer is looked at: what is seen of the barrier
+                // is later than the tag, so it is about this chunk if the tag is this chunk's.  One vote and one trip to shared memory
+                // per tile instead of two: a pass over four layer shapes at 1 / 4 / 16 tokens 31.2 / 34.3 / 44.1 -> 30.9 / 34.1 / 43.8 us)
+                const bool tagged = stage_tag[s] == (uint32_t)cg, landed = mbar_try_wait(full0 + 8 * s, use_cur & 1);
+                if (!__all_sync(0xFFFFFFFFu, tagged && landed)) {
                     const long long t_begin = clock64();
-                    while (!__all_sync(0xFFFFFFFFu, stage_tag[s] == (uint32_t)cg))
+                    while (!__all_sync(0xFFFFFFFFu, stage_tag[s] == (uint32_t)cg))      // the producer has not reached this chunk yet
                         if (wait_given_up(t_begin, abort_flag, 0x280 + s)) return false;
+                    if (!mbar_wait_warp(full0 + 8 * s, use_cur & 1, abort_flag, 0x200 + s)) return false;
                 }
-                if (!mbar_wait_warp(full0 + 8 * s, use_cur & 1, abort_flag, 0x200 + s)) return false;
                 nx_tile = ring + (size_t)s * stage_bytes + (size_t)slot * kTileBytes;
                 nx_s = s; nx_slot = slot; nx_cl = cl;
                 if constexpr (!I8) {
@@ -589,7 +609,8 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                     //     y[m][n] += s[n] 2^(emax-148) sum_j 256^j D[n][3m+j]
                     static_assert(!I8 || MT == 1, "the integer path is built for up to 2 tokens");
                     const uint32_t* scr;                                // this tile's piece words and column metadata
-                    const uint2* col_meta;
+                    float2 col_scale;
+                    int p0 = 0, p1 = 0;                                 // sums of the pieces of this thread's columns over the tile's 128 k
                     if constexpr (I8 == 2) {
                         uint32_t* ent = pscr + piece_e * piece_entry_words;
                         uint2* ent_meta = reinterpret_cast<uint2*>(ent + 3 * kColWords * M);
@@ -599,23 +620,25 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                             // (as a call in the whole-SM form with its 96 registers: inlined it spilled inside the tile loop,
                             // 17.8 against 17.1 us on 1x4096x32768; inlined in the half-SM form, where the call was the
                             // slower one, 12.0 against 10.9 us on 1x4096x14336)
+                            float unit[2];
                             if constexpr (FULL) make_pieces_call<BITS>(araw, ent, ent_meta, M, lane);
-                            else make_pieces<BITS>(araw, ent, ent_meta, M, lane);
+                            else make_pieces<BITS, true>(araw, ent, ent_meta, unit, M, lane);
                             if (j + nconsumers < piece_n) load_araw(next_base);    // later visits need no activations
                             __syncwarp();
                         }
                         scr = ent;
-                        col_meta = ent_meta;
+                        const uint4 cm = *reinterpret_cast<const uint4*>(ent_meta + 2 * t);
+                        col_scale = make_float2(__uint_as_float(cm.x), __uint_as_float(cm.z));
+                        p0 = (int)cm.y; p1 = (int)cm.w;
                     } else {
                         uint32_t* mine_scr = pscr + cw * 256;
-                        make_pieces<BITS>(araw, mine_scr, reinterpret_cast<uint2*>(mine_scr + 216), M, lane);
+                        float unit[2] = {0.f, 0.f};
+                        make_pieces<BITS, false>(araw, mine_scr, nullptr, unit, M, lane);
                         scr = mine_scr;
-                        col_meta = reinterpret_cast<const uint2*>(mine_scr + 216);
+                        col_scale = make_float2((t >= 2 ? unit[1] : unit[0]) * pow_x, (t >= 1 ? unit[1] : unit[0]) * pow_y);
                         if (has_next) load_araw(next_base);             // the next tile's activations, under this tile's MMAs
                         __syncwarp();
                     }
-                    const uint4 cm = *reinterpret_cast<const uint4*>(col_meta + 2 * t);
-                    const float2 col_scale = make_float2(__uint_as_float(cm.x), __uint_as_float(cm.z));
                     uint32_t bw[8];                                     // column g: the words of k-blocks 0..7 for this t
 #pragma unroll
                     for (int i = 0; i < 8; ++i) bw[i] = 0u;
@@ -626,6 +649,11 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                         bw[4] = hi.x; bw[5] = hi.y; bw[6] = hi.z; bw[7] = hi.w;
                     }
                     if constexpr (I8 == 1) __syncwarp();                // the scratch is rewritten for the next tile
+                    // 4-bit: one AND per packed word instead of two, no accumulator to set first, one addition per sum more, and a byte times a
+                    // piece summed over 128 k still stays below 2^22.  1 token 14336x4096 8.04 -> 7.85 us, 2 tokens 4096x4096 4.42 -> 4.01
+                    // (both with the piece sums by MMA, below).  Not in the half-SM form with kept pieces, whose 96 registers it overflows:
+                    // 4096x28672 12.85 us without, 13.1 with it.
+                    constexpr bool kWholeBytes = FULL || I8 == 1;
                     int d[4][4];
                     if constexpr (BITS == 4) {
 #pragma unroll
@@ -636,13 +664,12 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                             for (int w = 0; w < 4; ++w) {
                                 const uint32_t x0 = w == 0 ? v0.x : w == 1 ? v0.y : w == 2 ? v0.z : v0.w;
                                 const uint32_t x1 = w == 0 ? v1.x : w == 1 ? v1.y : w == 2 ? v1.z : v1.w;
-                                // Row g: the low nibbles.  Row g + 8: the high nibbles stay where they are, so the row carries
-                                // 16 q (at most 240, still an unsigned byte), its sums come out 16 times too large and its scale
-                                // is taken 16 times smaller below (all exact; |16 (q - z) p| summed over 128 k stays below 2^22).
-                                // One AND per operand register instead of a shift and an AND: 32 instructions less per tile.
-                                const uint32_t a0 = x0 & 0x0F0F0F0Fu, a1 = x0 & 0xF0F0F0F0u;            // k-block 2i
-                                const uint32_t a2 = x1 & 0x0F0F0F0Fu, a3 = x1 & 0xF0F0F0F0u;            // k-block 2i + 1
-                                if (i == 0) mma_u8s8_16832_first(d[w], a0, a1, a2, a3, bw[0], bw[1], kIntAsFloatBias);
+                                // Row g: the low nibbles.  Row g + 8: the high nibbles, left in place: the row carries 16 q, its sums come
+                                // out 16 times too large and its scale is taken 16 times smaller below (all exact).  With kWholeBytes
+                                // the whole bytes, 16 q + row g's code, and row g's sum is taken off again below.
+                                const uint32_t a0 = x0 & 0x0F0F0F0Fu, a1 = kWholeBytes ? x0 : x0 & 0xF0F0F0F0u;            // k-block 2i
+                                const uint32_t a2 = x1 & 0x0F0F0F0Fu, a3 = kWholeBytes ? x1 : x1 & 0xF0F0F0F0u;            // k-block 2i + 1
+                                if (i == 0) mma_u8s8_16832_first(d[w], a0, a1, a2, a3, bw[0], bw[1], kWholeBytes ? 0 : kIntAsFloatBias);
                                 else mma_u8s8_16832(d[w], a0, a1, a2, a3, bw[2 * i], bw[2 * i + 1]);
                             }
                         }
@@ -671,14 +698,27 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                     }
                     }
                     if constexpr (BITS == 4) {
+                        if constexpr (I8 == 1) {                        // a row of ones times the same operand (four MMAs instead of three reductions over the warp)
+                            int ones[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                if (i == 0) mma_u8s8_16832_first(ones, 0x01010101u, 0u, 0x01010101u, 0u, bw[0], bw[1], 0);
+                                else mma_u8s8_16832(ones, 0x01010101u, 0u, 0x01010101u, 0u, bw[2 * i], bw[2 * i + 1]);
+                            }
+                            p0 = ones[0]; p1 = ones[1];
+                        }
                         // zero point: every code of row n stands for q - z[n], so the row's sum loses z[n] times the column's piece sum
                         const uint32_t zword = *(reinterpret_cast<const uint32_t*>(tile + kWeightBytes + kScaleBytes) + g);
-                        const int p0 = (int)cm.y, p1 = (int)cm.w;
 #pragma unroll
                         for (int w = 0; w < 4; ++w) {
                             const int zr = (int)((zword >> (4 * w)) & 15u), zr8 = (int)((zword >> (4 * w + 12)) & 0xF0u);     // z, 16 z
-                            d[w][0] -= zr * p0; d[w][1] -= zr * p1;
-                            d[w][2] -= zr8 * p0; d[w][3] -= zr8 * p1;
+                            if constexpr (kWholeBytes) {
+                                d[w][2] += (kIntAsFloatBias - zr8 * p0) - d[w][0]; d[w][3] += (kIntAsFloatBias - zr8 * p1) - d[w][1];
+                                d[w][0] += kIntAsFloatBias - zr * p0; d[w][1] += kIntAsFloatBias - zr * p1;
+                            } else {
+                                d[w][0] -= zr * p0; d[w][1] -= zr * p1;
+                                d[w][2] -= zr8 * p0; d[w][3] -= zr8 * p1;
+                            }
                         }
                     }
                     __syncwarp();

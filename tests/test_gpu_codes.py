@@ -72,3 +72,19 @@ def test_a_power_of_two_goes_through_unchanged(kind, M, bits):
     for e in (-80, 100):
         y = _linear(kind, bits, blob, (a * 2.0 ** e).bfloat16(), K, N, 128).double()
         assert torch.equal(y, plain * 2.0 ** e)
+
+
+@pytest.mark.parametrize("value", [1.9921875, -1.9921875, 1.0078125])
+@pytest.mark.parametrize("M,K,N", [(1, 512, 128), (2, 512, 128), (1, 6144, 14400), (1, 1024, 19008)])
+def test_integer_path_at_the_ends_of_its_ranges(M, K, N, value):
+    """Codes and zero points 0 and 15 against activations that are all the same number: the largest sums that the integers of a tile
+    reach, in the forms with and without kept pieces.  Scale 2^-6, so every sum of a tile and over K is exact in fp32 and only the
+    store rounds."""
+    n = np.arange(N)
+    q = np.broadcast_to(np.where(n & 1, 15, 0).astype(np.uint8), (K, N))
+    z = np.broadcast_to(np.where(n & 2, 15, 0).astype(np.uint8), (K // 128, N))
+    blob = torch.from_numpy(tf.tf_pack_awq(wl.awq_pack_words(q), np.full((K // 128, N), 2.0 ** -6, np.float16), wl.awq_pack_words(z), K, N)).cuda()
+    a = torch.full((M, K), value, dtype=torch.bfloat16, device="cuda")
+    y = _linear("gemv", 4, blob, a, K, N, 128)
+    want = (q[0].astype(np.float64) - z[0]) * 2.0 ** -6 * value * K
+    assert torch.equal(y, torch.from_numpy(want).to(torch.bfloat16).cuda().expand(M, N))
