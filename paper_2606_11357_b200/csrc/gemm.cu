@@ -35,6 +35,7 @@
 // Every mbarrier wait is bounded; on a timeout all roles leave, TMEM is freed, the status word is set.
 #include <cuda.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstddef>
 
@@ -101,15 +102,6 @@ constexpr int kGemmFlagOffset = 4096;          // zero between calls
 constexpr size_t kGemmPartialOffset = kWorkspaceZeroBytes;      // behind the GEMV's partial-sum slots, which must stay zero
 constexpr int kGemmMaxGrid = 160;
 static_assert(kGemmFlagOffset >= kGemvStatusBytes && kGemmFlagOffset + 4 * 4 * kGroups * kGemmMaxGrid <= kWorkspaceHeadBytes, "workspace layout shared with the GEMV");
-
-// 32-bit arithmetic: at most 256 x 16 x 256 units (N, K <= 32768, M <= 4096) times at most 161 CTAs stays below 2^28,
-// and these divisions sit between the start of a CTA and its first copy.
-__device__ __forceinline__ int unit_start(int cta, int total, int grid) {
-    return static_cast<int>((static_cast<uint32_t>(cta) * static_cast<uint32_t>(total)) / static_cast<uint32_t>(grid));
-}
-__device__ __forceinline__ int unit_owner(int unit, int total, int grid) {
-    return static_cast<int>(((static_cast<uint32_t>(unit) + 1u) * static_cast<uint32_t>(grid) - 1u) / static_cast<uint32_t>(total));
-}
 
 // The CTA's unit range [u_begin, u_end) as segments of one output tile each, in processing order: the last tile first.  A tile
 // that is cut between CTAs belongs to the CTA that has its last k-tile.  For that CTA it is the first tile of its range and comes
@@ -274,7 +266,7 @@ __device__ __forceinline__ uint32_t times_scale(uint32_t d, uint32_t hi2, uint32
 template <int BITS, int BT, int G = 1>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restrict__ blob,
-            __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int n_tiles, int m_tiles, int bt, int act_stages, int wp_stages, int aligned,
+            __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int n_tiles, int m_tiles, int bt, int act_stages, int wp_stages, int aligned, const Ranges ranges,
             uint8_t* __restrict__ workspace, uint32_t debug) {
     static_assert(G == 1 || BITS == 4, "several groups per tile: the 4-bit format only");
     constexpr int kTileBytes = tile_bytes(BITS, G);
@@ -297,11 +289,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
 
     // (the shuffle tells the compiler that the warp number is uniform in the warp)
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int total_units = n_tiles * m_tiles * ktiles;   // unit = (output tile, k-tile of 128)
-    // aligned: whole tiles only (no tile is shared between CTAs); otherwise the units are split evenly
-    const int total_tiles = n_tiles * m_tiles;
-    const int u_begin = aligned ? unit_start(blockIdx.x, total_tiles, gridDim.x) * ktiles : unit_start(blockIdx.x, total_units, gridDim.x);
-    const int u_end = aligned ? unit_start(blockIdx.x + 1, total_tiles, gridDim.x) * ktiles : unit_start(blockIdx.x + 1, total_units, gridDim.x);
+    // unit = (output tile, k-tile of 128); aligned: ranges of whole tiles (no tile is shared between CTAs)
+    // Several CTAs per tile: the grid has a row of CTAs per tile, which share its k-tiles.  Otherwise it has one row.
+    const int cta = blockIdx.y * gridDim.x + blockIdx.x;
+    const int u_begin = ranges.start(blockIdx.x) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
+    const int u_end = ranges.start(blockIdx.x + 1) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
     const Segments segs(u_begin, u_end, ktiles);
     const int strips = (N + kTileN - 1) / kTileN;
     const bool header_ok = header_matches(blob, BITS, (uint32_t)K, (uint32_t)N) && group_size_fits(blob, G);
@@ -483,11 +475,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                 if (!waited) { grid_dependency_wait(); waited = true; }        // y and the workspace belong to earlier kernels until now
                 if (dkt0 + dlen != ktiles) {
                     // the owner's warp of the same number takes what this one stores, so each pair has a flag of its own
-                    share.contribute(slots + blockIdx.x * kSlotVec, q);
+                    share.contribute(slots + cta * kSlotVec, q);
                     __syncwarp();
-                    if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + blockIdx.x * 4 * kGroups), "r"(1u) : "memory");
+                    if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + cta * 4 * kGroups), "r"(1u) : "memory");
                 } else if (dkt0 != 0) {
-                    const int first = unit_owner(dtile * ktiles, total_units, gridDim.x), others = blockIdx.x - first;
+                    const int first = gridDim.y > 1 ? dtile * gridDim.x : ranges.owner(dtile * ktiles), others = cta - first;
                     for (int o = 0; o < others; o += 32) {              // a lane per contributor
                         uint32_t* flag = flags + (first + o + lane) * 4 * kGroups;
                         const bool mine = o + lane < others;
@@ -613,7 +605,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
     __syncthreads();
     if (threadIdx.x == 0) {
         if (!header_ok) {
-            if (blockIdx.x == 0) { status->code = TF_ERR_BLOB; status->detail = 1; }
+            if (cta == 0) { status->code = TF_ERR_BLOB; status->detail = 1; }
         } else if (bars->abort_flag != 0) {
             status->code = TF_ERR_TIMEOUT;
             status->detail = bars->abort_flag;
@@ -641,15 +633,16 @@ size_t gemm_workspace_bytes(int M, int K, int N) {
 namespace {
 
 // How the work is spread over the CTAs.  Whole tiles only: nothing has to be put together, but the last wave of tiles may
-// leave SMs idle.  Even split of the (tile, k-tile) units over `grid` CTAs: the owner of a cut tile adds up the others' parts
-// at the end of its range.  The candidates are one CTA per SM and, where there are fewer tiles than SMs, every whole number of
-// CTAs per tile; the one with the smallest estimate is taken.  Measured (ns): a k-tile 450 + 1.5 bt (dequantization up to
+// leave SMs idle.  Split of the (tile, k-tile) units over `grid` CTAs: the owner of a cut tile adds up the others' parts
+// at the end of its range.  The candidates are one CTA per SM, in equal ranges, and, where there are fewer tiles than SMs, every whole
+// number of CTAs per tile; the one with the smallest estimate is taken.  Measured (ns): a k-tile 450 + 1.5 bt (dequantization up to
 // about 128 tokens, MMAs above); a cut 2000 (parts stored, flagged and seen) and 550 for every trip to the L2 that brings the
 // parts: two CTAs' at a time, 64 tokens at a time; 1000 less where a range is longer than two tiles, whose first part was
 // stored long before.
 struct GemmSplit {
-    int grid;
+    int grid, rows;            // CTAs; rows of the grid: one, or one per tile
     bool whole_tiles;
+    Ranges ranges;             // of whole tiles, or of units
 };
 GemmSplit split_gemm(int tiles, int ktiles, int bt, int sm_count) {
     const long long units = (long long)tiles * ktiles, t_unit = 450 + 3 * bt / 2;
@@ -664,6 +657,19 @@ GemmSplit split_gemm(int tiles, int ktiles, int bt, int sm_count) {
     };
     for (int per_tile = 2; per_tile * tiles <= sm_count && per_tile <= ktiles; ++per_tile) consider(per_tile * tiles, per_tile - 1);
     if (tiles % sm_count != 0 && units >= sm_count) consider(sm_count, (ktiles + units / sm_count - 1) / (units / sm_count));
+    // Up to 128 tokens, one CTA per SM: the last ten CTAs get what they are late by, 2 us, less (77x2944x11016 14.3 -> 14.1 us, 24x4096x14336
+    // 16.8 -> 16.3, 40x8192x8192 18.8 -> 18.6, 128 tokens no difference).  Wider tiles are long calls, and fewer SMs than CTAs leave
+    // nobody late.
+    constexpr int kLate = 10, kLateNs = 2000;
+    // Several CTAs per tile: the owner of the last k-tile takes as much more as its k-tiles last while the others' parts are on
+    // their way (us with even shares / this: 128x4096x4096 12.5 / 12.3, 60x4096x1024 8.25 / 8.05, int8 300x4096x4096 17.7 / 17.2).
+    constexpr int kOwnNs = 1900;
+    const int mean = (int)(units / sm_count);
+    const bool some_late = best.grid == sm_count && bt <= 128 && sm_count >= 8 * kLate;
+    best.rows = !best.whole_tiles && best.grid % tiles == 0 ? tiles : 1;
+    if (best.whole_tiles) best.ranges = Ranges::make(tiles, best.grid);
+    else if (best.rows > 1) best.ranges = Ranges::make(ktiles, best.grid / best.rows, 1, -(int)(kOwnNs / t_unit));
+    else best.ranges = Ranges::make((int)units, best.grid, some_late ? kLate : 0, std::min((int)(kLateNs / t_unit), mean / 2));
     return best;
 }
 
@@ -699,7 +705,7 @@ cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, in
     if (sm_count > kGemmMaxGrid) sm_count = kGemmMaxGrid;
     const GemmSplit split = split_gemm(n_tiles * m_tiles, K / kTileK, bt, sm_count);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(split.grid, 1, 1);
+    cfg.gridDim = dim3(split.grid / split.rows, split.rows, 1);
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
     cfg.dynamicSmemBytes = rings.smem_bytes;
     cfg.stream = stream;
@@ -710,7 +716,7 @@ cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, in
     cfg.numAttrs = 1;
     note_whole_sm_launch(stream);
     return cudaLaunchKernelEx(&cfg, gemm_kernel<BITS, BT, G>, map, static_cast<const uint8_t*>(blob), static_cast<__nv_bfloat16*>(y), M, K,
-                              N, K / kTileK, n_tiles, m_tiles, bt, rings.act_stages, rings.wp_stages, split.whole_tiles ? 1 : 0, static_cast<uint8_t*>(workspace), debug_word());
+                              N, K / kTileK, n_tiles, m_tiles, bt, rings.act_stages, rings.wp_stages, split.whole_tiles ? 1 : 0, split.ranges, static_cast<uint8_t*>(workspace), debug_word());
 }
 
 template <int BITS, int G = 1>

@@ -198,3 +198,26 @@ def test_cut_tiles_on_two_streams_at_once():
     for _, ws, y in lanes:
         assert tf.tf_device_status(ws) == 0
         assert np.array_equal(gu.bits_of(y), want)
+
+
+# how the work is cut: rows of CTAs per tile (two to seven, uneven shares, more CTAs than the owner's share has k-tiles), one CTA per SM with
+# shorter ranges for the last ones, whole tiles
+@pytest.mark.parametrize("bits,group", [(4, 128), (4, 64), (8, 128)])
+@pytest.mark.parametrize("M,K,N", [(24, 4096, 4096), (17, 896, 2560), (60, 4096, 1032), (128, 1280, 5120), (256, 2048, 2048), (40, 2944, 11016), (100, 640, 12000),
+                                   (32, 256, 2048), (130, 384, 18944)])
+def test_gemm_cuts(bits, group, M, K, N):
+    """Twice on one workspace: the same bits, its head left zero, and within the stated tolerance on sampled columns."""
+    p = wl.make_w4(M, K, N, group_size=group, seed=M + K + N) if bits == 4 else wl.make_w8(M, K, N, seed=M + K + N)
+    blob, a = torch.from_numpy(gu.pack(p)).cuda(), gu.to_device_bf16(p.a_bf16)
+    ws = torch.zeros(tf.tf_workspace_size(tf.TF_OP_GEMM_W4A16, M, K, N), dtype=torch.uint8, device="cuda")
+    ys = []
+    for _ in range(2):
+        y = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+        if group == 128:
+            getattr(tf, f"tf_gemm_w{bits}a16")(blob, a, y, M, K, N, ws)
+        else:
+            tf.tf_gemm_w4a16_grouped(blob, a, y, M, K, N, group, ws)
+        assert tf.tf_device_status(ws) == 0 and not bool(ws[:1069056].any())
+        ys.append(gu.bits_of(y))
+    assert np.array_equal(ys[0], ys[1])
+    gu.check_against_oracle(p, ys[0], columns=np.unique(np.concatenate([np.arange(0, N, 41), [N - 1]])))
