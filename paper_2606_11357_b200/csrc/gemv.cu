@@ -1120,35 +1120,31 @@ GemvPlan plan_gemv(int bits, int M, int K, int N, int sm_count, int groups) {
     return p;
 }
 
-// What this library launched last on a stream: whole-SM kernel or half-SM GEMV.  A scheduling hint only (see
-// launch_one): a stale, missing or raced entry costs overlap between kernels, never correctness.
+// What this library launched last on a stream.  A scheduling hint (see launch_one): a stale, missing or raced entry costs
+// overlap between kernels.
 namespace {
 constexpr int kLaunchNotes = 8;
 std::atomic<uintptr_t> g_note_stream[kLaunchNotes];
-std::atomic<int> g_note_whole_sm[kLaunchNotes];
+std::atomic<int> g_note_kind[kLaunchNotes];
 std::atomic<unsigned> g_note_next{0};
+uintptr_t note_key(cudaStream_t stream) { return reinterpret_cast<uintptr_t>(stream) + 1; }          // 0 = empty slot
+}  // namespace
 
-bool last_launch_was_half_sm(cudaStream_t stream) {
-    const uintptr_t key = reinterpret_cast<uintptr_t>(stream) + 1;          // 0 = empty slot
+LaunchKind last_launch(cudaStream_t stream) {
     for (int i = 0; i < kLaunchNotes; ++i)
-        if (g_note_stream[i].load(std::memory_order_relaxed) == key) return g_note_whole_sm[i].load(std::memory_order_relaxed) == 0;
-    return false;
+        if (g_note_stream[i].load(std::memory_order_relaxed) == note_key(stream)) return static_cast<LaunchKind>(g_note_kind[i].load(std::memory_order_relaxed));
+    return LaunchKind::kNone;
 }
-void note_launch(cudaStream_t stream, bool whole_sm) {
-    const uintptr_t key = reinterpret_cast<uintptr_t>(stream) + 1;
+void note_launch(cudaStream_t stream, LaunchKind kind) {
     for (int i = 0; i < kLaunchNotes; ++i)
-        if (g_note_stream[i].load(std::memory_order_relaxed) == key) {
-            g_note_whole_sm[i].store(whole_sm ? 1 : 0, std::memory_order_relaxed);
+        if (g_note_stream[i].load(std::memory_order_relaxed) == note_key(stream)) {
+            g_note_kind[i].store(static_cast<int>(kind), std::memory_order_relaxed);
             return;
         }
     const int slot = (int)(g_note_next.fetch_add(1, std::memory_order_relaxed) % kLaunchNotes);
-    g_note_whole_sm[slot].store(whole_sm ? 1 : 0, std::memory_order_relaxed);
-    g_note_stream[slot].store(key, std::memory_order_relaxed);
+    g_note_kind[slot].store(static_cast<int>(kind), std::memory_order_relaxed);
+    g_note_stream[slot].store(note_key(stream), std::memory_order_relaxed);
 }
-}  // namespace
-
-void note_whole_sm_launch(cudaStream_t stream) { note_launch(stream, true); }
-
 
 template <int BITS>
 static cudaError_t configure_bits() {
@@ -1190,15 +1186,16 @@ static cudaError_t launch_one(const GemvPlan& p, const void* blob, const void* a
     // with two CTAs each, 11 us lost per transition, until the next whole-SM kernel).  So a half-SM GEMV that does not
     // follow another half-SM GEMV of this library on its stream asks for a little more than half of an SM's shared
     // memory: two of its CTAs no longer fit on one SM, a CTA of the next (plain) half-SM GEMV still fits beside it.
-    if (!FULL && !last_launch_was_half_sm(stream) && cfg.dynamicSmemBytes < (size_t)kGemvSoloSmemBytes)
+    const int early = may_start_early(stream);
+    if (!FULL && last_launch(stream) != LaunchKind::kHalfSm && cfg.dynamicSmemBytes < (size_t)kGemvSoloSmemBytes)
         cfg.dynamicSmemBytes = kGemvSoloSmemBytes;
-    note_launch(stream, FULL);
+    note_launch(stream, FULL ? LaunchKind::kWholeSm : LaunchKind::kHalfSm);
     // Programmatic dependent launch: a CTA uses less than half of an SM (shared memory, registers), so the
     // CTAs of the next GEMV on the stream become resident while this one still runs, fill their rings with
     // weights and then wait for this kernel to finish before they touch activations, y or the workspace.
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = early;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (p.cluster > 1) {

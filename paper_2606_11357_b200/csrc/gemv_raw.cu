@@ -385,7 +385,7 @@ cudaError_t launch_gemv_raw(const RawGemvPlan& p, const uint32_t* qweight, const
                             const uint32_t* qzeros, const void* a, void* y, int M, int K, int N, int group_size,
                             void* workspace, cudaStream_t stream) {
     float* partial = static_cast<float*>(workspace);
-    note_whole_sm_launch(stream);   // not a half-SM GEMV: the next one must not assume it follows one
+    note_launch(stream, LaunchKind::kWholeSm);   // not a half-SM GEMV: the next one must not assume it follows one
     cudaError_t e;
     if (p.mma) {
         dim3 grid(p.col_blocks, p.splits, 1);

@@ -152,8 +152,13 @@ cudaError_t configure_gemv_kernels();
 uint32_t debug_word();
 void set_debug_word(uint32_t word);
 
-// Tell the GEMV launcher that a whole-SM kernel of this library (the GEMM) was launched on `stream`.
-void note_whole_sm_launch(cudaStream_t stream);
+// What this library launched last on a stream (the last eight streams are kept; a scheduling hint, see launch_one in gemv.cu).
+enum class LaunchKind : int { kNone = 0, kHalfSm, kWholeSm, kRepack };
+void note_launch(cudaStream_t stream, LaunchKind kind);
+LaunchKind last_launch(cudaStream_t stream);
+// GEMV and GEMM read packed weights before they wait for the kernels ahead of them.  Straight behind the kernel that packs, they
+// are launched as ordinary kernels, so that its stores are done.
+inline int may_start_early(cudaStream_t stream) { return last_launch(stream) == LaunchKind::kRepack ? 0 : 1; }
 
 cudaError_t launch_unpack_w4(const void* blob, uint8_t* q, uint8_t* z, uint16_t* s, int K, int N,
                              int group_size, cudaStream_t stream);

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/tilefuse.h"
+#include "async.cuh"
 #include "kernels.h"
 #include "layout.h"
 
@@ -28,20 +29,22 @@ __device__ __forceinline__ void transpose_bytes(uint32_t r0, uint32_t r1, uint32
     out[3] = __byte_perm(c, d, 0x7632);
 }
 
-// A CTA re-tiles two neighbouring tiles (128 k x 128 n).  Thread (kb, t, strip, w) moves the 8 x 8 nibble block of rows
-// 16 kb + 4t .. +3 and words 2w, 2w + 1 of its strip: it reads 4 x 8 bytes, transposes them in registers and writes
-// one word of each of the eight lanes (g, t).  A warp reads four 64-byte row segments per load and writes 64-byte runs per
-// store, so every sector is moved once.  Bound by DRAM; the form before it, one thread per output word, made eight 4-byte loads
-// for each (most of them the same words, from the L1) and was bound by them: 4096 x 14336 took 65.6 us (0.9 TB/s),
-// now 11.3 us (5.4 TB/s).
-constexpr int kRepackThreads = 256;
+// A CTA re-tiles four neighbouring tiles (128 k x 256 n).  A thread moves two 8 x 8 nibble blocks, of rows 16 kb + 4t .. +3 (t and t + 2)
+// and words 2w, 2w + 1 of its strip: it reads 8 x 8 bytes, transposes them in registers and writes one word of each of the
+// eight lanes (g, t).  A warp reads 128-byte row segments, so every sector is moved once.  Bound by DRAM: 4096 x 14336 takes 11.4 us
+// in a chain (5.3 TB/s).  Launched as a programmatic dependent, whose CTAs wait for the kernels before it themselves: with a plain
+// launch it was 13.8 us, 1024 x 4096 4.1 (now 2.7).  (Two tiles per CTA: 1 % slower.  One thread per output word, eight 4-byte loads
+// for each: 65.6 us.)  It releases its own dependents only by ending: the GEMV and the GEMM read packed weights before they wait for
+// the kernels ahead of them.
+constexpr int kRepackThreads = 256, kRepackStrips = 4;
 template <bool kPairs, int G>      // G: groups per tile; kPairs: rows are a whole number of word pairs, so a thread's two words are one 8-byte load
 __global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32_t* __restrict__ qweight, const uint16_t* __restrict__ scales,
                                                                     const uint32_t* __restrict__ qzeros, uint8_t* __restrict__ out, int K, int N,
                                                                     int group_size, int ktiles, int strips) {
     constexpr int tile_bytes_here = w4_tile_bytes(G);
-    const int T = blockIdx.y, S0 = 2 * blockIdx.x;
+    const int T = blockIdx.y, S0 = kRepackStrips * blockIdx.x;
     const int row_words = N >> 3;
+    grid_dependency_wait();                  // the arrays may come from earlier kernels, and they may still read what `out` held
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         tf_blob_header h = {};
         h.magic = kMagic; h.version = kBlobVersion; h.bits = 4; h.K = (uint32_t)K; h.N = (uint32_t)N;
@@ -55,13 +58,13 @@ __global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32
     // ---- metadata: per strip and group 32 words of scale pairs and 8 of zero points ----------------------------------
     // The loads first, so that they are on their way together with those of the weights; the words are put together and
     // stored at the end.  A scale word takes two values, a zero word eight.
-    constexpr int kMetaWords = G * (kScaleBytes + kZeroBytes) / 4, kItems = (2 * kMetaWords + kRepackThreads - 1) / kRepackThreads;
+    constexpr int kMetaWords = G * (kScaleBytes + kZeroBytes) / 4, kItems = (kRepackStrips * kMetaWords + kRepackThreads - 1) / kRepackThreads;
     uint32_t meta[kItems][8];
 #pragma unroll
     for (int it = 0; it < kItems; ++it) {
         const int i = threadIdx.x + it * kRepackThreads;
-        const int S = S0 + (i >= kMetaWords), wi = i >= kMetaWords ? i - kMetaWords : i;
-        if (i >= 2 * kMetaWords || S >= strips) continue;
+        const int S = S0 + i / kMetaWords, wi = i % kMetaWords;
+        if (i >= kRepackStrips * kMetaWords || S >= strips) continue;
         const int n0 = S * kTileN;
         if (wi < G * (kScaleBytes / 4)) {                             // [group][g][w] -> (2w, 2w + 1) = columns +0, +8
             const int gr = wi / (kScaleBytes / 4), rest = wi % (kScaleBytes / 4);
@@ -81,45 +84,53 @@ __global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32
     }
     // ---- weights -----------------------------------------------------------------------------------------------
     {
-        const int w = threadIdx.x & 3, S = S0 + ((threadIdx.x >> 2) & 1), t = (threadIdx.x >> 3) & 3, kb = threadIdx.x >> 5;
+        const int w = threadIdx.x & 3, S = S0 + ((threadIdx.x >> 2) & 3), kb = threadIdx.x >> 5;
         if (S < strips) {
             const int word0 = S * (kTileN / 8) + 2 * w;
-            const uint32_t* src = qweight + (size_t)(T * kTileK + 16 * kb + 4 * t) * row_words + word0;
-            uint32_t even[4], odd[4];                                    // padded columns: q = z = 0, s = 0
+            uint32_t even[2][4], odd[2][4];                              // padded columns: q = z = 0, s = 0
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                even[r] = odd[r] = 0u;
-                if (kPairs) {
-                    if (word0 < row_words) {
-                        const uint2 v = __ldcs(reinterpret_cast<const uint2*>(src + (size_t)r * row_words));
-                        even[r] = v.x; odd[r] = v.y;
+            for (int it = 0; it < 2; ++it) {
+                const int t = ((threadIdx.x >> 4) & 1) + 2 * it;
+                const uint32_t* src = qweight + (size_t)(T * kTileK + 16 * kb + 4 * t) * row_words + word0;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    even[it][r] = odd[it][r] = 0u;
+                    if (kPairs) {
+                        if (word0 < row_words) {
+                            const uint2 v = __ldcs(reinterpret_cast<const uint2*>(src + (size_t)r * row_words));
+                            even[it][r] = v.x; odd[it][r] = v.y;
+                        }
+                    } else {
+                        if (word0 < row_words) even[it][r] = __ldg(src + (size_t)r * row_words);
+                        if (word0 + 1 < row_words) odd[it][r] = __ldg(src + (size_t)r * row_words + 1);
                     }
-                } else {
-                    if (word0 < row_words) even[r] = __ldg(src + (size_t)r * row_words);
-                    if (word0 + 1 < row_words) odd[r] = __ldg(src + (size_t)r * row_words + 1);
                 }
             }
             // low and high nibbles of byte b: columns {0, 4, 1, 5}[b] and {2, 6, 3, 7}[b]; a lane's word takes rows
             // 0, 2, 1, 3 in its bytes, the even word's code in the low nibble, the odd word's in the high one
-            uint32_t lo[4], hi[4], a[4], b[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                lo[r] = select_bits(even[r], odd[r] << 4, 0x0F0F0F0Fu);
-                hi[r] = select_bits(even[r] >> 4, odd[r], 0x0F0F0F0Fu);
+            for (int it = 0; it < 2; ++it) {
+                const int t = ((threadIdx.x >> 4) & 1) + 2 * it;
+                uint32_t lo[4], hi[4], a[4], b[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    lo[r] = select_bits(even[it][r], odd[it][r] << 4, 0x0F0F0F0Fu);
+                    hi[r] = select_bits(even[it][r] >> 4, odd[it][r], 0x0F0F0F0Fu);
+                }
+                transpose_bytes(lo[0], lo[2], lo[1], lo[3], a);
+                transpose_bytes(hi[0], hi[2], hi[1], hi[3], b);
+                uint32_t* dst = reinterpret_cast<uint32_t*>(tile_of(S)) + (kb * 32 + t) * 4 + w;      // lane (g, t): 16 g words further
+                dst[0] = a[0]; dst[4 * 16] = a[1]; dst[16] = a[2]; dst[5 * 16] = a[3];
+                dst[2 * 16] = b[0]; dst[6 * 16] = b[1]; dst[3 * 16] = b[2]; dst[7 * 16] = b[3];
             }
-            transpose_bytes(lo[0], lo[2], lo[1], lo[3], a);
-            transpose_bytes(hi[0], hi[2], hi[1], hi[3], b);
-            uint32_t* dst = reinterpret_cast<uint32_t*>(tile_of(S)) + (kb * 32 + t) * 4 + w;      // lane (g, t): 16 g words further
-            dst[0] = a[0]; dst[4 * 16] = a[1]; dst[16] = a[2]; dst[5 * 16] = a[3];
-            dst[2 * 16] = b[0]; dst[6 * 16] = b[1]; dst[3 * 16] = b[2]; dst[7 * 16] = b[3];
         }
     }
     // ---- metadata, stored --------------------------------------------------------------------------------------------
 #pragma unroll
     for (int it = 0; it < kItems; ++it) {
         const int i = threadIdx.x + it * kRepackThreads;
-        const int S = S0 + (i >= kMetaWords), wi = i >= kMetaWords ? i - kMetaWords : i;
-        if (i >= 2 * kMetaWords || S >= strips) continue;
+        const int S = S0 + i / kMetaWords, wi = i % kMetaWords;
+        if (i >= kRepackStrips * kMetaWords || S >= strips) continue;
         uint32_t word = 0;
         if (wi < G * (kScaleBytes / 4)) {
             word = meta[it][0] | (meta[it][1] << 16);
@@ -137,12 +148,21 @@ __global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32
 cudaError_t launch_repack_awq(const uint32_t* qweight, const uint16_t* scales, const uint32_t* qzeros, void* out, int K, int N,
                               int group_size, cudaStream_t stream) {
     const int strips = (N + kTileN - 1) / kTileN, ktiles = K / kTileK;
-    const dim3 grid((strips + 1) / 2, ktiles);
+    const dim3 grid((strips + kRepackStrips - 1) / kRepackStrips, ktiles);
     const int G = groups_per_tile(group_size);
     auto* kernel = (N / 8) % 2 == 0 ? (G == 1 ? repack_awq_kernel<true, 1> : G == 2 ? repack_awq_kernel<true, 2> : repack_awq_kernel<true, 4>)
                                     : (G == 1 ? repack_awq_kernel<false, 1> : G == 2 ? repack_awq_kernel<false, 2> : repack_awq_kernel<false, 4>);
-    kernel<<<grid, kRepackThreads, 0, stream>>>(qweight, scales, qzeros, static_cast<uint8_t*>(out), K, N, group_size, ktiles, strips);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kRepackThreads, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    note_launch(stream, LaunchKind::kRepack);
+    return cudaLaunchKernelEx(&cfg, kernel, qweight, scales, qzeros, static_cast<uint8_t*>(out), K, N, group_size, ktiles, strips);
 }
 
 }  // namespace tf

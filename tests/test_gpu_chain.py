@@ -138,3 +138,39 @@ def test_w8_integer_path_chain():
         o1, o2 = gu.bits_of(y1), gu.bits_of(y2)
         gu.check_against_oracle(p1, o1)
         gu.check_against_oracle(with_activations(p2, o1), o2)
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("kind,M,K,N", [("gemv", 1, 1024, 4096), ("gemv", 4, 2048, 1032), ("gemm", 40, 1024, 4096)])
+def test_packing_between_calls(kind, M, K, N, captured):
+    """The device packer rewrites one blob between calls that read it, with nothing but the stream to order them, and reads arrays that
+    a copy just ahead of it has put there: every result is that of its own weights."""
+    problems = [wl.make_w4(M, K, N, seed=60 + i) for i in range(3)]
+    sources = [[torch.from_numpy(p.qweight.view(np.int32)).cuda(), torch.from_numpy(p.scales_f16).cuda(), torch.from_numpy(p.qzeros.view(np.int32)).cuda()] for p in problems]
+    a = [gu.to_device_bf16(p.a_bf16) for p in problems]
+    arrays = [torch.empty_like(t) for t in sources[0]]
+    blob = torch.zeros(tf.tf_packed_size(4, K, N, 128), dtype=torch.uint8, device="cuda")
+    ys = [torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in problems]
+    ws = torch.zeros(tf.tf_workspace_size(tf.TF_OP_GEMV_W4A16 if kind == "gemv" else tf.TF_OP_GEMM_W4A16, M, K, N), dtype=torch.uint8, device="cuda")
+    call = tf.tf_gemv_w4a16 if kind == "gemv" else tf.tf_gemm_w4a16
+
+    def chain():
+        for i in range(len(problems)):
+            for dst, src in zip(arrays, sources[i]):
+                dst.copy_(src)
+            tf.tf_pack_awq_device(*arrays, K, N, 128, blob)
+            for _ in range(2):
+                call(blob, a[i], ys[i], M, K, N, ws)
+
+    chain()
+    if captured:
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            chain()
+        for y in ys:
+            y.fill_(float("nan"))
+        graph.replay()
+    assert tf.tf_device_status(ws) == 0
+    for p, y in zip(problems, ys):
+        gu.check_against_oracle(p, gu.bits_of(y))
