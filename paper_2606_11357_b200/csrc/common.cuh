@@ -71,22 +71,33 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// Header fields every kernel compares with its arguments (first 24 bytes of the blob).
+// Header fields that kernels compare with its arguments (first 24 bytes of the blob).
 __device__ __forceinline__ bool header_matches(const void* blob, uint32_t bits, uint32_t K, uint32_t N) {
     const uint4 h = __ldg(reinterpret_cast<const uint4*>(blob));            // magic, version, bits, K
     const uint2 h2 = __ldg(reinterpret_cast<const uint2*>(blob) + 2);       // N, group_size
     return h.x == kMagic && h.y == kBlobVersion && h.z == bits && h.w == K && h2.x == N;
 }
 
-// The group size recorded in the header, and whether it fits a kernel built for G groups per tile (G = 1: any
-// multiple of the tile's k-extent; G = 2, 4: exactly 128 / G).
+// The group size recorded in the header.
 __device__ __forceinline__ uint32_t header_group_size(const void* blob) {
     return __ldg(reinterpret_cast<const uint32_t*>(blob) + 5);
 }
-__device__ __forceinline__ bool group_size_fits(const void* blob, int G) {
-    const uint32_t gs = header_group_size(blob);
-    return G == 1 ? (gs >= (uint32_t)kTileK && gs % kTileK == 0) : gs == (uint32_t)(kTileK / G);
-}
+// The same in two steps, for a kernel that has something to do while the header is on its way: the words are asked for at its start
+// and judged where the answer is needed (GEMV, floating-point path, a chain of whole-SM kernels, where the set-up of the last CTAs is on
+// the call's way: 4 tokens 4096x6144 5.76 -> 5.56 us, 14336x4096 8.77 -> 8.56, 16 tokens 4096x28672 18.7 -> 18.5).  With the group size, which has to fit a kernel built for G groups per tile (G = 1: any
+// multiple of the tile's k-extent; G = 2, 4: exactly 128 / G).
+struct HeaderWords {
+    uint4 a;            // magic, version, bits, K
+    uint2 b;            // N, group size
+    __device__ __forceinline__ explicit HeaderWords(const void* blob)
+        : a(__ldg(reinterpret_cast<const uint4*>(blob))), b(__ldg(reinterpret_cast<const uint2*>(blob) + 2)) {}
+    // (the empty statement keeps the compiler from judging once, ahead of everything: the wait for the words would be there too)
+    __device__ __forceinline__ bool fit(uint32_t bits, uint32_t K, uint32_t N, int G) {
+        asm volatile("" : "+r"(a.x), "+r"(a.y), "+r"(a.z), "+r"(a.w), "+r"(b.x), "+r"(b.y));
+        return a.x == kMagic && a.y == kBlobVersion && a.z == bits && a.w == K && b.x == N &&
+               (G == 1 ? (b.y >= (uint32_t)kTileK && b.y % kTileK == 0) : b.y == (uint32_t)(kTileK / G));
+    }
+};
 
 __device__ __forceinline__ float fp16_bits_to_float(uint16_t h) {
     return __half2float(__ushort_as_half(h));

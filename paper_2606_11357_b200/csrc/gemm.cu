@@ -296,7 +296,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
     const int u_end = ranges.start(blockIdx.x + 1) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
     const Segments segs(u_begin, u_end, ktiles);
     const int strips = (N + kTileN - 1) / kTileN;
-    const bool header_ok = header_matches(blob, BITS, (uint32_t)K, (uint32_t)N) && group_size_fits(blob, G);
+    HeaderWords header(blob);
     DeviceStatus* status = reinterpret_cast<DeviceStatus*>(workspace);
     float4* slots = reinterpret_cast<float4*>(workspace + kGemmPartialOffset);
 
@@ -342,7 +342,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
             mbar_init(smem_u32(&bars->wp_empty[s]), 4 * kChunk);      // the groups of the chunk
         }
         mbar_init_fence();
-        if (header_ok && !drop_weights) produce_weights(0, early_chunks);
+        if (header.fit(BITS, (uint32_t)K, (uint32_t)N, G) && !drop_weights) produce_weights(0, early_chunks);
     } else if (threadIdx.x >= 32 && threadIdx.x < 32 + kGroups) {
         mbar_init(smem_u32(&bars->op_full[threadIdx.x - 32]), kTied ? 5 : 4);
         mbar_init(smem_u32(&bars->op_done[threadIdx.x - 32]), 1);
@@ -363,6 +363,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    const bool header_ok = header.fit(BITS, (uint32_t)K, (uint32_t)N, G);
     // The next kernel of the stream may start as SMs become free: its set-up and its first weights then run under the last
     // CTAs of this one (released at the end of the kernel instead, a short GEMM took 1 to 2 us longer in a chain).
     grid_launch_dependents();

@@ -307,7 +307,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     DeviceStatus* status = reinterpret_cast<DeviceStatus*>(workspace);
     float* partials = reinterpret_cast<float*>(workspace + kGemvPartialOffset);
 
-    const bool header_ok = header_matches(blob, BITS, (uint32_t)K, (uint32_t)N) && group_size_fits(blob, G);
+    HeaderWords header(blob);
 
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kGemvMaxStages);
     const uint32_t seg_full0 = smem_u32(bars + 2 * kGemvMaxStages), seg_free0 = seg_full0 + 16;
@@ -331,7 +331,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
             stage_tag[s] = 0xFFFFFFFFu;
         }
         mbar_init_fence();
-        if (header_ok && (debug & kDebugDropWeights) == 0 && !early.done()) issue_weights(early, issued++);
+        if (header.fit(BITS, (uint32_t)K, (uint32_t)N, G) && (debug & kDebugDropWeights) == 0 && !early.done()) issue_weights(early, issued++);
     }
     // One thread per ring stage, one more for the rest: the set-up sits between the start of a CTA and its first
     // weight copy (one thread doing all of it in turn cost the decode step 1.7 us).
@@ -351,6 +351,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
         mbar_init_fence();
     }
     __syncthreads();
+    const bool header_ok = header.fit(BITS, (uint32_t)K, (uint32_t)N, G);
     // Programmatic dependent launch: the next kernel on the stream may start as SMs free up.  In this kernel
     // only the packed weights (constants) are read before grid_dependency_wait(): the producer lane waits before it copies activations,
     // every consumer warp waits before its first activation load, the reducer warp before it touches y or the
