@@ -980,12 +980,12 @@ static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool f
     // 18.1 whole SM with 8 / 12 / 16 warps; 4096x14336 int8 15.8 us half SM, 12.7 / 13.3 / 14.6 whole SM with 8 / 12 / 16.
     p.consumers = p.i8 && p.full ? gemv_i8_full_consumers(bits) : gemv_max_consumers(mt, p.full);
     // Floating-point path up to 8 tokens: 12 warps only for long ranges of 4-bit tiles.  Eight have fewer partial sums to add up
-    // at the end of a strip and less of the ring in their hands: 4 tokens 4096x4096 5.29 us against 5.59 with 12, x6144 6.82 and
-    // 7.04, x8192 7.55 either way, then x9472 7.37 and 7.33, x14336 9.81 and 9.94, x28672 16.39 and 15.81; int8 8 tokens 4096x4096
-    // 6.42 and 6.71, x9472 9.76 and 10.21, x28672 22.1 and 23.1.  (10, 11 and 14 warps are slower than 8, 12 and 16 everywhere, 14336x4096 11.1 us
-    // against 10.6: with a multiple of the tiles of a chunk a warp always works on the same place of a stage, and a stage is
-    // freed by warps that are about equally far.)
-    if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < kGemvFpTwelveWarpsFromTiles)) p.consumers = 8;
+    // at the end of a strip and less of the ring in their hands: us with 8 / 12, 4 tokens 14336x4096 (49 tiles) 8.35 / 8.53, 4096x14336 8.78
+    // either way, a decoder layer 33.7 / 34.0; 4096x28672 (97 tiles) 16.4 / 15.8 and int8, 8 tokens, 22.1 / 23.1 in an earlier form.  With
+    // four groups per tile, whose scales are more work, 5 tokens 4096x14336 9.85 / 9.62.  (10, 11 and 14 warps are slower than 8, 12 and
+    // 16 everywhere, 14336x4096 11.1 us against 10.6: with a multiple of the tiles of a chunk a warp always works on the same place of
+    // a stage, and a stage is freed by warps that are about equally far.)
+    if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < (p.groups == 1 ? kGemvFpTwelveWarpsFromTiles : kGemvFpTwelveWarpsFromTilesGrouped))) p.consumers = 8;
     if (tiles_per_cta < p.consumers) p.consumers = tiles_per_cta < 4 ? 4 : tiles_per_cta;
     p.threads = 32 * (p.consumers + 2);          // + producer warp + reducer warp
     const int kr = gemv_chunk_tiles(bits);
@@ -1008,12 +1008,13 @@ static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool f
     // whole-SM integer path: a ring deeper than eight stages was slower (1x4096x32768 4-bit: 17.0 / 16.9 / 17.5 us with
     // 6 / 8 / 10 stages; int8 1x4096x14336: 12.8 / 12.5 / 12.7 us with 6 / 8 / 11)
     if (p.i8 && p.full && stages > kGemvI8FullMaxStages) stages = kGemvI8FullMaxStages;
-    // floating-point path up to 8 tokens on 4-bit tiles: five stages (two in the hands of 8 consumer warps, three in those of 12, the
-    // others in flight).  Measured, with 12 warps, at 4 tokens with 4 / 5 / 6 / 7 / 9 stages: 4096x14336 12.2 / 11.6 / 11.7 / 11.9 / 12.3 us,
-    // 4096x32768 20.9 / 19.8 / 19.9 / 20.1 / 20.5 us; int8 tiles (four or six stages in the warps' hands) want the deep ring:
-    // 4096x14336 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us.  (Why a deeper ring is slower on 4-bit tiles was not established;
-    // the consumers, not HBM, set the pace of this path.)
-    if (!p.i8 && mt == 1 && bits == 4 && stages > kGemvFpW4MaxStages) stages = kGemvFpW4MaxStages;
+    // floating-point path up to 8 tokens on 4-bit tiles: five stages with 8 consumer warps (two in their hands), six with 12 (three).
+    // us with 5 / 6 / 7 stages: 8 warps, 4 tokens 4096x6144 5.57 / 5.71 / 5.71, 14336x4096 8.35 / - / 9.01; 12 warps 4096x28672 14.25 / 14.07 /
+    // 14.07, 6 tokens, group 64, 7424x18440 16.4 / 16.1 / 16.2, four groups per tile 5 tokens 4096x14336 9.58 / 9.77.  int8 tiles (four or six
+    // stages in the warps' hands) want the deep ring: 4096x14336 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us with 4 / 5 / 6 / 7 / 9 in an earlier form.
+    // (Why a deeper ring is slower on 4-bit tiles was not established.)
+    const int most = p.consumers > 8 && p.groups < 4 ? kGemvFpW4MaxStages12 : kGemvFpW4MaxStages8;
+    if (!p.i8 && mt == 1 && bits == 4 && stages > most) stages = most;
     // Integer path: where a range passes over the same k-tiles more than once and K is a multiple of 128 x consumer
     // warps, every warp meets the same k-tiles on each pass and keeps the activation pieces it has prepared (one table
     // entry per k-tile instead of one scratch entry per warp), if that costs the ring no stage.

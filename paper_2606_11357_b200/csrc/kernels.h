@@ -10,7 +10,7 @@ namespace tf {
 #define TF_I8_FULL_BYTES_W4 (288 * 1024)
 #endif
 #ifndef TF_I8_FULL_BYTES_W8
-#define TF_I8_FULL_BYTES_W8 (160 * 1024)
+#define TF_I8_FULL_BYTES_W8 (96 * 1024)
 #endif
 
 // ---- GEMV (persistent streaming kernel) ----------------------------------------------------------
@@ -48,6 +48,8 @@ constexpr int kGemvPieceEntryBytes = 512;
 // eight stages; with about 66 KB of tiles in the warps' hands (8 warps on int8, 16 on 4-bit tiles) it streams long
 // ranges faster than the half-SM form, which wins on short ranges because the next GEMV's CTAs sit beside it with
 // their rings full.
+// int8, one token, us half SM / whole SM: 1024x8192 (67 KB) 2.41 / 3.13, 2048x4096 3.20 / 3.46, then 14336x1024 (119 KB) 5.99 / 4.82, 4096x3072
+// (133 KB) 5.33 / 4.08, 4096x4096 5.47 / 4.66, 2048x11008 6.30 / 5.60; two tokens 4096x4096 5.55 / 4.90.
 constexpr int kGemvFullFromBytesI8W4 = TF_I8_FULL_BYTES_W4;
 constexpr int kGemvFullFromBytesI8W8 = TF_I8_FULL_BYTES_W8;
 // 4-bit tiles, the half-SM form without / with its activation pieces kept (piece table).  Figures: us per call in a chain of one
@@ -63,8 +65,8 @@ constexpr int kGemvFullFromBytesI8W8 = TF_I8_FULL_BYTES_W8;
 // it 4096x20480 11.89 / 11.33, 3072x26624 11.90 / 11.25).
 constexpr int kGemvFullFromBytesI8W4Kept = 448 * 1024;
 constexpr int kGemvI8FullMaxStages = 8;
-constexpr int kGemvFpW4MaxStages = 5;
-constexpr int kGemvFpTwelveWarpsFromTiles = 32;
+constexpr int kGemvFpW4MaxStages8 = 5, kGemvFpW4MaxStages12 = 6;                              // with 8 and with 12 consumer warps (four groups per tile: 5)
+constexpr int kGemvFpTwelveWarpsFromTiles = 60, kGemvFpTwelveWarpsFromTilesGrouped = 32;      // one group per tile; two or four
 constexpr int kGemvMaxDevices = 64;            // devices the per-device caches cover
 constexpr int kGemvMaxStages = 48;
 constexpr int kGemvBarrierBytes = 4096;       // 2 x 48 mbarriers + flags, then the chunk tags of the stages
