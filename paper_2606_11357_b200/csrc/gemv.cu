@@ -76,12 +76,11 @@ __device__ __forceinline__ void mma_u8s8_16832_first(int d[4], uint32_t a0, uint
 }
 
 // int -> float for |v| < 2^22 without the conversion unit: the bits of the integer 0x4B400000 + v are the float
-// 1.5 * 2^23 + v, exactly.  The integer MMAs start their accumulators at kIntAsFloatBias, so a tile's sums come out of
-// the tensor pipe already in that form, and (f - 1.5 * 2^23) * c is one fused multiply-add with -1.5 * 2^23 * c.
+// 1.5 * 2^23 + v, exactly.  A tile's sums get the bias as the start of the MMAs' accumulators or with the zero point, and (f - 1.5 * 2^23) * c is one fused multiply-add with -1.5 * 2^23 * c.
 constexpr int kIntAsFloatBias = 0x4B400000;
 constexpr float kIntAsFloatBiasValue = 12582912.0f;
 
-// Even split of `total` tiles over `grid` CTAs.  32-bit: the products stay below 2^26 (at most 256 x 512 tiles, K and N <= 32768,
+// Even split of `total` tiles (or strips) over the CTAs of a cluster (or the clusters); the grid's own ranges come with the launch.  32-bit: the products stay below 2^26 (at most 256 x 512 tiles, K and N <= 32768,
 // times at most 257), and a 64-bit division is several times the instructions.  These sit between the start of a CTA and its
 // first weight copy, in the reducer's bookkeeping and in the cluster-mode finish.
 __device__ __forceinline__ int range_start(int cta, int total, int grid) {

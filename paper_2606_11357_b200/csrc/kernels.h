@@ -23,8 +23,8 @@ namespace tf {
 //     consumer warps, a warp keeps the activation pieces of the k-tiles it has visited (piece table) instead of
 //     preparing them per tile.
 //   floating-point path up to 8 tokens: the whole SM and 8 consumer warps, 12 for long ranges of 4-bit tiles; on 4-bit tiles
-//     a ring of five stages (two or three in the warps' hands; deeper was measured slower), on int8 tiles the deepest that fits.
-//     A consumer warp of this path needs about 20 issue cycles per packed word of 8 weights (measured on registers alone), and
+//     a ring of five or six stages (two or three in the warps' hands; deeper was measured slower), on int8 tiles the deepest that fits.
+//     A consumer warp of this path executes 460 instructions per tile (4 tokens), and
 //     since a GEMV may not read its activations before the kernel ahead of it has completed, only one kernel's consumers
 //     work on an SM at a time: room for a waiting neighbour is worth less than a deep ring and, on long ranges, a third
 //     warp per scheduler.
