@@ -11,8 +11,10 @@
  *   - "host" / "device" on a pointer says which memory it must point into.
  *   - The caller owns every buffer.  The library allocates nothing, frees nothing and
  *     keeps no pointer after a call returns.
- *     (It remembers, per process, which kind of kernel it launched last on a stream; that
- *     only steers how consecutive kernels overlap.)
+ *     (It remembers, per process, which kind of kernel it launched last on each of the last 32
+ *     streams.  A GEMV or GEMM may start before the kernel ahead of it on the stream has ended only
+ *     where one is remembered since the last tf_pack_awq_device there; a stream that is not
+ *     remembered gets an ordinary launch.)
  *   - Device calls are asynchronous on `cuda_stream` (a cudaStream_t passed as void*;
  *     NULL = the default stream) and never synchronise, except tf_device_status.
  *   - Errors are return codes.  Nothing is printed, nothing aborts, no exception
@@ -24,8 +26,8 @@
  *     10.x gives TF_ERR_ARCH.
  *   - Thread safety: every entry point may be called from several host threads at once.  The
  *     library's only state is per-device caches of immutable facts (device attributes, "this
- *     kernel's attributes are set", occupancy answers) and the per-stream note above, all held
- *     in atomics; a race on first use repeats an idempotent query.  The caller keeps calls that
+ *     kernel's attributes are set", occupancy answers), held in atomics -- a race on first use
+ *     repeats an idempotent query -- and the per-stream notes above, held under a lock.  The caller keeps calls that
  *     share a workspace (or the fixed scratch of tf_gemv_w4a16_static) from overlapping on the
  *     GPU, and makes the CUDA device current on the calling thread.
  */

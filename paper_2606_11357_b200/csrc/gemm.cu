@@ -713,12 +713,15 @@ cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, in
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see grid_dependency_wait() in the kernel
-    attr[0].val.programmaticStreamSerializationAllowed = may_start_early(stream);
+    const StreamNote note(stream);
+    attr[0].val.programmaticStreamSerializationAllowed = note.may_start_early() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    note_launch(stream, LaunchKind::kWholeSm);
-    return cudaLaunchKernelEx(&cfg, gemm_kernel<BITS, BT, G>, map, static_cast<const uint8_t*>(blob), static_cast<__nv_bfloat16*>(y), M, K,
-                              N, K / kTileK, n_tiles, m_tiles, bt, rings.act_stages, rings.wp_stages, split.whole_tiles ? 1 : 0, split.ranges, static_cast<uint8_t*>(workspace), debug_word());
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_kernel<BITS, BT, G>, map, static_cast<const uint8_t*>(blob), static_cast<__nv_bfloat16*>(y),
+                                             M, K, N, K / kTileK, n_tiles, m_tiles, bt, rings.act_stages, rings.wp_stages,
+                                             split.whole_tiles ? 1 : 0, split.ranges, static_cast<uint8_t*>(workspace), debug_word());
+    if (e == cudaSuccess) note.launched(LaunchKind::kWholeSm);
+    return e;
 }
 
 template <int BITS, int G = 1>

@@ -1121,31 +1121,31 @@ GemvPlan plan_gemv(int bits, int M, int K, int N, int sm_count, int groups) {
     return p;
 }
 
-// What this library launched last on a stream.  A scheduling hint (see launch_one): a stale, missing or raced entry costs
-// overlap between kernels.
-namespace {
-constexpr int kLaunchNotes = 8;
-std::atomic<uintptr_t> g_note_stream[kLaunchNotes];
-std::atomic<int> g_note_kind[kLaunchNotes];
-std::atomic<unsigned> g_note_next{0};
-uintptr_t note_key(cudaStream_t stream) { return reinterpret_cast<uintptr_t>(stream) + 1; }          // 0 = empty slot
-}  // namespace
+static LaunchNotes g_notes;
 
-LaunchKind last_launch(cudaStream_t stream) {
-    for (int i = 0; i < kLaunchNotes; ++i)
-        if (g_note_stream[i].load(std::memory_order_relaxed) == note_key(stream)) return static_cast<LaunchKind>(g_note_kind[i].load(std::memory_order_relaxed));
-    return LaunchKind::kNone;
+// The runtime's number of a stream may not be asked for while the stream is capturing (it ends the capture with an error); there the handle names
+// it, but for cudaStreamPerThread, which is one handle for many.  The stream's place in the graph has to be a single node as well: with
+// several, some are other streams' work.  (Both questions and the notes' lock are 0.11 us of host time per call.)
+StreamNote::StreamNote(cudaStream_t stream) : name{0, 0, false}, seen{LaunchKind::kNone, 0} {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long capture = 0;
+    const cudaGraphNode_t* nodes = nullptr;
+    const cudaGraphEdgeData* edges = nullptr;
+    cudaGraph_t graph = nullptr;
+    size_t count = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo_v3(stream, &status, &capture, &graph, &nodes, &edges, &count);
+    if (e == cudaSuccess && status == cudaStreamCaptureStatusNone) {
+        e = cudaStreamGetId(stream, &name.stream);
+        name.known = e == cudaSuccess;
+    } else if (e == cudaSuccess && status == cudaStreamCaptureStatusActive) {
+        name = {reinterpret_cast<uintptr_t>(stream), capture, stream != cudaStreamPerThread};
+    }
+    if (e != cudaSuccess) cudaGetLastError();       // (the launch itself reports what is wrong)
+    seen = g_notes.look(name);
+    if (name.capture != 0 && count != 1) seen.kind = LaunchKind::kNone;
 }
-void note_launch(cudaStream_t stream, LaunchKind kind) {
-    for (int i = 0; i < kLaunchNotes; ++i)
-        if (g_note_stream[i].load(std::memory_order_relaxed) == note_key(stream)) {
-            g_note_kind[i].store(static_cast<int>(kind), std::memory_order_relaxed);
-            return;
-        }
-    const int slot = (int)(g_note_next.fetch_add(1, std::memory_order_relaxed) % kLaunchNotes);
-    g_note_kind[slot].store(static_cast<int>(kind), std::memory_order_relaxed);
-    g_note_stream[slot].store(note_key(stream), std::memory_order_relaxed);
-}
+void StreamNote::launched(LaunchKind kind) const { g_notes.launched(name, seen, kind); }
+void StreamNote::packed() const { g_notes.packed(name); }
 
 template <int BITS>
 static cudaError_t configure_bits() {
@@ -1187,16 +1187,15 @@ static cudaError_t launch_one(const GemvPlan& p, const void* blob, const void* a
     // with two CTAs each, 11 us lost per transition, until the next whole-SM kernel).  So a half-SM GEMV that does not
     // follow another half-SM GEMV of this library on its stream asks for a little more than half of an SM's shared
     // memory: two of its CTAs no longer fit on one SM, a CTA of the next (plain) half-SM GEMV still fits beside it.
-    const int early = may_start_early(stream);
-    if (!FULL && last_launch(stream) != LaunchKind::kHalfSm && cfg.dynamicSmemBytes < (size_t)kGemvSoloSmemBytes)
+    const StreamNote note(stream);
+    if (!FULL && !note.follows_half_sm() && cfg.dynamicSmemBytes < (size_t)kGemvSoloSmemBytes)
         cfg.dynamicSmemBytes = kGemvSoloSmemBytes;
-    note_launch(stream, FULL ? LaunchKind::kWholeSm : LaunchKind::kHalfSm);
     // Programmatic dependent launch: a CTA uses less than half of an SM (shared memory, registers), so the
     // CTAs of the next GEMV on the stream become resident while this one still runs, fill their rings with
     // weights and then wait for this kernel to finish before they touch activations, y or the workspace.
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = early;
+    attr[0].val.programmaticStreamSerializationAllowed = note.may_start_early() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (p.cluster > 1) {
@@ -1212,9 +1211,11 @@ static cudaError_t launch_one(const GemvPlan& p, const void* blob, const void* a
         ce = encode_bf16_map(&act_map, a, 3, dims, strides, box);
         if (ce != cudaSuccess) return ce;
     }
-    return cudaLaunchKernelEx(&cfg, gemv_stream_kernel<BITS, MT, FULL, CL, I8, G>, act_map, static_cast<const uint8_t*>(blob),
-                              static_cast<const __nv_bfloat16*>(a), static_cast<__nv_bfloat16*>(y), M, K, N, p.ktiles, p.total_tiles, p.stages, p.stage_bytes,
-                              p.cluster, p.nclusters, p.ranges, p.xslot_bytes, p.nred, p.piece_tab, static_cast<uint8_t*>(workspace), debug_word());
+    ce = cudaLaunchKernelEx(&cfg, gemv_stream_kernel<BITS, MT, FULL, CL, I8, G>, act_map, static_cast<const uint8_t*>(blob),
+                            static_cast<const __nv_bfloat16*>(a), static_cast<__nv_bfloat16*>(y), M, K, N, p.ktiles, p.total_tiles, p.stages, p.stage_bytes,
+                            p.cluster, p.nclusters, p.ranges, p.xslot_bytes, p.nred, p.piece_tab, static_cast<uint8_t*>(workspace), debug_word());
+    if (ce == cudaSuccess) note.launched(FULL ? LaunchKind::kWholeSm : LaunchKind::kHalfSm);
+    return ce;
 }
 
 template <int BITS>

@@ -385,7 +385,7 @@ cudaError_t launch_gemv_raw(const RawGemvPlan& p, const uint32_t* qweight, const
                             const uint32_t* qzeros, const void* a, void* y, int M, int K, int N, int group_size,
                             void* workspace, cudaStream_t stream) {
     float* partial = static_cast<float*>(workspace);
-    note_launch(stream, LaunchKind::kWholeSm);   // not a half-SM GEMV: the next one must not assume it follows one
+    const StreamNote note(stream);
     cudaError_t e;
     if (p.mma) {
         dim3 grid(p.col_blocks, p.splits, 1);
@@ -399,7 +399,9 @@ cudaError_t launch_gemv_raw(const RawGemvPlan& p, const uint32_t* qweight, const
     if (e != cudaSuccess) return e;
     const int MN = M * N;
     gemv_awq_raw_finish_kernel<<<(MN + 255) / 256, 256, 0, stream>>>(partial, static_cast<__nv_bfloat16*>(y), MN, p.splits);
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    if (e == cudaSuccess) note.launched(LaunchKind::kWholeSm);   // not a half-SM GEMV: the next one must not assume it follows one
+    return e;
 }
 
 }  // namespace tf

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "launch_notes.h"
+
 namespace tf {
 
 // Tuning knobs of the integer path (overridable at compile time for measurements).
@@ -154,13 +156,17 @@ cudaError_t configure_gemv_kernels();
 uint32_t debug_word();
 void set_debug_word(uint32_t word);
 
-// What this library launched last on a stream (the last eight streams are kept; a scheduling hint, see launch_one in gemv.cu).
-enum class LaunchKind : int { kNone = 0, kHalfSm, kWholeSm, kRepack };
-void note_launch(cudaStream_t stream, LaunchKind kind);
-LaunchKind last_launch(cudaStream_t stream);
-// GEMV and GEMM read packed weights before they wait for the kernels ahead of them.  Straight behind the kernel that packs, they
-// are launched as ordinary kernels, so that its stores are done.
-inline int may_start_early(cudaStream_t stream) { return last_launch(stream) == LaunchKind::kRepack ? 0 : 1; }
+// What is known to have been launched last on `stream` (launch_notes.h).  A launch asks when it begins and notes itself once it has been
+// made.
+struct StreamNote {
+    StreamName name;
+    LaunchNotes::Seen seen;
+    explicit StreamNote(cudaStream_t stream);
+    bool may_start_early() const { return seen.kind != LaunchKind::kNone; }
+    bool follows_half_sm() const { return seen.kind == LaunchKind::kHalfSm; }
+    void launched(LaunchKind kind) const;
+    void packed() const;
+};
 
 cudaError_t launch_unpack_w4(const void* blob, uint8_t* q, uint8_t* z, uint16_t* s, int K, int N,
                              int group_size, cudaStream_t stream);

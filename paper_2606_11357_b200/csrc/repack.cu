@@ -161,8 +161,10 @@ cudaError_t launch_repack_awq(const uint32_t* qweight, const uint16_t* scales, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    note_launch(stream, LaunchKind::kRepack);
-    return cudaLaunchKernelEx(&cfg, kernel, qweight, scales, qzeros, static_cast<uint8_t*>(out), K, N, group_size, ktiles, strips);
+    const StreamNote note(stream);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, qweight, scales, qzeros, static_cast<uint8_t*>(out), K, N, group_size, ktiles, strips);
+    note.packed();
+    return e;
 }
 
 }  // namespace tf
