@@ -123,6 +123,25 @@ __device__ __forceinline__ void grid_launch_dependents() {
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// Loads of what earlier kernels of the stream have written, for a kernel that may have started before they ended: volatile, which
+// keeps them behind the wait, and coherent.  (__ldg and const __restrict__ promise data that nobody writes while the grid exists.
+// __ldcg and __ldcs promise nothing, but the compiler takes them for functions of the address and may move them ahead of a wait or out of a
+// loop.)
+__device__ __forceinline__ uint32_t load_behind_wait(const uint16_t* p) {
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t load_behind_wait(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 load_once_behind_wait(const uint2* p) {       // not wanted again: first to leave the L2
+    uint2 v;
+    asm volatile("ld.global.cs.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
 
 // ---- thread-block clusters ---------------------------------------------------------------------------
 // Address of the same shared-memory location in CTA `rank` of this cluster (shared::cluster window).

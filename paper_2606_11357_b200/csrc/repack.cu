@@ -38,13 +38,13 @@ __device__ __forceinline__ void transpose_bytes(uint32_t r0, uint32_t r1, uint32
 // the kernels ahead of them.
 constexpr int kRepackThreads = 256, kRepackStrips = 4;
 template <bool kPairs, int G>      // G: groups per tile; kPairs: rows are a whole number of word pairs, so a thread's two words are one 8-byte load
-__global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32_t* __restrict__ qweight, const uint16_t* __restrict__ scales,
-                                                                    const uint32_t* __restrict__ qzeros, uint8_t* __restrict__ out, int K, int N,
+__global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32_t* qweight, const uint16_t* scales,
+                                                                    const uint32_t* qzeros, uint8_t* __restrict__ out, int K, int N,
                                                                     int group_size, int ktiles, int strips) {
     constexpr int tile_bytes_here = w4_tile_bytes(G);
     const int T = blockIdx.y, S0 = kRepackStrips * blockIdx.x;
     const int row_words = N >> 3;
-    grid_dependency_wait();                  // the arrays may come from earlier kernels, and they may still read what `out` held
+    grid_dependency_wait();                  // the arrays may come from earlier kernels, and those may still read what `out` held
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         tf_blob_header h = {};
         h.magic = kMagic; h.version = kBlobVersion; h.bits = 4; h.K = (uint32_t)K; h.N = (uint32_t)N;
@@ -70,15 +70,15 @@ __global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32
             const int gr = wi / (kScaleBytes / 4), rest = wi % (kScaleBytes / 4);
             const int n = n0 + 16 * (rest & 3) + (rest >> 2);
             const int grp = G > 1 ? T * G + gr : T * kTileK / group_size;
-            meta[it][0] = n < N ? __ldg(scales + (size_t)grp * N + n) : 0u;
-            meta[it][1] = n + 8 < N ? __ldg(scales + (size_t)grp * N + n + 8) : 0u;
+            meta[it][0] = n < N ? load_behind_wait(scales + (size_t)grp * N + n) : 0u;
+            meta[it][1] = n + 8 < N ? load_behind_wait(scales + (size_t)grp * N + n + 8) : 0u;
         } else {                                                      // [group][g]
             const int gr = (wi - G * (kScaleBytes / 4)) / (kZeroBytes / 4);
             const int grp = G > 1 ? T * G + gr : T * kTileK / group_size;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {                             // nibble j: column 16 (j & 3) + 8 (j >> 2) + g
                 const int zw = n0 / 8 + 2 * (j & 3) + (j >> 2);
-                meta[it][j] = zw < row_words ? __ldg(qzeros + (size_t)grp * row_words + zw) : 0u;
+                meta[it][j] = zw < row_words ? load_behind_wait(qzeros + (size_t)grp * row_words + zw) : 0u;
             }
         }
     }
@@ -97,12 +97,12 @@ __global__ void __launch_bounds__(kRepackThreads) repack_awq_kernel(const uint32
                     even[it][r] = odd[it][r] = 0u;
                     if (kPairs) {
                         if (word0 < row_words) {
-                            const uint2 v = __ldcs(reinterpret_cast<const uint2*>(src + (size_t)r * row_words));
+                            const uint2 v = load_once_behind_wait(reinterpret_cast<const uint2*>(src + (size_t)r * row_words));
                             even[it][r] = v.x; odd[it][r] = v.y;
                         }
                     } else {
-                        if (word0 < row_words) even[it][r] = __ldg(src + (size_t)r * row_words);
-                        if (word0 + 1 < row_words) odd[it][r] = __ldg(src + (size_t)r * row_words + 1);
+                        if (word0 < row_words) even[it][r] = load_behind_wait(src + (size_t)r * row_words);
+                        if (word0 + 1 < row_words) odd[it][r] = load_behind_wait(src + (size_t)r * row_words + 1);
                     }
                 }
             }
@@ -161,7 +161,7 @@ cudaError_t launch_repack_awq(const uint32_t* qweight, const uint16_t* scales, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const StreamNote note(stream);
+    const StreamNote note(stream);           // (a packing goes by nothing; it is noted whatever became of the launch)
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, qweight, scales, qzeros, static_cast<uint8_t*>(out), K, N, group_size, ktiles, strips);
     note.packed();
     return e;

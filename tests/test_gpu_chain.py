@@ -174,3 +174,35 @@ def test_packing_between_calls(kind, M, K, N, captured):
     assert tf.tf_device_status(ws) == 0
     for p, y in zip(problems, ys):
         gu.check_against_oracle(p, gu.bits_of(y))
+
+
+@pytest.mark.parametrize("M,K,N", [(16, 256, 1024), (3, 384, 264), (200, 512, 4096)])
+@pytest.mark.parametrize("group", [128, 32])
+def test_packing_what_the_call_just_ahead_has_written(M, K, N, group):
+    """The packer starts before the GEMV or GEMM ahead of it has ended, and its three arrays are parts of that call's result, rewritten in place
+    each time: what it packs is what that call wrote.  (264 columns: rows of 33 words, read one by one.)"""
+    rows = K // group
+    words = [K * N // 8, (rows * N // 2 + 3) // 4 * 4, (rows * N // 8 + 3) // 4 * 4]           # qweight, scales, qzeros; each 16-byte aligned
+    Np = (sum(words) * 2 // M // 64 + 1) * 64                                                # M x Np bf16 results hold them
+    kind, Kp = "gemv" if M <= 16 else "gemm", 2048
+    p = wl.make_w4(M, Kp, Np, seed=80 + M)
+    producer, ws = torch.from_numpy(gu.pack(p)).cuda(), torch.zeros(tf.tf_workspace_size(tf.TF_OP_GEMM_W4A16, M, Kp, Np), dtype=torch.uint8, device="cuda")
+    call = tf.tf_gemv_w4a16 if kind == "gemv" else tf.tf_gemm_w4a16
+    inputs = [gu.to_device_bf16(p.a_bf16), gu.to_device_bf16(p.a_bf16[:, ::-1].copy()), gu.to_device_bf16(p.a_bf16 ^ np.uint16(0x8000))]
+    y = torch.zeros(M, Np, dtype=torch.bfloat16, device="cuda")
+    flat = y.view(-1).view(torch.int32)
+    q, s, z = flat[:words[0]], flat[words[0]:words[0] + words[1]], flat[words[0] + words[1]:sum(words)]
+    blobs = [torch.zeros(tf.tf_packed_size(4, K, N, group), dtype=torch.uint8, device="cuda") for _ in inputs]
+    call(producer, inputs[0], y, M, Kp, Np, ws)
+    for a, blob in zip(inputs, blobs):
+        call(producer, a, y, M, Kp, Np, ws)
+        tf.tf_pack_awq_device(q, s, z, K, N, group, blob)
+    assert tf.tf_device_status(ws) == 0
+    for a, blob in zip(inputs, blobs):
+        call(producer, a, y, M, Kp, Np, ws)
+        torch.cuda.synchronize()
+        words_now = flat.cpu().numpy()
+        hq = words_now[:words[0]].view(np.uint32).reshape(K, N // 8)
+        hs = words_now[words[0]:words[0] + words[1]].view(np.float16)[:rows * N].reshape(rows, N)
+        hz = words_now[words[0] + words[1]:sum(words)].view(np.uint32)[:rows * N // 8].reshape(rows, N // 8)
+        assert np.array_equal(tf.tf_pack_awq(hq.copy(), hs.copy(), hz.copy(), K, N, group), blob.cpu().numpy())
