@@ -208,7 +208,7 @@ struct DrainShare {
 #pragma unroll
                         for (int h = 0; h < 2; ++h)
                             if (o + b < others && (k == 0 || second))
-                                x[b][k][h] = __ldcg(slots + (o + b) * stride + slot_index(quarter, c + k * kGroups) + 32 * h);
+                                x[b][k][h] = load_behind_wait(slots + (o + b) * stride + slot_index(quarter, c + k * kGroups) + 32 * h);
             };
             load(0);
 #pragma unroll

@@ -250,7 +250,7 @@ struct NoActMap {};
 template <int I8> using GemvActMap = std::conditional_t<I8 == 0, CUtensorMap, NoActMap>;      // floating-point path: [K / 64][M][64] activations
 template <int BITS, int MT, bool FULL, bool CL, int I8, int G = 1>
 __global__ void __launch_bounds__(gemv_max_threads(BITS, MT, FULL, I8 != 0), FULL ? 1 : 2)
-gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t* __restrict__ blob, const __nv_bfloat16* __restrict__ a_glob, __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int total_tiles,
+gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t* __restrict__ blob, const __nv_bfloat16* a_glob, __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int total_tiles,
                    int nstages, int stage_bytes, int csize, int nclusters, const Ranges ranges, int xslot_bytes, int nred, int piece_tab,
                    uint8_t* __restrict__ workspace, uint32_t debug) {
     static_assert(G == 1 || (BITS == 4 && !I8 && !CL && FULL), "several groups per tile: 4-bit, floating-point path, whole SM");
@@ -513,7 +513,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 araw[m] = make_uint2(0u, 0u);
-                if (m < M) araw[m] = __ldcg(reinterpret_cast<const uint2*>(base + (size_t)m * K + 4 * lane));
+                if (m < M) araw[m] = load_behind_wait(reinterpret_cast<const uint2*>(base + (size_t)m * K + 4 * lane));
             }
         };
         constexpr int kColWords = kGemvPieceColWords;

@@ -9,7 +9,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2606_11357_b200", "csrc")
 
 
-@pytest.mark.parametrize("name", ["repack.cu"])
+@pytest.mark.parametrize("name", ["repack.cu", "gemv.cu", "gemm.cu"])
 def test_loads_of_earlier_kernels_results_stay_behind_the_wait(name):
     code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
     assert "grid_dependency_wait()" in code
