@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "launch_notes.h"
+#include "split.h"
 
 namespace tf {
 
@@ -94,37 +95,6 @@ constexpr int kGemvPartialOffset = kWorkspaceHeadBytes;
 constexpr int kGemvSlotBytes = kGemvMaxM * 64 * 4;
 constexpr size_t kWorkspaceZeroBytes = kGemvPartialOffset + (size_t)kGemvMaxGrid * kGemvSlotBytes;
 constexpr size_t kGemvWorkspaceBytes = kWorkspaceZeroBytes;
-
-// How a sequence of units (tiles) is dealt out to CTAs as contiguous ranges.  A CTA finds its range without a division, which would
-// sit between its start and its first copy: of the first on_time CTAs `more` get size + 1 units, the rest size, and the others, the late
-// ones, likewise.  (GEMM 24x4096x14336 18.2 us with two divisions per CTA, 16.8 without, 40x8192x8192 20.5 and 18.8; GEMV 16 tokens
-// 14336x4096 10.9 and 10.5, 4 tokens 9.0 and 8.8.)
-// CTAs start in the order of their index as SMs come free; in a chain of kernels that take a whole SM each, the last ten or so start up
-// to 3 us behind the others, and the call ends with them.  So they can be given shorter ranges.
-struct Ranges {
-    int on_time, size, more, bulk;             // the first on_time CTAs share the first bulk units
-    int late_size, late_more;
-    static Ranges make(int units, int ctas, int late = 0, int less = 0) {      // `late` CTAs get about `less` units less than the others
-        Ranges r;
-        const int late_units = late > 0 ? late * ((units + late * less) / ctas - less) : 0;
-        r.on_time = ctas - late;
-        r.bulk = units - late_units;
-        r.size = r.bulk / r.on_time; r.more = r.bulk % r.on_time;
-        r.late_size = late > 0 ? late_units / late : 0; r.late_more = late > 0 ? late_units % late : 0;
-        return r;
-    }
-#ifdef __CUDACC__
-    __device__ int start(int cta) const {
-        const int c = cta - on_time;
-        return c <= 0 ? cta * size + min(cta, more) : bulk + c * late_size + min(c, late_more);
-    }
-    __device__ int owner(int unit) const {
-        const bool late = unit >= bulk;
-        const int u = late ? unit - bulk : unit, q = late ? late_size : size, m = late ? late_more : more, head = m * (q + 1);
-        return (late ? on_time : 0) + (int)(u < head ? (uint32_t)u / (uint32_t)(q + 1) : m + (uint32_t)(u - head) / (uint32_t)q);
-    }
-#endif
-};
 
 struct GemvPlan {
     int grid;          // persistent CTAs
