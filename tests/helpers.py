@@ -1,5 +1,6 @@
 """Shared helpers for the tests: tolerance rule, tiny independent encoders, golden readers."""
 import os
+import re
 
 import numpy as np
 
@@ -62,6 +63,10 @@ def read_golden_dequant():
             kind, q, z, s, a, w, aw = line.split()
             cases.append((kind, int(q), int(z), float(s), float(a), float(w), float(aw)))
     return cases
+
+
+with open(os.path.join(os.path.dirname(GOLDEN), "..", "include", "tilefuse.h")) as _fh:
+    WORKSPACE_ZERO_BYTES = int(re.search(r"#define TF_WORKSPACE_ZERO_BYTES\s+(\d+)", _fh.read()).group(1))
 
 
 # ----------------------------------------------------------------------------------------------

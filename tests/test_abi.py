@@ -8,6 +8,7 @@ import sys
 import numpy as np
 import pytest
 
+from helpers import WORKSPACE_ZERO_BYTES
 from paper_2606_11357_b200 import binding as tf
 from paper_2606_11357_b200 import build as tfbuild
 
@@ -96,7 +97,7 @@ def test_compute_calls_validate_before_touching_the_gpu():
 def test_gemm_workspace_is_one_slot_of_partial_sums_per_cta(M, tokens):
     """Behind the zeroed part: fp32 sums of one tile (128 columns x the widest token tile of the call's class) for each of 160 CTAs."""
     for op in (tf.TF_OP_GEMM_W4A16, tf.TF_OP_GEMM_W8A16):
-        assert tf.tf_workspace_size(op, M, 4096, 14336) == 1069056 + 160 * 128 * tokens * 4
+        assert tf.tf_workspace_size(op, M, 4096, 14336) == WORKSPACE_ZERO_BYTES + 160 * 128 * tokens * 4
 
 
 def test_device_calls_check_their_arguments_before_the_library_is_called():

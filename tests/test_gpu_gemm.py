@@ -6,7 +6,7 @@ import torch
 from oracle import tilefuse_oracle as orc
 from paper_2606_11357_b200 import binding as tf
 from paper_2606_11357_b200 import workloads as wl
-from helpers import bf16_bits_to_f64
+from helpers import WORKSPACE_ZERO_BYTES, bf16_bits_to_f64
 import gpu_util as gu
 
 pytestmark = pytest.mark.gpu
@@ -217,7 +217,7 @@ def test_gemm_cuts(bits, group, M, K, N):
             getattr(tf, f"tf_gemm_w{bits}a16")(blob, a, y, M, K, N, ws)
         else:
             tf.tf_gemm_w4a16_grouped(blob, a, y, M, K, N, group, ws)
-        assert tf.tf_device_status(ws) == 0 and not bool(ws[:1069056].any())
+        assert tf.tf_device_status(ws) == 0 and not bool(ws[:WORKSPACE_ZERO_BYTES].any())
         ys.append(gu.bits_of(y))
     assert np.array_equal(ys[0], ys[1])
     gu.check_against_oracle(p, ys[0], columns=np.unique(np.concatenate([np.arange(0, N, 41), [N - 1]])))
