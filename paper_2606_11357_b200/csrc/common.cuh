@@ -84,8 +84,8 @@ __device__ __forceinline__ uint32_t header_group_size(const void* blob) {
 }
 // The same in two steps, for a kernel that has something to do while the header is on its way: the words are asked for at its start
 // and judged where the answer is needed (GEMV, floating-point path, a chain of whole-SM kernels, where the set-up of the last CTAs is on
-// the call's way: 4 tokens 4096x6144 5.76 -> 5.56 us, 14336x4096 8.77 -> 8.56, 16 tokens 4096x28672 18.7 -> 18.5).  With the group size, which has to fit a kernel built for G groups per tile (G = 1: any
-// multiple of the tile's k-extent; G = 2, 4: exactly 128 / G).
+// the call's way: 4 tokens 4096x6144 5.76 -> 5.56 us, 14336x4096 8.77 -> 8.56, 16 tokens 4096x28672 18.7 -> 18.5).  With the group
+// size, which has to fit a kernel built for G groups per tile (G = 1: any multiple of the tile's k-extent; G = 2, 4: exactly 128 / G).
 struct HeaderWords {
     uint4 a;            // magic, version, bits, K
     uint2 b;            // N, group size

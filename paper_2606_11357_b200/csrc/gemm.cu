@@ -28,10 +28,11 @@
 // (split_gemm).  A CTA that computes part of a tile whose last k-tile is another CTA's does that first and writes its fp32 sums
 // to the workspace; the owner of the last k-tile adds them to its own in CTA order (deterministic) and stores y.
 // What bounds it: with 256 tokens the tensor pipe, 73 % active over a launch (inside a tile a k-tile takes 1060 cycles, 1024 of them
-// MMA; start, drains and cuts bring it to about 1400), at a clock that the power limit holds down in a loop (1.4 to 1.6 GHz); up to 128 tokens the issue slots of the dequant warps and the waits of the warp that issues
-// the MMAs (0.43 to 0.6 us per k-tile), for short calls the 4 to 5 us around them.  Before (eight dequant warps on one k-tile at
-// a time, a packed ring of 26 KB, partial sums through an arrival counter): 0.61 to 0.83 us per k-tile; 32x4096x18944 24.1 ->
-// 20.2 us, 96x2944x11016 18.9 -> 15.0, 297x2944x11016 33.5 -> 25.5, W8 1024x4096x4096 32.9 -> 29.6, 512x4096x4096 31.1 -> 24.3.
+// MMA; start, drains and cuts bring it to about 1400), at a clock that the power limit holds down in a loop (1.4 to 1.6 GHz); up
+// to 128 tokens the issue slots of the dequant warps and the waits of the warp that issues the MMAs (0.43 to 0.6 us per k-tile),
+// for short calls the 4 to 5 us around them.  us per call in a chain: 32x4096x18944 17.9, 96x2944x11016 13.9, 297x2944x11016 26.1,
+// int8 1024x4096x4096 28.2, 512x4096x4096 20.5.  (With eight dequant warps on one k-tile at a time, a packed ring of 26 KB and partial
+// sums through an arrival counter a k-tile took 0.61 to 0.83 us and these calls 24.1, 18.9, 33.5, 32.9 and 31.1.)
 // Every mbarrier wait is bounded; on a timeout all roles leave, TMEM is freed, the status word is set.
 #include <cuda.h>
 
@@ -95,12 +96,13 @@ inline GemmRings gemm_rings(int bits, int BT, int bt, int G) {
     return r;
 }
 
-// workspace: [0,16) status | [kGemmFlagOffset, + 64 * CTAs) "this dequant warp's part of its CTA's slot is filled" | (the GEMV's partial-sum slots, not
-// touched here) | one slot of BT tokens x 128 columns of fp32 sums per CTA (the part of a tile it contributes)
+// workspace: [0,16) status | [kGemmFlagOffset, + 64 * CTAs) "this dequant warp's part of its CTA's slot is filled" | (the GEMV's
+// partial-sum slots, not touched here) | one slot of BT tokens x 128 columns of fp32 sums per CTA (the part of a tile it contributes)
 constexpr int kGemmFlagOffset = 4096;          // zero between calls
 constexpr size_t kGemmPartialOffset = kWorkspaceZeroBytes;      // behind the GEMV's partial-sum slots, which must stay zero
 constexpr int kGemmMaxGrid = 160;
-static_assert(kGemmFlagOffset >= kGemvStatusBytes && kGemmFlagOffset + 4 * 4 * kGroups * kGemmMaxGrid <= kWorkspaceHeadBytes, "workspace layout shared with the GEMV");
+static_assert(kGemmFlagOffset >= kGemvStatusBytes && kGemmFlagOffset + 4 * 4 * kGroups * kGemmMaxGrid <= kWorkspaceHeadBytes,
+              "workspace layout shared with the GEMV");
 
 // The CTA's unit range [u_begin, u_end) as segments of one output tile each, in processing order: the last tile first.  A tile
 // that is cut between CTAs belongs to the CTA that has its last k-tile.  For that CTA it is the first tile of its range and comes
@@ -265,7 +267,8 @@ __device__ __forceinline__ uint32_t times_scale(uint32_t d, uint32_t hi2, uint32
 template <int BITS, int BT, int G = 1>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restrict__ blob,
-            __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int n_tiles, int m_tiles, int bt, int act_stages, int wp_stages, int aligned, const Ranges ranges,
+            __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int n_tiles, int m_tiles, int bt, int act_stages,
+            int wp_stages, int aligned, const Ranges ranges,
             uint8_t* __restrict__ workspace, uint32_t debug) {
     static_assert(G == 1 || BITS == 4, "several groups per tile: the 4-bit format only");
     constexpr int kTileBytes = tile_bytes(BITS, G);

@@ -13,10 +13,10 @@
 //                   Floating-point path (3..16 tokens, small groups): a stage also gets the activations of its tiles by a
 //                   tensor copy, the first ones behind the dependency wait.
 //   consumer warps: take tiles round-robin.  Floating-point path: the activations lie in the ring, brought once per CTA,
-//                   as deep ahead as the ring, by no instruction or wait of a consumer warp.  (Before, a warp loaded the
-//                   fragments of its next tile to registers, with 9..16 tokens to a buffer of its own, which took 3 to 5 of
-//                   its 26 thousand cycles and the room of four ring stages.  4096x28672: 4 tokens 16.3 -> 15.7 us, 8 tokens
-//                   17.6 -> 15.9, 16 tokens 23.2 -> 20.4; 16 tokens 4096x4096 7.9 -> 7.2, int8 4096x9472 12.8 -> 10.5.)
+//                   as deep ahead as the ring, by no instruction or wait of a consumer warp.  (Loaded by the warps, fragments of
+//                   the next tile to registers or, with 9..16 tokens, to a buffer of the warp's own, they took 3 to 5 of a warp's 26
+//                   thousand cycles and the room of four ring stages: the change alone took 4096x28672 from 16.3 to 15.7 us at
+//                   4 tokens, from 17.6 to 15.9 at 8 and from 23.2 to 20.4 at 16.  It is 14.1, 14.1 and 18.5 now.)
 //                   Integer path: a lane reads its 4 k of the tile's 128 per token straight from global memory (they
 //                   sit in L2), one tile ahead and never before the kernels ahead of this one on the stream have completed.
 //                   128-bit shared loads, codes -> exact small-integer bf16
@@ -30,10 +30,10 @@
 //   The last segment of a range is on the way of the whole call, and nobody has tiles left: there the consumer warps add up a
 //   slice each (two token rows), and those of the CTA that puts a cut strip together fetch the same slice of the others' sums, asked
 //   for before they wait for their own.  From the last consumer to the end of the kernel it took 2.2 us (4 tokens, 14336x4096)
-//   when the one reducer warp did it, one contributor after the other, and takes 1.0 now.  us per call, before -> after: 16 tokens 14336x4096 12.8 -> 11.0, 4096x6144 8.7 -> 7.1, 4 tokens 4096x4096 5.1 -> 4.5, 14336x4096 9.8 -> 9.0, 6 tokens, group 64,
-//   7424x18440 17.4 -> 16.4, 1 and 16 tokens 32768x1024 10.1 -> 7.2 and 14.1 -> 9.3.  The integer path has one slice; its reducer
-//   does the same, as it has time to look for the others' sums while the consumers work (by a consumer warp: 1 token 14336x4096 8.4
-//   us, by the reducer 8.2).
+//   when the one reducer warp did it, one contributor after the other, and takes 1.0 now: that change alone, us per call, 16 tokens
+//   14336x4096 12.8 -> 11.0, 4096x6144 8.7 -> 7.1, 4 tokens 4096x4096 5.1 -> 4.5, 14336x4096 9.8 -> 9.0, 1 and 16 tokens 32768x1024
+//   10.1 -> 7.2 and 14.1 -> 9.3.  The integer path has one slice; its reducer does the same, as it has time to look for the
+//   others' sums while the consumers work (by a consumer warp 1 token 14336x4096 took 8.4 us where the reducer took 8.2).
 //
 // A range may cut a strip (64 output columns) in two.  A CTA that holds a whole strip stores y
 // directly.  Otherwise its fp32 partial goes to the workspace, and the CTA that has the strip's first tile
@@ -76,13 +76,15 @@ __device__ __forceinline__ void mma_u8s8_16832_first(int d[4], uint32_t a0, uint
 }
 
 // int -> float for |v| < 2^22 without the conversion unit: the bits of the integer 0x4B400000 + v are the float
-// 1.5 * 2^23 + v, exactly.  A tile's sums get the bias as the start of the MMAs' accumulators or with the zero point, and (f - 1.5 * 2^23) * c is one fused multiply-add with -1.5 * 2^23 * c.
+// 1.5 * 2^23 + v, exactly.  A tile's sums get the bias as the start of the MMAs' accumulators or with the zero point, and
+// (f - 1.5 * 2^23) * c is one fused multiply-add with -1.5 * 2^23 * c.
 constexpr int kIntAsFloatBias = 0x4B400000;
 constexpr float kIntAsFloatBiasValue = 12582912.0f;
 
-// Even split of `total` tiles (or strips) over the CTAs of a cluster (or the clusters); the grid's own ranges come with the launch.  32-bit: the products stay below 2^26 (at most 256 x 512 tiles, K and N <= 32768,
-// times at most 257), and a 64-bit division is several times the instructions.  These sit between the start of a CTA and its
-// first weight copy, in the reducer's bookkeeping and in the cluster-mode finish.
+// Even split of `total` tiles (or strips) over the CTAs of a cluster (or the clusters); the grid's own ranges come with the launch.
+// 32-bit: the products stay below 2^26 (at most 256 x 512 tiles, K and N <= 32768, times at most 257), and a 64-bit division is several
+// times the instructions.  These sit between the start of a CTA and its first weight copy, in the reducer's bookkeeping and in
+// the cluster-mode finish.
 __device__ __forceinline__ int range_start(int cta, int total, int grid) {
     return static_cast<int>((static_cast<uint32_t>(cta) * static_cast<uint32_t>(total)) / static_cast<uint32_t>(grid));
 }
@@ -250,8 +252,9 @@ struct NoActMap {};
 template <int I8> using GemvActMap = std::conditional_t<I8 == 0, CUtensorMap, NoActMap>;      // floating-point path: [K / 64][M][64] activations
 template <int BITS, int MT, bool FULL, bool CL, int I8, int G = 1>
 __global__ void __launch_bounds__(gemv_max_threads(BITS, MT, FULL, I8 != 0), FULL ? 1 : 2)
-gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t* __restrict__ blob, const __nv_bfloat16* a_glob, __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int total_tiles,
-                   int nstages, int stage_bytes, int csize, int nclusters, const Ranges ranges, int xslot_bytes, int nred, int piece_tab,
+gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t* __restrict__ blob, const __nv_bfloat16* a_glob,
+                   __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int total_tiles, int nstages, int stage_bytes,
+                   int csize, int nclusters, const Ranges ranges, int xslot_bytes, int nred, int piece_tab,
                    uint8_t* __restrict__ workspace, uint32_t debug) {
     static_assert(G == 1 || (BITS == 4 && !I8 && !CL && FULL), "several groups per tile: 4-bit, floating-point path, whole SM");
     static_assert((FULL || I8) && (!CL || MT == 2) && (I8 != 2 || BITS == 4), "forms that plan_gemv never chooses");
@@ -364,7 +367,8 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
     constexpr int kVec = (I8 ? 2 : kTok) / 2;             // slices of a strip
     auto hand_over = [&](float4 v, int e, int to) {
         if (CL) {
-            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(map_to_cta(smem_u32(xred + (size_t)crank * xslot_bytes), (uint32_t)to) + (32 * e + lane) * 16),
+            const uint32_t slot = map_to_cta(smem_u32(xred + (size_t)crank * xslot_bytes), (uint32_t)to);
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(slot + (32 * e + lane) * 16),
                          "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
         } else {
             __stcg(reinterpret_cast<float4*>(partials + (size_t)crank * (kGemvMaxM * kTileN)) + 32 * e + lane, never_plus_zero(v));
@@ -974,17 +978,17 @@ static int max_resident_clusters(int csize) {
 static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool full) {
     const int mt = M <= 8 ? 1 : 2;
     p.full = full;
-    // whole-SM integer path: about 66 KB of tiles in the consumer warps' hands (16 warps on 4-bit tiles, 8 on int8 tiles)
-    // and the rest of the ring in flight.  Measured alone, one token: 4096x32768 4-bit 20.7 us half SM, 20.7 / 18.8 /
-    // 18.1 whole SM with 8 / 12 / 16 warps; 4096x14336 int8 15.8 us half SM, 12.7 / 13.3 / 14.6 whole SM with 8 / 12 / 16.
+    // whole-SM integer path: about 66 KB of tiles in the consumer warps' hands (16 warps on 4-bit tiles, 8 on int8 tiles) and the rest
+    // of the ring in flight (when it was chosen, one token, 8 / 12 / 16 warps: 4096x32768 4-bit 20.7 / 18.8 / 18.1 us, 4096x14336 int8
+    // 12.7 / 13.3 / 14.6).
     p.consumers = p.i8 && p.full ? gemv_i8_full_consumers(bits) : gemv_max_consumers(mt, p.full);
     // Floating-point path up to 8 tokens: 12 warps only for long ranges of 4-bit tiles.  Eight have fewer partial sums to add up
-    // at the end of a strip and less of the ring in their hands: us with 8 / 12, 4 tokens 14336x4096 (49 tiles) 8.35 / 8.53, 4096x14336 8.78
-    // either way, a decoder layer 33.7 / 34.0; 4096x28672 (97 tiles) 16.4 / 15.8 and int8, 8 tokens, 22.1 / 23.1 in an earlier form.  With
-    // four groups per tile, whose scales are more work, 5 tokens 4096x14336 9.85 / 9.62.  (10, 11 and 14 warps are slower than 8, 12 and
-    // 16 everywhere, 14336x4096 11.1 us against 10.6: with a multiple of the tiles of a chunk a warp always works on the same place of
-    // a stage, and a stage is freed by warps that are about equally far.)
-    if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < (p.groups == 1 ? kGemvFpTwelveWarpsFromTiles : kGemvFpTwelveWarpsFromTilesGrouped))) p.consumers = 8;
+    // at the end of a strip and less of the ring in their hands: us with 8 / 12, 4 tokens 14336x4096 (49 tiles) 8.35 / 8.53, a decoder layer
+    // 33.7 / 34.0; 4096x28672 (97 tiles), when it was chosen, 16.4 / 15.8 and int8 at 8 tokens 22.1 / 23.1.  With four groups per tile,
+    // whose scales are more work, 5 tokens 4096x14336 9.85 / 9.62.  A multiple of the tiles of a chunk, so that a warp always works on
+    // the same place of a stage and a stage is freed by warps that are about equally far (10, 11 and 14 warps are slower than 8, 12, 16).
+    const int twelve_from = p.groups == 1 ? kGemvFpTwelveWarpsFromTiles : kGemvFpTwelveWarpsFromTilesGrouped;
+    if (mt == 1 && !p.i8 && (bits == 8 || tiles_per_cta < twelve_from)) p.consumers = 8;
     if (tiles_per_cta < p.consumers) p.consumers = tiles_per_cta < 4 ? 4 : tiles_per_cta;
     p.threads = 32 * (p.consumers + 2);          // + producer warp + reducer warp
     const int kr = gemv_chunk_tiles(bits);
@@ -1004,21 +1008,21 @@ static void lay_out_gemv(GemvPlan& p, int bits, int M, int tiles_per_cta, bool f
     // no more stages than the range has chunks
     const int chunks = (tiles_per_cta + kr - 1) / kr + 2;
     if (stages > chunks) stages = chunks;
-    // whole-SM integer path: a ring deeper than eight stages was slower (1x4096x32768 4-bit: 17.0 / 16.9 / 17.5 us with
-    // 6 / 8 / 10 stages; int8 1x4096x14336: 12.8 / 12.5 / 12.7 us with 6 / 8 / 11)
+    // whole-SM integer path: a ring deeper than eight stages was slower (when it was chosen, 1x4096x32768 4-bit 17.0 / 16.9 / 17.5 us
+    // with 6 / 8 / 10 stages, int8 1x4096x14336 12.8 / 12.5 / 12.7 with 6 / 8 / 11)
     if (p.i8 && p.full && stages > kGemvI8FullMaxStages) stages = kGemvI8FullMaxStages;
     // floating-point path up to 8 tokens on 4-bit tiles: five stages with 8 consumer warps (two in their hands), six with 12 (three).
-    // us with 5 / 6 / 7 stages: 8 warps, 4 tokens 4096x6144 5.57 / 5.71 / 5.71, 14336x4096 8.35 / - / 9.01; 12 warps 4096x28672 14.25 / 14.07 /
-    // 14.07, 6 tokens, group 64, 7424x18440 16.4 / 16.1 / 16.2, four groups per tile 5 tokens 4096x14336 9.58 / 9.77.  int8 tiles (four or six
-    // stages in the warps' hands) want the deep ring: 4096x14336 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us with 4 / 5 / 6 / 7 / 9 in an earlier form.
-    // (Why a deeper ring is slower on 4-bit tiles was not established.)
+    // us with 5 / 6 / 7 stages: 8 warps, 4 tokens 4096x6144 5.57 / 5.71 / 5.71, 14336x4096 8.35 / - / 9.01; 12 warps 4096x28672 14.25 /
+    // 14.07 / 14.07, four groups per tile 5 tokens 4096x14336 9.58 / 9.77.  (Why a deeper ring is slower on 4-bit tiles was not
+    // established.)  int8 tiles (four or six stages in the warps' hands) want the deep ring: when it was chosen, 4096x14336 at 4 tokens
+    // 19.6 / 18.4 / 17.4 / 16.6 / 16.0 us with 4 / 5 / 6 / 7 / 9 (11.8 now).
     const int most = p.consumers > 8 && p.groups < 4 ? kGemvFpW4MaxStages12 : kGemvFpW4MaxStages8;
     if (!p.i8 && mt == 1 && bits == 4 && stages > most) stages = most;
     // Integer path: where a range passes over the same k-tiles more than once and K is a multiple of 128 x consumer
     // warps, every warp meets the same k-tiles on each pass and keeps the activation pieces it has prepared (one table
     // entry per k-tile instead of one scratch entry per warp), if that costs the ring no stage.
     p.piece_tab = 0;
-    // (4-bit weights only: on int8 tiles, whole SM, the table was the slower form, 13.1 against 12.5 us on 1x4096x14336)
+    // (4-bit weights only: on int8 tiles, whole SM, the table was the slower form, 13.1 against 12.5 us on 1x4096x14336 then)
     if (p.i8 && bits == 4 && tiles_per_cta >= p.ktiles + p.consumers && p.ktiles % p.consumers == 0) {
         const int table = (p.ktiles * kGemvPieceEntryBytes * M + 1023) / 1024 * 1024;
         int with = (gemv_smem_budget(mt, p.full) - (base + table)) / p.stage_bytes;
@@ -1064,7 +1068,7 @@ GemvPlan plan_gemv(int bits, int M, int K, int N, int sm_count, int groups) {
         int want = 0;
         if (tiles_per_cta < nc) {
             // (A strip of fewer k-tiles is one CTA's.  With eight tiles per CTA all the same, its strips came one after the
-            // other, 1 us each: 1x512x4096 took 3.4 us, now 2.4; 4x128x4096 10.5, now 2.2.)
+            // other, 1 us each: 1x512x4096 took 3.4 us, now 2.0; 4x128x4096 10.5, now 2.0.)
             want = p.ktiles < nc ? p.ktiles * ((p.strips + p.grid - 1) / p.grid) : nc;
         } else if (tiles_per_cta <= 2 * nc) {
             const int rounds = (tiles_per_cta + nc - 1) / nc;

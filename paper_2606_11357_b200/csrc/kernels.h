@@ -51,21 +51,17 @@ constexpr int kGemvPieceEntryBytes = 512;
 // eight stages; with about 66 KB of tiles in the warps' hands (8 warps on int8, 16 on 4-bit tiles) it streams long
 // ranges faster than the half-SM form, which wins on short ranges because the next GEMV's CTAs sit beside it with
 // their rings full.
-// int8, one token, us half SM / whole SM: 1024x8192 (67 KB) 2.41 / 3.13, 2048x4096 3.20 / 3.46, then 14336x1024 (119 KB) 5.99 / 4.82, 4096x3072
-// (133 KB) 5.33 / 4.08, 4096x4096 5.47 / 4.66, 2048x11008 6.30 / 5.60; two tokens 4096x4096 5.55 / 4.90.
+// int8, one token, us half SM / whole SM: 1024x8192 (67 KB per CTA) 2.41 / 3.13, 2048x4096 3.20 / 3.46, 14336x1024 (119 KB) 5.99 / 4.82,
+// 4096x4096 5.47 / 4.66.
 constexpr int kGemvFullFromBytesI8W4 = TF_I8_FULL_BYTES_W4;
 constexpr int kGemvFullFromBytesI8W8 = TF_I8_FULL_BYTES_W8;
-// 4-bit tiles, the half-SM form without / with its activation pieces kept (piece table).  Figures: us per call in a chain of one
-// shape, one token, half SM / whole SM.
-// Without the table a tile costs a half-SM warp its preparation as well, and eight warps fall behind sixteen: 3584x18944 (233 KB)
-// 8.79 / 8.91, 5120x13824 (245 KB) 9.64 / 9.36, 5120x16384 (291 KB) 10.86 / 10.24, x20480 (362 KB) 13.26 / 12.22, 7168x16384
-// 13.75 / 12.78.  The forms cross near 240 KB in such a chain; the line is at 288 KB because a pass that goes from half-SM calls
-// to a whole-SM one pays about 1 us for the change (5120x20480 among three half-SM calls, 36.75 / 36.5).
-// With it a tile costs so little that the short start and the neighbour's full ring win: 3072x32768 (349 KB) 11.84 / 11.90,
-// 4096x20480 (291 KB) 10.47 / 10.87, x28672 (403 KB) 13.22 / 13.45, x30720 (432 KB) 14.04 / 14.20.  4096x32768 (461 KB), 14.69 / 14.83,
-// is the longest range that keeps its pieces; there the forms are within 1 %, and it stays on the other side.  The table fits for
-// K of 1024 to 4096 (multiples of 1024) at one token; at two tokens for 1024 and 2048, whose ranges stay below 288 KB (without
-// it 4096x20480 11.89 / 11.33, 3072x26624 11.90 / 11.25).
+// 4-bit tiles, one token, us per call in a chain of one shape, half SM / whole SM.  Without its activation pieces kept (piece table) a
+// tile costs a half-SM warp its preparation as well, and eight warps fall behind sixteen: 3584x18944 (233 KB) 8.79 / 8.91, 5120x13824
+// (245 KB) 9.64 / 9.36, 5120x16384 (291 KB) 10.86 / 10.24.  The forms cross near 240 KB; the line is at 288 KB because a pass that goes from
+// half-SM calls to a whole-SM one pays about 1 us for the change.  With the table a tile costs so little that the short start
+// and the neighbour's full ring win: 4096x20480 (291 KB) 10.47 / 10.87, x30720 (432 KB) 14.04 / 14.20; 4096x32768 (461 KB), the longest
+// range that keeps its pieces, 14.69 / 14.83, is on the other side.  The table fits for K of 1024 to 4096 at one token, 1024 and
+// 2048 at two.
 constexpr int kGemvFullFromBytesI8W4Kept = 448 * 1024;
 constexpr int kGemvI8FullMaxStages = 8;
 constexpr int kGemvFpW4MaxStages8 = 5, kGemvFpW4MaxStages12 = 6;                              // with 8 and with 12 consumer warps (four groups per tile: 5)
@@ -75,7 +71,7 @@ constexpr int kGemvMaxStages = 48;
 constexpr int kGemvBarrierBytes = 4096;       // 2 x 48 mbarriers + flags, then the chunk tags of the stages
 // A ring stage holds one bulk copy of several contiguous tiles (about 16.6 KB either way) and, on the floating-point path, their
 // activations.  (4-bit tiles, floating-point path: with two tiles per copy the one lane that issues the copies sets the pace, 4
-// tokens 4096x28672 19.0 us against 15.7 with four; with five, six or eight a stage is freed late: 16.0, 15.9, 16.5.)
+// tokens 4096x28672 19.0 us against 15.7 with four when it was chosen; with five, six or eight a stage is freed late: 16.0, 15.9, 16.5.)
 __host__ __device__ constexpr int gemv_chunk_tiles(int bits) { return bits == 4 ? 4 : 2; }
 constexpr int kGemvStageBytes = 17408;        // integer path: 17 x 1024 >= 4 x 4256 and >= 2 x 8320
 constexpr int kGemvMaxM = 16;

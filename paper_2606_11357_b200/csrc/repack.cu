@@ -33,7 +33,7 @@ __device__ __forceinline__ void transpose_bytes(uint32_t r0, uint32_t r1, uint32
 // and words 2w, 2w + 1 of its strip: it reads 8 x 8 bytes, transposes them in registers and writes one word of each of the
 // eight lanes (g, t).  A warp reads 128-byte row segments, so every sector is moved once.  Bound by DRAM: 4096 x 14336 takes 11.4 us
 // in a chain (5.3 TB/s).  Launched as a programmatic dependent, whose CTAs wait for the kernels before it themselves: with a plain
-// launch it was 13.8 us, 1024 x 4096 4.1 (now 2.7).  (Two tiles per CTA: 1 % slower.  One thread per output word, eight 4-byte loads
+// launch it was 13.8 us, 1024 x 4096 4.1 (now 2.1 from a graph).  (Two tiles per CTA: 1 % slower.  One thread per output word, eight 4-byte loads
 // for each: 65.6 us.)  It releases its own dependents only by ending: the GEMV and the GEMM read packed weights before they wait for
 // the kernels ahead of them.
 constexpr int kRepackThreads = 256, kRepackStrips = 4;
