@@ -387,6 +387,11 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
         l.last = owner_of(l.strip * ktiles + ktiles - 1 - cbase);
         return l;
     };
+    // Where this lane's float4 of slice e lies among the 32 of the slice: on the floating-point path the four-column units of a token row are
+    // permuted by the row's pair, because the four threads of a warp that write one column of eight tokens would otherwise meet in a bank: at
+    // the end of a call eight warps write at once, 1024 wavefronts at 16 tokens, 256 this way (16 tokens 4096x1024 4.37 -> 4.00 us,
+    // 4096x28672 18.5 -> 17.6, 4 tokens 4096x1024 3.19 -> 3.07, 4096x14336 8.65 -> 8.42).
+    auto red_lane = [&](int e) { return I8 ? lane : lane ^ (2 * (e & 3)); };
     // One warp's part in it: slice e, from buffer rb in its use ru.  What other CTAs hold of a cut strip is asked for before the wait
     // for this CTA's own sums, by a warp that has nothing else to do (`poll`) again and again.
     auto finish = [&](const Last& l, int e, int rb, int ru, bool poll) {
@@ -405,7 +410,7 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
         }
         if (!mbar_wait_warp(bar, ru & 1, abort_flag, 0x410)) return;
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4* src = reinterpret_cast<const float4*>(red + (size_t)rb * nconsumers * kRedWarp) + 32 * e + lane;
+        const float4* src = reinterpret_cast<const float4*>(red + (size_t)rb * nconsumers * kRedWarp) + 32 * e + red_lane(e);
 #pragma unroll 4
         for (int w = 0; w < nconsumers; ++w) add_to(sum, src[w * (kRedWarp / 4)]);         // fixed order: warp 0 + warp 1 + ...
         if (!l.whole && !finisher) {
@@ -477,9 +482,9 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                 // this slower: 36.7 against 35.7 us over four shapes at 4 tokens.)
 #pragma unroll 4
                 for (int w = 0; w < nconsumers; ++w) {
-                    const float4* src = reinterpret_cast<const float4*>(red + (size_t)(rb * nconsumers + w) * kRedWarp) + lane;
+                    const float4* src = reinterpret_cast<const float4*>(red + (size_t)(rb * nconsumers + w) * kRedWarp);
 #pragma unroll
-                    for (int e = 0; e < kVec; ++e) add_to(sum[e], src[32 * e]);
+                    for (int e = 0; e < kVec; ++e) add_to(sum[e], src[32 * e + red_lane(e)]);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(seg_free0 + 8 * rb);         // consumers may reuse the buffer
@@ -857,10 +862,12 @@ gemv_stream_kernel(const __grid_constant__ GemvActMap<I8> act_map, const uint8_t
                     if (I8 && t != 0) continue;                 // integer path: tokens 0 and 1 sit in the t = 0 threads, the buffer has two rows
                     // (the floating-point path multiplies with codes in 64ths)
                     constexpr float kUnit = I8 ? 1.f : kCodeUnit;
-                    mine[tok * kTileN + 16 * w + g] = kUnit * acc[w][mt][0];
-                    mine[(tok + 1) * kTileN + 16 * w + g] = kUnit * acc[w][mt][1];
-                    mine[tok * kTileN + 16 * w + g + 8] = kUnit * acc[w][mt][2];
-                    mine[(tok + 1) * kTileN + 16 * w + g + 8] = kUnit * acc[w][mt][3];
+                    // rows g and g + 8 of the block; floating-point path: in the order of red_lane
+                    const int lo = I8 ? 16 * w + g : 4 * (4 * w ^ 2 * t) + g, hi = I8 ? lo + 8 : lo ^ 8;
+                    mine[tok * kTileN + lo] = kUnit * acc[w][mt][0];
+                    mine[(tok + 1) * kTileN + lo] = kUnit * acc[w][mt][1];
+                    mine[tok * kTileN + hi] = kUnit * acc[w][mt][2];
+                    mine[(tok + 1) * kTileN + hi] = kUnit * acc[w][mt][3];
                 }
             __syncwarp();
             if (lane == 0) mbar_arrive(seg_full0 + 8 * rb);
