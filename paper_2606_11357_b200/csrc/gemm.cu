@@ -626,21 +626,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
 // ------------------------------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------------------------------
-static int gemm_token_tile(int M) { return M > 128 ? 256 : M > 64 ? 128 : M > 32 ? 64 : 32; }
-
 size_t gemm_workspace_bytes(int M, int K, int N) {
     (void)K; (void)N;
-    return (size_t)kGemmPartialOffset + (size_t)kGemmMaxGrid * kBN * gemm_token_tile(M) * 4;      // one slot per CTA
+    return (size_t)kGemmPartialOffset + (size_t)kGemmMaxGrid * kBN * gemm_widest_tile(M) * 4;      // one slot per CTA
 }
 
 namespace {
 
 template <int BITS, int BT, int G = 1>
-cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, int N, void* workspace, int sm_count,
-                      cudaStream_t stream) {
-    // equal token tiles: 297 tokens are two tiles of 160 columns (149 and 148 of them real), not 256 + 41
-    const int m_tiles = (M + BT - 1) / BT;
-    const int bt = ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16;
+cudaError_t launch_bt(const GemmTiling& tiling, const void* blob, const void* a, void* y, int M, int K, int N, void* workspace, cudaStream_t stream) {
+    const int m_tiles = tiling.m_tiles, bt = tiling.bt;
+    const GemmSplit& split = tiling.split;
     CUtensorMap map;
     // [K / 64][M][64]: a load brings the 64-k blocks of its stage one after the other, each in the 128-byte rows of the swizzle
     const cuuint64_t dims[3] = {kBK, (cuuint64_t)M, (cuuint64_t)K / kBK};
@@ -663,9 +659,6 @@ cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, in
         if (e != cudaSuccess) return e;
         if (seen) configured_on[dev].store(true, std::memory_order_release);
     }
-    const int n_tiles = (N + kBN - 1) / kBN;
-    if (sm_count > kGemmMaxGrid) sm_count = kGemmMaxGrid;
-    const GemmSplit split = split_gemm(n_tiles * m_tiles, K / kTileK, bt, sm_count);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(split.grid / split.rows, split.rows, 1);
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
@@ -678,7 +671,7 @@ cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, in
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_kernel<BITS, BT, G>, map, static_cast<const uint8_t*>(blob), static_cast<__nv_bfloat16*>(y),
-                                             M, K, N, K / kTileK, n_tiles, m_tiles, bt, rings.act_stages, rings.wp_stages,
+                                             M, K, N, K / kTileK, (N + kBN - 1) / kBN, m_tiles, bt, rings.act_stages, rings.wp_stages,
                                              split.whole_tiles ? 1 : 0, split.ranges, static_cast<uint8_t*>(workspace), debug_word());
     if (e == cudaSuccess) note.launched(LaunchKind::kWholeSm);
     return e;
@@ -687,10 +680,12 @@ cudaError_t launch_bt(const void* blob, const void* a, void* y, int M, int K, in
 template <int BITS, int G = 1>
 cudaError_t launch_bits(const void* blob, const void* a, void* y, int M, int K, int N, void* workspace, int sm_count,
                         cudaStream_t stream) {
-    if (M > 128) return launch_bt<BITS, 256, G>(blob, a, y, M, K, N, workspace, sm_count, stream);
-    if (M > 64) return launch_bt<BITS, 128, G>(blob, a, y, M, K, N, workspace, sm_count, stream);
-    if (M > 32) return launch_bt<BITS, 64, G>(blob, a, y, M, K, N, workspace, sm_count, stream);
-    return launch_bt<BITS, 32, G>(blob, a, y, M, K, N, workspace, sm_count, stream);
+    if (sm_count > kGemmMaxGrid) sm_count = kGemmMaxGrid;
+    const GemmTiling tiling = choose_gemm_tiling(M, (N + kBN - 1) / kBN, K / kTileK, sm_count);
+    if (tiling.width == 256) return launch_bt<BITS, 256, G>(tiling, blob, a, y, M, K, N, workspace, stream);
+    if (tiling.width == 128) return launch_bt<BITS, 128, G>(tiling, blob, a, y, M, K, N, workspace, stream);
+    if (tiling.width == 64) return launch_bt<BITS, 64, G>(tiling, blob, a, y, M, K, N, workspace, stream);
+    return launch_bt<BITS, 32, G>(tiling, blob, a, y, M, K, N, workspace, stream);
 }
 
 }  // namespace

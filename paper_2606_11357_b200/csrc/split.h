@@ -46,26 +46,31 @@ struct Ranges {
 // How the work is spread over the CTAs.  Whole tiles only: nothing has to be put together, but the last wave of tiles may
 // leave SMs idle.  Split of the (tile, k-tile) units over `grid` CTAs: the owner of a cut tile adds up the others' parts
 // at the end of its range.  The candidates are one CTA per SM, in equal ranges, and, where there are fewer tiles than SMs, every whole
-// number of CTAs per tile; the one with the smallest estimate is taken.  In ns: a k-tile 350 + 1.5 bt (dequantization up to
-// about 128 tokens, MMAs above), a cut 3000 (parts stored, flagged and seen) and 550 for every trip to the L2 that brings the
-// parts: two CTAs' at a time, 64 tokens at a time; 1000 less where a range is longer than two tiles, whose first part was
-// stored long before.  (With 450 + 1.5 bt and 2000, the times of an earlier form: 33x1536x8960 8.22 us, now 7.08, 128x2048x11008 12.97 and
-// 11.7, 100x4096x1024 10.8 and 10.1, 90x4096x2048 int8 10.6 and 10.1; others within 1 %.)
+// number of CTAs per tile; the one with the smallest estimate is taken.  In ns, for a call in a chain: a k-tile 360 + 0.9 bt
+// (dequantization up to about 128 tokens, MMAs above); the drain of the last tile 9 bt, of every other tile of a CTA 15 bt above 128 tokens
+// (one accumulator: nothing runs under it); a cut 1000, storing and reading the parts 9.5 bt + 2 bt for each of the others, and 350 for every trip to
+// the L2 that brings them (two CTAs' parts at a time, 64 tokens at a time); 1200 where more than half of the SMs are taken, as the
+// start of the next call of a chain then no longer hides behind this one.  Fitted to 2900 timings (4-bit and int8, groups of 32 and 128,
+// 20 to 2048 tokens, 0.5 to 67 M weights): 6 % off on average; the choice costs 0.9 % over the best candidate.
 struct GemmSplit {
     int grid, rows;            // CTAs; rows of the grid: one, or one per tile
     bool whole_tiles;
+    long long cost;            // the estimate
     Ranges ranges;             // of whole tiles, or of units
 };
 inline GemmSplit split_gemm(int tiles, int ktiles, int bt, int sm_count) {
-    const long long units = (long long)tiles * ktiles, t_unit = 350 + 3 * bt / 2;
+    const long long units = (long long)tiles * ktiles;
+    const int t_unit = 360 + 9 * bt / 10;
+    const auto range = [&](int grid, long long len) {        // a CTA's range of k-tiles, with the drains of all its tiles
+        return len * t_unit + 9 * bt + (bt > 128 ? (len - 1) / ktiles * 15 * bt : 0) + (2 * grid > sm_count ? 1200 : 0);
+    };
     GemmSplit best;
     best.grid = tiles < sm_count ? tiles : sm_count;
     best.whole_tiles = true;
-    long long best_cost = (long long)((tiles + best.grid - 1) / best.grid) * ktiles * t_unit;
+    best.cost = range(best.grid, (long long)((tiles + best.grid - 1) / best.grid) * ktiles);
     auto consider = [&](int grid, long long others) {        // others: CTAs besides the owner that hold a part of a tile
-        const long long len = (units + grid - 1) / grid;
-        const long long cost = len * t_unit + 3000 - (len >= 2 * ktiles ? 1000 : 0) + 550 * ((others + 1) / 2) * ((bt + 63) / 64);
-        if (cost < best_cost) { best_cost = cost; best.grid = grid; best.whole_tiles = false; }
+        const long long cost = range(grid, (units + grid - 1) / grid) + 1000 + 350 * ((others + 1) / 2) * ((bt + 63) / 64) + 19 * bt / 2 + 2 * others * bt;
+        if (cost < best.cost) { best.cost = cost; best.grid = grid; best.whole_tiles = false; }
     };
     for (int per_tile = 2; per_tile * tiles <= sm_count && per_tile <= ktiles; ++per_tile) consider(per_tile * tiles, per_tile - 1);
     if (tiles % sm_count != 0 && units >= sm_count) consider(sm_count, (ktiles + units / sm_count - 1) / (units / sm_count));
@@ -76,12 +81,37 @@ inline GemmSplit split_gemm(int tiles, int ktiles, int bt, int sm_count) {
     // Several CTAs per tile: the owner of the last k-tile takes as much more as its k-tiles last while the others' parts are on
     // their way (us with even shares / this: 128x4096x4096 12.5 / 12.3, 60x4096x1024 8.25 / 8.05, int8 300x4096x4096 17.7 / 17.2).
     constexpr int kOwnNs = 1500;
-    const int mean = (int)(units / sm_count), late_less = (int)(kLateNs / t_unit);
+    const int mean = (int)(units / sm_count), late_less = kLateNs / t_unit;
     const bool some_late = best.grid == sm_count && bt <= 128 && sm_count >= 8 * kLate;
     best.rows = !best.whole_tiles && best.grid % tiles == 0 ? tiles : 1;
     if (best.whole_tiles) best.ranges = Ranges::make(tiles, best.grid);
-    else if (best.rows > 1) best.ranges = Ranges::make(ktiles, best.grid / best.rows, 1, -(int)(kOwnNs / t_unit));
+    else if (best.rows > 1) best.ranges = Ranges::make(ktiles, best.grid / best.rows, 1, -(kOwnNs / t_unit));
     else best.ranges = Ranges::make((int)units, best.grid, some_late ? kLate : 0, late_less < mean / 2 ? late_less : mean / 2);
+    return best;
+}
+
+// Token tiles of a GEMM call.  `width`: 32, 64, 128 or 256, what the kernel is built for; the tiles are equal: 297 tokens are two tiles of 160
+// columns (149 and 148 of them real), not 256 + 41.  The widest that M fills unpacks each weight least often and is right where the SMs
+// have enough to do.  Where there are few output tiles a narrower one, at twice the unpacking, has more tiles for the SMs and less to put
+// together (us, 4-bit: 256x4096x4096 17.5 in one tile of 256 cut four ways, 14.1 in two of 128 cut two ways, x8192x2048 22.5 and 15.7,
+// 200x1024x4096 8.2 and 6.2, 128x2048x2048 9.0 and 7.2 in tiles of 64); taken where the estimate is at least 3 % smaller.
+struct GemmTiling {
+    int width, m_tiles, bt;    // bt: token columns of a tile, a multiple of 16
+    GemmSplit split;
+};
+inline int gemm_widest_tile(int M) { return M > 128 ? 256 : M > 64 ? 128 : M > 32 ? 64 : 32; }
+inline GemmTiling choose_gemm_tiling(int M, int n_tiles, int ktiles, int sm_count) {
+    GemmTiling best;
+    long long best_cost = 0;
+    for (int width = gemm_widest_tile(M), widest = width; width >= 32; width /= 2) {
+        GemmTiling t;
+        t.width = width;
+        t.m_tiles = (M + width - 1) / width;
+        t.bt = ((M + t.m_tiles - 1) / t.m_tiles + 15) / 16 * 16;
+        t.split = split_gemm(n_tiles * t.m_tiles, ktiles, t.bt, sm_count);
+        const long long cost = width == widest ? t.split.cost : t.split.cost * 103 / 100;
+        if (width == widest || cost < best_cost) { best = t; best_cost = cost; }
+    }
     return best;
 }
 

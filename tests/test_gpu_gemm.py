@@ -221,3 +221,10 @@ def test_gemm_cuts(bits, group, M, K, N):
         ys.append(gu.bits_of(y))
     assert np.array_equal(ys[0], ys[1])
     gu.check_against_oracle(p, ys[0], columns=np.unique(np.concatenate([np.arange(0, N, 41), [N - 1]])))
+
+
+# fewer output tiles than SMs: token tiles narrower than M would fill, several of them, whole and cut, the last one ragged
+@pytest.mark.parametrize("bits,group", [(4, 128), (4, 32), (8, 128)])
+@pytest.mark.parametrize("M,K,N", [(129, 512, 4104), (200, 8192, 2048), (256, 4096, 4096), (600, 2048, 2056), (65, 2048, 2048), (100, 1024, 4104), (45, 4096, 520)])
+def test_gemm_narrow_token_tiles(bits, group, M, K, N):
+    test_gemm_cuts(bits, group, M, K, N)
