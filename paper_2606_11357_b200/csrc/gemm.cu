@@ -33,6 +33,12 @@
 // for short calls the 4 to 5 us around them.  us per call in a chain: 32x4096x18944 17.9, 96x2944x11016 13.9, 297x2944x11016 26.1,
 // int8 1024x4096x4096 28.2, 512x4096x4096 20.5.  (With eight dequant warps on one k-tile at a time, a packed ring of 26 KB and partial
 // sums through an arrival counter a k-tile took 0.61 to 0.83 us and these calls 24.1, 18.9, 33.5, 32.9 and 31.1.)
+// Pairs of CTAs (PAIR): two CTAs of a cluster, on neighbouring SMs, share an output tile of 256 columns x bt tokens.  One MMA of 256 rows
+// (cta_group::2) works on both halves, so each SM loads and holds only half of the activations.  A CTA on its own is bound by what its SM can
+// take from the L2: 64 KB of activations and 8.5 KB of weights per k-tile of 256 tokens, 62 bytes per cycle at 1195 cycles; a pair takes 41 KB and
+// 1100 cycles, and moves fewer bytes, which under the power limit is worth as much: us, 2048x4096x14336 203.9 -> 193.6, 512x32768x4096
+// 119.6 -> 116.5, 1024x4096x8584 59.6 -> 53.9.  Each CTA unpacks and drains its own 128 columns; CTA 0 issues the MMAs, and the barriers that its MMA
+// warp waits on are arrived at by both (choose_gemm_tiling says when).
 // Every mbarrier wait is bounded; on a timeout all roles leave, TMEM is freed, the status word is set.
 #include <cuda.h>
 
@@ -79,10 +85,10 @@ constexpr int kGemmSmemFixed = 1024 /*alignment slack*/ + 4 * kGroups * kDrainWa
 struct GemmRings {
     int act_stage_bytes, act_stages, wp_stages, smem_bytes;
 };
-inline GemmRings gemm_rings(int bits, int BT, int bt, int G) {
+inline GemmRings gemm_rings(int bits, int BT, int act_rows, int G) {
     GemmRings r;
     const int left = kGemmSmemMax - kGemmSmemFixed, wp = wp_stage_bytes(bits, BT, G), round = kGroups / chunk_tiles(bits, BT);
-    r.act_stage_bytes = bt * act_stage_k(BT) * 2;
+    r.act_stage_bytes = act_rows * act_stage_k(BT) * 2;
     if (tied(BT)) {
         r.act_stages = kGroups;
         r.wp_stages = (left - r.act_stages * r.act_stage_bytes) / wp / round * round;
@@ -264,7 +270,7 @@ __device__ __forceinline__ uint32_t times_scale(uint32_t d, uint32_t hi2, uint32
 // G = groups per tile: 1 for group sizes that are multiples of 128, 2 / 4 for the 4-bit group sizes 64 / 32.
 // BT = the widest token tile of the instantiation (it sizes the rings); bt = the token columns of this call's tiles, a
 // multiple of 16.
-template <int BITS, int BT, int G = 1>
+template <int BITS, int BT, int G, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restrict__ blob,
             __nv_bfloat16* __restrict__ y, int M, int K, int N, int ktiles, int n_tiles, int m_tiles, int bt, int act_stages,
@@ -278,7 +284,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
     constexpr int kAccs = BT > 128 ? 1 : 2;               // accumulators in tensor memory: where two fit, the next tile's MMAs run under a drain
     constexpr int kActK = act_stage_k(BT);
     constexpr bool kTied = tied(BT);
-    const int act_stage = bt * kActK * 2;                // bytes, a multiple of 1024 (bt is one of 16)
+    static_assert(!PAIR || !kTied, "pairs of CTAs: the widest token tile only");
+    // PAIR: this CTA is one of two that share an output tile of 256 columns; each has 128 of them and loads half of the token rows
+    const int rank = PAIR ? (int)cta_rank_in_cluster() : 0;
+    const int act_rows = PAIR ? bt / 2 : bt;             // token rows of a stage
+    const int act_stage = act_rows * kActK * 2;          // bytes, a multiple of 1024 (act_rows is one of 16)
     constexpr size_t kSlotVec = (size_t)kBN * BT / 4;     // float4 of a CTA's slot
 
     extern __shared__ uint8_t smem_raw[];
@@ -293,14 +303,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     // unit = (output tile, k-tile of 128); aligned: ranges of whole tiles (no tile is shared between CTAs)
     // Several CTAs per tile: the grid has a row of CTAs per tile, which share its k-tiles.  Otherwise it has one row.
-    const int cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const int u_begin = ranges.start(blockIdx.x) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
-    const int u_end = ranges.start(blockIdx.x + 1) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
+    // (pairs: all of this counts pairs, and a pair's CTAs do the same in step)
+    const int gx = blockIdx.x / (PAIR ? 2 : 1), gridx = gridDim.x / (PAIR ? 2 : 1);
+    const int cta = blockIdx.y * gridx + gx;
+    const int u_begin = ranges.start(gx) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
+    const int u_end = ranges.start(gx + 1) * (aligned ? ktiles : 1) + blockIdx.y * ktiles;
     const Segments segs(u_begin, u_end, ktiles);
     const int strips = (N + kTileN - 1) / kTileN;
     HeaderWords header(blob);
     DeviceStatus* status = reinterpret_cast<DeviceStatus*>(workspace);
-    float4* slots = reinterpret_cast<float4*>(workspace + kGemmPartialOffset);
+    float4* slots = reinterpret_cast<float4*>(workspace + kGemmPartialOffset) + (PAIR ? rank * kSlotVec : 0);
+    constexpr size_t kSlotStride = (PAIR ? 2 : 1) * kSlotVec;            // from one CTA's slot to that of the next with the same columns
+    const auto first_strip = [&](int tile) { return PAIR ? 4 * (tile / m_tiles) + 2 * rank : 2 * (tile / m_tiles); };
 
     // Producer W: packed weight tiles (weights + scales + zeros in one payload), the chunks [from, to) of the CTA's range.  The first
     // wp_stages chunks find their stages free.
@@ -310,8 +324,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
         for (int i = 0; i < segs.count; ++i) {
             int tile, kt0, len;
             segs.get(i, tile, kt0, len);
-            const int strip0 = 2 * (tile / m_tiles);
-            const bool two = strip0 + 1 < strips;
+            const int strip0 = first_strip(tile);
+            const bool one = !PAIR || strip0 < strips, two = strip0 + 1 < strips;
             const uint8_t* src = blob + kHeaderBytes + ((size_t)strip0 * ktiles + kt0) * kTileBytes;
             for (int T = 0; T < len; T += kChunk, src += kChunk * kTileBytes, ++n) {
                 if (n >= to) return;
@@ -319,8 +333,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                     if (n >= wp_stages && !mbar_wait(smem_u32(&bars->wp_empty[s]), parity, abort_flag, 0x300 + s)) return;
                     const uint32_t bar = smem_u32(&bars->wp_full[s]), dst = smem_u32(wp_ring + s * kWpStageBytes);
                     const uint32_t bytes = min(kChunk, len - T) * kTileBytes;
-                    mbar_arrive_expect_tx(bar, two ? 2 * bytes : bytes);
-                    bulk_copy_g2s(dst, src, bytes, bar);
+                    mbar_arrive_expect_tx(bar, two ? 2 * bytes : one ? bytes : 0);
+                    if (one) bulk_copy_g2s(dst, src, bytes, bar);
                     if (two) bulk_copy_g2s(dst + kChunk * kTileBytes, src + (size_t)ktiles * kTileBytes, bytes, bar);
                 }
                 if (++s == wp_stages) { s = 0; parity ^= 1u; }
@@ -346,12 +360,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
         mbar_init_fence();
         if (header.fit(BITS, (uint32_t)K, (uint32_t)N, G) && !drop_weights) produce_weights(0, early_chunks);
     } else if (threadIdx.x >= 32 && threadIdx.x < 32 + kGroups) {
-        mbar_init(smem_u32(&bars->op_full[threadIdx.x - 32]), kTied ? 5 : 4);
+        mbar_init(smem_u32(&bars->op_full[threadIdx.x - 32]), kTied ? 5 : PAIR ? 8 : 4);
         mbar_init(smem_u32(&bars->op_done[threadIdx.x - 32]), 1);
         mbar_init_fence();
     } else if (threadIdx.x >= 128 && threadIdx.x < 128 + kAccs) {
         mbar_init(smem_u32(&bars->acc_full[threadIdx.x - 128]), 1);
-        mbar_init(smem_u32(&bars->acc_empty[threadIdx.x - 128]), 4 * kGroups);      // every dequant warp has drained its share
+        mbar_init(smem_u32(&bars->acc_empty[threadIdx.x - 128]), (PAIR ? 8 : 4) * kGroups);      // every dequant warp has drained its share
         mbar_init_fence();
     } else if (threadIdx.x == 160) {
         bars->abort_flag = 0;
@@ -359,11 +373,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
         mbar_init_fence();
     }
     if (warp == 2) {
-        tmem_alloc(smem_u32(&bars->tmem_base), kTmemCols);
-        tmem_relinquish();
+        if constexpr (PAIR) {
+            tmem_alloc_pair(smem_u32(&bars->tmem_base), kTmemCols);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(smem_u32(&bars->tmem_base), kTmemCols);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();             // the barriers of both CTAs are ready
     tc_fence_after();
     const bool header_ok = header.fit(BITS, (uint32_t)K, (uint32_t)N, G);
     // The next kernel of the stream may start as SMs become free: its set-up and its first weights then run under the last
@@ -387,14 +407,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
             for (int i = 0; i < segs.count && ok; ++i) {
                 int tile, kt0, len;
                 segs.get(i, tile, kt0, len);
-                const int token0 = tile % m_tiles * bt;
+                const int token0 = tile % m_tiles * bt + rank * act_rows;
                 for (int T = 0; T < len * (kTileK / kActK); ++T) {
                     if (kTied) s = s0 + T % kChunk;
                     ok = mbar_wait(smem_u32(kTied ? &bars->op_done[s] : &bars->act_empty[s]), kTied ? (parity >> s) & 1u : parity, abort_flag, 0x310 + s);
                     if (!ok) break;
                     const uint32_t bar = smem_u32(kTied ? &bars->op_full[s] : &bars->act_full[s]);
-                    mbar_arrive_expect_tx(bar, bt * kActK * 2);
-                    tma_load_3d(smem_u32(act_ring + s * act_stage), &act_map, 0, token0, (2 * kt0 * kBK + T * kActK) / kBK, bar);
+                    const int z = (2 * kt0 * kBK + T * kActK) / kBK;
+                    if constexpr (PAIR) {               // both halves are counted by the barrier of the CTA that issues the MMAs
+                        if (rank == 0) mbar_arrive_expect_tx(bar, 2 * act_stage);
+                        tma_load_3d_pair(smem_u32(act_ring + s * act_stage), &act_map, 0, token0, z, map_to_cta(bar, 0));
+                    } else {
+                        mbar_arrive_expect_tx(bar, act_stage);
+                        tma_load_3d(smem_u32(act_ring + s * act_stage), &act_map, 0, token0, z, bar);
+                    }
                     if (kTied) {
                         parity ^= 1u << s;
                         if (T % kChunk == kChunk - 1 || T == len - 1) s0 = (s0 + kChunk) % kGroups;
@@ -403,9 +429,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
             }
         } else if (warp == 3 && lane == 0) {
             if (!drop_weights) produce_weights(early_chunks, 1 << 30);
-        } else if (warp == 1) {
+        } else if (warp == 1 && rank == 0) {
             // ================= MMA issuer: one elected lane of the converged warp =================================
-            const uint32_t idesc = umma_idesc_bf16(kBN, bt);
+            const uint32_t idesc = umma_idesc_bf16(PAIR ? 2 * kBN : kBN, bt);
+            const auto commit = [](uint32_t bar) { PAIR ? tc_commit_pair(bar) : tc_commit(bar); };
+            const auto wait = [&](uint64_t* bar, uint32_t parity, uint32_t site) {
+                return PAIR ? mbar_wait_warp_cluster(smem_u32(bar), parity, abort_flag, site) : mbar_wait_warp(smem_u32(bar), parity, abort_flag, site);
+            };
             int s0 = 0, as = 0;                               // the chunk's first operand stage (= group)
             uint32_t parity = 0, aparity = 0;                 // bit s of `parity`: operand stage s
             bool ok = true;
@@ -414,15 +444,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                 segs.get(i, tile, kt0, len);
                 const int acc = i % kAccs;
                 const uint32_t d = tmem_base + acc * (kTmemAccCols / kAccs);
-                ok = mbar_wait_warp(smem_u32(&bars->acc_empty[acc]), (i / kAccs & 1) ^ 1, abort_flag, 0x400);
+                ok = wait(&bars->acc_empty[acc], (i / kAccs & 1) ^ 1, 0x400);
                 tc_fence_after();
                 for (int T = 0; T < len && ok; ++T) {
                     const int s = s0 + T % kChunk;
-                    ok = mbar_wait_warp(smem_u32(&bars->op_full[s]), (parity >> s) & 1u, abort_flag, 0x410 + s);
+                    ok = wait(&bars->op_full[s], (parity >> s) & 1u, 0x410 + s);
                     parity ^= 1u << s;
 #pragma unroll
                     for (int part = 0; part < kTileK / kActK; ++part) {
-                        if (!kTied) ok = ok && mbar_wait_warp(smem_u32(&bars->act_full[as]), aparity, abort_flag, 0x420 + as);
+                        if (!kTied) ok = ok && wait(&bars->act_full[as], aparity, 0x420 + as);
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t b_desc = umma_desc_k_sw128(smem_u32(act_ring + (kTied ? s : as) * act_stage));
@@ -430,9 +460,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                         if (elect_one()) {
 #pragma unroll
                             for (int j = 0; j < kActK / 16; ++j)   // 16 k per instruction: 8 TMEM columns / 32 smem bytes
-                                tc_mma_f16_tmem_a(d, a + 8 * j, b_desc + 2 * (j & 3) + (j >> 2) * (bt * kBK * 2 / 16), idesc, (T | part | j) != 0 ? 1u : 0u);
-                            if (!kTied) tc_commit(smem_u32(&bars->act_empty[as]));
-                            if (part == kTileK / kActK - 1) tc_commit(smem_u32(&bars->op_done[s]));
+                                if constexpr (PAIR) tc_mma_f16_tmem_a_pair(d, a + 8 * j, b_desc + 2 * (j & 3), idesc, (T | part | j) != 0 ? 1u : 0u);
+                                else tc_mma_f16_tmem_a(d, a + 8 * j, b_desc + 2 * (j & 3) + (j >> 2) * (bt * kBK * 2 / 16), idesc, (T | part | j) != 0 ? 1u : 0u);
+                            if (!kTied) commit(smem_u32(&bars->act_empty[as]));
+                            if (part == kTileK / kActK - 1) commit(smem_u32(&bars->op_done[s]));
                         }
                         __syncwarp();
                         if (!kTied && ++as == act_stages) { as = 0; aparity ^= 1u; }
@@ -440,7 +471,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                     if (T % kChunk == kChunk - 1 || T == len - 1) s0 = (s0 + kChunk) % kGroups;
                 }
                 if (!ok) break;
-                if (elect_one()) tc_commit(smem_u32(&bars->acc_full[acc]));
+                if (elect_one()) commit(smem_u32(&bars->acc_full[acc]));
                 __syncwarp();
             }
         } else if (warp >= kFirstDequant) {
@@ -470,6 +501,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
             int duty = 0, last_seg = 0;
             DrainShare share;
             share.part = group; share.lane = lane; share.chunks = bt / 8;
+            // arrivals on the barriers of the CTA that issues the MMAs
+            const auto arrive_issuer = [&](uint64_t* bar) {
+                if constexpr (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(bar), 0));
+                else mbar_arrive(smem_u32(bar));
+            };
             share.tbuf = drain_buf + (warp - kFirstDequant) * kDrainWarpBytes;
             auto do_duty = [&](int sidx) -> bool {
                 const int acc = sidx % kAccs;
@@ -477,18 +513,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                 tc_fence_after();
                 int dtile, dkt0, dlen;
                 segs.get(sidx, dtile, dkt0, dlen);
-                const int n0 = dtile / m_tiles * kBN + 32 * q, token0 = dtile % m_tiles * bt;
+                const int n0 = first_strip(dtile) * kTileN + 32 * q, token0 = dtile % m_tiles * bt;
                 share.tmem = tmem_base + acc * (kTmemAccCols / kAccs) + quarter;
                 if (!waited) { grid_dependency_wait(); waited = true; }        // y and the workspace belong to earlier kernels until now
                 if (dkt0 + dlen != ktiles) {
                     // the owner's warp of the same number takes what this one stores, so each pair has a flag of its own
-                    share.contribute(slots + cta * kSlotVec, q);
+                    share.contribute(slots + cta * kSlotStride, q);
                     __syncwarp();
-                    if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + cta * 4 * kGroups), "r"(1u) : "memory");
+                    if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + (PAIR ? 2 * cta + rank : cta) * 4 * kGroups), "r"(1u) : "memory");
                 } else if (dkt0 != 0) {
-                    const int first = gridDim.y > 1 ? dtile * gridDim.x : ranges.owner(dtile * ktiles), others = cta - first;
+                    const int first = gridDim.y > 1 ? dtile * gridx : ranges.owner(dtile * ktiles), others = cta - first;
                     for (int o = 0; o < others; o += 32) {              // a lane per contributor
-                        uint32_t* flag = flags + (first + o + lane) * 4 * kGroups;
+                        uint32_t* flag = flags + (PAIR ? 2 * (first + o + lane) + rank : first + o + lane) * 4 * kGroups;
                         const bool mine = o + lane < others;
                         const long long t_begin = clock64();
                         for (;;) {
@@ -500,19 +536,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                         if (mine) *flag = 0;                            // zero for the next call
                     }
                     __syncwarp();
-                    share.finish(slots + first * kSlotVec, kSlotVec, others, q, y, M, N, n0, token0);
+                    share.finish(slots + first * kSlotStride, kSlotStride, others, q, y, M, N, n0, token0);
                 } else {
                     share.whole(y, M, N, n0, token0);
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bars->acc_empty[acc]));
+                if (lane == 0) arrive_issuer(&bars->acc_empty[acc]);
                 return true;
             };
             for (int i = 0; i < segs.count && ok; ++i) {
                 int tile, kt0, len;
                 segs.get(i, tile, kt0, len);
-                const bool strip_exists = 2 * (tile / m_tiles) + strip_sel < strips;
+                const bool strip_exists = first_strip(tile) + strip_sel < strips;
                 int T = behind * kChunk;
                 for (; T < len && ok; T += kRound * kChunk) {
                     auto release_stage = [&]() {
@@ -599,7 +635,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars->op_full[group]));
+                    if (lane == 0) arrive_issuer(&bars->op_full[group]);
                 }
                 behind = (T - (len + kChunk - 1) / kChunk * kChunk) / kChunk;
             }
@@ -613,7 +649,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
     __syncthreads();
     if (threadIdx.x == 0) {
         if (!header_ok) {
-            if (cta == 0) { status->code = TF_ERR_BLOB; status->detail = 1; }
+            if (cta == 0 && rank == 0) { status->code = TF_ERR_BLOB; status->detail = 1; }
         } else if (bars->abort_flag != 0) {
             status->code = TF_ERR_TIMEOUT;
             status->detail = bars->abort_flag;
@@ -622,9 +658,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
         }
     }
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();             // nobody touches the other CTA's memory any more (every wait above is bounded)
     if (warp == 2) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
+        else tmem_dealloc(tmem_base, kTmemCols);
     }
 }
 
@@ -638,7 +676,7 @@ size_t gemm_workspace_bytes(int M, int K, int N) {
 
 namespace {
 
-template <int BITS, int BT, int G = 1>
+template <int BITS, int BT, int G, bool PAIR = false>
 cudaError_t launch_bt(const GemmTiling& tiling, const void* blob, const void* a, void* y, int M, int K, int N, void* workspace, cudaStream_t stream) {
     const int m_tiles = tiling.m_tiles, bt = tiling.bt;
     const GemmSplit& split = tiling.split;
@@ -646,11 +684,12 @@ cudaError_t launch_bt(const GemmTiling& tiling, const void* blob, const void* a,
     // [K / 64][M][64]: a load brings the 64-k blocks of its stage one after the other, each in the 128-byte rows of the swizzle
     const cuuint64_t dims[3] = {kBK, (cuuint64_t)M, (cuuint64_t)K / kBK};
     const cuuint64_t strides[2] = {(cuuint64_t)K * 2, kBK * 2};
-    const cuuint32_t box[3] = {kBK, (cuuint32_t)bt, (cuuint32_t)(act_stage_k(BT) / kBK)};
+    const int act_rows = PAIR ? bt / 2 : bt;
+    const cuuint32_t box[3] = {kBK, (cuuint32_t)act_rows, (cuuint32_t)(act_stage_k(BT) / kBK)};
     cudaError_t me = encode_bf16_map(&map, a, 3, dims, strides, box);
     if (me != cudaSuccess) return me;
 
-    const GemmRings rings = gemm_rings(BITS, BT, bt, G);
+    const GemmRings rings = gemm_rings(BITS, BT, act_rows, G);
     // function attributes belong to one device: set them once per device and kernel (twice is harmless)
     constexpr int kMaxDevices = 64;
     // (an atomic flag: two host threads may both find it unset and both set the attribute, which is harmless)
@@ -659,23 +698,25 @@ cudaError_t launch_bt(const GemmTiling& tiling, const void* blob, const void* a,
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     const bool seen = dev >= 0 && dev < kMaxDevices;
     if (!seen || !configured_on[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_kernel<BITS, BT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(gemm_kernel<BITS, BT, G, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kGemmSmemMax);
         if (e != cudaSuccess) return e;
         if (seen) configured_on[dev].store(true, std::memory_order_release);
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(split.grid / split.rows, split.rows, 1);
+    cfg.gridDim = dim3(split.grid / split.rows * (PAIR ? 2 : 1), split.rows, 1);
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
     cfg.dynamicSmemBytes = rings.smem_bytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see grid_dependency_wait() in the kernel
     const StreamNote note(stream);
     attr[0].val.programmaticStreamSerializationAllowed = note.may_start_early() ? 1 : 0;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_kernel<BITS, BT, G>, map, static_cast<const uint8_t*>(blob), static_cast<__nv_bfloat16*>(y),
+    cfg.numAttrs = PAIR ? 2 : 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_kernel<BITS, BT, G, PAIR>, map, static_cast<const uint8_t*>(blob), static_cast<__nv_bfloat16*>(y),
                                              M, K, N, K / kTileK, (N + kBN - 1) / kBN, m_tiles, bt, rings.act_stages, rings.wp_stages,
                                              split.whole_tiles ? 1 : 0, split.ranges, static_cast<uint8_t*>(workspace), debug_word());
     if (e == cudaSuccess) note.launched(LaunchKind::kWholeSm);
@@ -687,6 +728,7 @@ cudaError_t launch_bits(const void* blob, const void* a, void* y, int M, int K, 
                         cudaStream_t stream) {
     if (sm_count > kGemmMaxGrid) sm_count = kGemmMaxGrid;
     const GemmTiling tiling = choose_gemm_tiling(M, (N + kBN - 1) / kBN, K / kTileK, sm_count);
+    if (tiling.pair) return launch_bt<BITS, 256, G, true>(tiling, blob, a, y, M, K, N, workspace, stream);
     if (tiling.width == 256) return launch_bt<BITS, 256, G>(tiling, blob, a, y, M, K, N, workspace, stream);
     if (tiling.width == 128) return launch_bt<BITS, 128, G>(tiling, blob, a, y, M, K, N, workspace, stream);
     if (tiling.width == 64) return launch_bt<BITS, 64, G>(tiling, blob, a, y, M, K, N, workspace, stream);

@@ -98,3 +98,9 @@ def test_short_limit_alone_changes_nothing():
 
 def test_debug_inject_rejects_out_of_range():
     assert tf.lib().tf_debug_inject(1 << 24, 0) == 2
+
+
+def test_waits_run_out_in_a_pair_of_ctas():
+    """Whichever CTA of a pair gives up first, both reach their end and the next call is right."""
+    test_bounded_wait_runs_out_and_the_library_recovers("gemm", 4, 1000, 4096, 4104)
+    test_waits_that_run_out_while_the_data_arrives("gemm", 4, 1000, 4096, 4104)

@@ -228,3 +228,10 @@ def test_gemm_cuts(bits, group, M, K, N):
 @pytest.mark.parametrize("M,K,N", [(129, 512, 4104), (200, 8192, 2048), (256, 4096, 4096), (600, 2048, 2056), (65, 2048, 2048), (100, 1024, 4104), (45, 4096, 520)])
 def test_gemm_narrow_token_tiles(bits, group, M, K, N):
     test_gemm_cuts(bits, group, M, K, N)
+
+
+# pairs of CTAs: whole tiles and tiles cut between pairs, in equal ranges and in rows, with a pair whose second half has no columns, ragged columns and tokens
+@pytest.mark.parametrize("bits,group", [(4, 128), (4, 64), (4, 32), (8, 128)])
+@pytest.mark.parametrize("M,K,N", [(1000, 4096, 4104), (300, 4096, 11016), (256, 32768, 2184)])
+def test_gemm_pairs_of_ctas(bits, group, M, K, N):
+    test_gemm_cuts(bits, group, M, K, N)

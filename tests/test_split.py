@@ -58,10 +58,10 @@ CASES = {
                 for (int n_tiles : {1, 2, 9, 32, 87, 256})
                     for (int M = 1; M <= 4096; M += M < 300 ? 1 : 61) {
                         const GemmTiling t = choose_gemm_tiling(M, n_tiles, ktiles, sms);
-                        const int tiles = n_tiles * t.m_tiles;
+                        const int tiles = (t.pair ? (n_tiles + 1) / 2 : n_tiles) * t.m_tiles;
                         // a kernel that exists, a slot that the workspace has room for, every token in a tile and no tile without one
                         bool ok = t.width <= gemm_widest_tile(M) && (t.width == 32 || t.width == 64 || t.width == 128 || t.width == 256);
-                        ok = ok && t.bt % 16 == 0 && t.bt >= 16 && t.bt <= t.width && t.bt * t.m_tiles >= M && t.bt * (t.m_tiles - 1) < M;
+                        ok = ok && t.bt % (t.pair ? 32 : 16) == 0 && (!t.pair || (t.width == 256 && 2 * t.split.grid <= sms)) && t.bt >= 16 && t.bt <= t.width && t.bt * t.m_tiles >= M && t.bt * (t.m_tiles - 1) < M;
                         if (t.split.whole_tiles) ok = ok && sound(t.split.ranges, tiles, t.split.grid);
                         else if (t.split.rows > 1) ok = ok && t.split.rows == tiles && sound(t.split.ranges, ktiles, t.split.grid / t.split.rows);
                         else ok = ok && sound(t.split.ranges, tiles * ktiles, t.split.grid);
