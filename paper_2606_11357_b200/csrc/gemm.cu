@@ -77,7 +77,7 @@ __host__ __device__ constexpr int wp_stage_bytes(int bits, int bt, int G) { retu
 __host__ __device__ constexpr bool tied(int bt) { return bt <= 128; }
 __host__ __device__ constexpr int act_stage_k(int bt) { return tied(bt) ? kTileK : kBK; }
 constexpr int kGemmSmemMax = 227 * 1024;  // dynamic shared memory one CTA may ask for
-constexpr int kDrainWarpBytes = 512;      // per dequant warp: 8 tokens x 32 columns of bf16, for the drain of an accumulator
+constexpr int kDrainWarpBytes = 1024;     // per dequant warp: 16 tokens x 32 columns of bf16, for the drain of an accumulator
 constexpr int kGemmBarrierBytes = 1024;
 constexpr int kGemmSmemFixed = 1024 /*alignment slack*/ + 4 * kGroups * kDrainWarpBytes + kGemmBarrierBytes;
 // The rings share what the fixed part leaves: the activations (of the call's own bt columns) come first where they are tied;
@@ -148,100 +148,107 @@ static_assert(sizeof(GemmBarriers) <= kGemmBarrierBytes, "barrier block");
 
 static_assert(offsetof(GemmBarriers, wait_kcycles) == offsetof(GemmBarriers, abort_flag) + 4, "mbar_wait reads the limit behind the flag");
 
-// What a dequant warp does with its share of a segment's accumulator: the 8-token chunks `part`, `part + 4`, ... of its lane
-// quarter.  A chunk is read in the fragment layout of 8 x 8 matrices (thread (g, t): of columns 8i + g, i = 0..3, the
-// tokens 2t and 2t + 1), the next one being on its way out of tensor memory meanwhile.
+// What a dequant warp does with its share of a segment's accumulator: the chunks `part`, `part + 4`, ... of its lane quarter, of 8 MATS
+// tokens each: 16, or 8 where that is what gives every group of warps a chunk (32 tokens).  A chunk is read in the fragment layout of 8 x 8
+// matrices (see tmem_ld_16x256b), the next one being on its way out of tensor memory meanwhile.  No MMA runs on a tile of 256 tokens until
+// it is empty, so what counts is the chain of latencies of a chunk, and how few chunks there are (with 8 tokens a tile of 256 took 3700
+// cycles, with 16 2900; a part of a cut one is bound by the L2, 128 KB of every CTA's in 5000 cycles).
+template <int MATS>
 struct DrainShare {
     uint32_t tmem;             // accumulator, this lane quarter
-    int part, lane, chunks;    // chunks = bt / 8
-    uint8_t* tbuf;             // 512 bytes of this warp
+    int part, lane, chunks;    // chunks = bt / (8 MATS)
+    uint8_t* tbuf;             // 512 MATS bytes of this warp
 
-    // Rounds a chunk and stores it.  y wants a token's columns side by side: the four matrices are transposed by one stmatrix
-    // through 512 bytes and stored as 16 bytes per lane, 8 columns of one token.
-    __device__ __forceinline__ void store(const float (&v)[8], __nv_bfloat16* y, int M, int N, int n0, int token0) const {
-        const int n8 = n0 + 8 * (lane & 3), tl = lane >> 2, tok = token0 + tl;
-        uint32_t m[4];
+    // A chunk rounded: matrix i of its eight columns c in m[c][i].
+    __device__ __forceinline__ static void round(const float (&v)[8 * MATS], uint32_t (&m)[MATS][4]) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) m[i] = pack_bf16(kCodeUnit * v[2 * i], kCodeUnit * v[2 * i + 1]);      // the operand holds weights in 64ths
-        stmatrix_x4_trans(smem_u32(tbuf) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane & 7) >> 1)) & 3) * 16, m);
+        for (int c = 0; c < MATS; ++c)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {       // the operand holds weights in 64ths
+                const int r = 4 * MATS * (i >> 1) + 4 * c + 2 * (i & 1);
+                m[c][i] = pack_bf16(kCodeUnit * v[r], kCodeUnit * v[r + 1]);
+            }
+    }
+    // ... and stored.  y wants a token's columns side by side: the matrices are transposed by stmatrix and stored as 16 bytes per lane,
+    // 8 columns of one token.
+    __device__ __forceinline__ void store(const uint32_t (&m)[MATS][4], __nv_bfloat16* y, int M, int N, int n0, int token0) const {
+        const int n8 = n0 + 8 * (lane & 3), tl = lane >> 2;
+        const uint32_t put = smem_u32(tbuf) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane & 7) >> 1)) & 3) * 16;
+#pragma unroll
+        for (int c = 0; c < MATS; ++c) stmatrix_x4_trans(put + 512 * c, m[c]);
         __syncwarp();
-        const uint4 d = *reinterpret_cast<const uint4*>(tbuf + tl * 64 + (((lane & 3) ^ (tl >> 1)) & 3) * 16);
-        if (tok < M && n8 < N) *reinterpret_cast<uint4*>(y + (size_t)tok * N + n8) = d;
+        const uint8_t* get = tbuf + tl * 64 + (((lane & 3) ^ (tl >> 1)) & 3) * 16;
+        __nv_bfloat16* to = y + (size_t)(token0 + tl) * N + n8;
+#pragma unroll
+        for (int c = 0; c < MATS; ++c) {
+            const uint4 d = *reinterpret_cast<const uint4*>(get + 512 * c);
+            if (token0 + tl + 8 * c < M && n8 < N) *reinterpret_cast<uint4*>(to + (size_t)(8 * c) * N) = d;
+        }
         __syncwarp();
     }
-    // A whole tile: round and store.
+    // A whole tile.
     __device__ __forceinline__ void whole(__nv_bfloat16* y, int M, int N, int n0, int token0) const {
-        uint32_t r[8];
-        if (part < chunks) tmem_ld_16x256b_pair(tmem + 8 * part, r);
+        float v[8 * MATS];
+        uint32_t m[MATS][4];
+        if (part < chunks) tmem_ld_16x256b(tmem + 8 * MATS * part, v);
 #pragma unroll 1
         for (int c = part; c < chunks; c += kGroups) {
-            tmem_ld_wait();
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
-            if (c + kGroups < chunks) tmem_ld_16x256b_pair(tmem + 8 * (c + kGroups), r);
-            store(v, y, M, N, n0, token0 + 8 * c);
+            tmem_ld_wait_for(v);
+            round(v, m);
+            if (c + kGroups < chunks) tmem_ld_16x256b(tmem + 8 * MATS * (c + kGroups), v);
+            store(m, y, M, N, n0, token0 + 8 * MATS * c);
         }
     }
-    // Where this lane's eight sums of chunk c lie in a slot (as two float4, 32 apart): a warp moves 512 bytes at a time.
-    __device__ __forceinline__ int slot_index(int quarter, int c) const { return (quarter * chunks + c) * 64 + lane; }
+    // Where this lane's sums of chunk c lie in a slot (as 2 MATS float4, 32 apart): a warp moves 512 bytes at a time.
+    __device__ __forceinline__ int slot_index(int quarter, int c) const { return (quarter * chunks + c) * 64 * MATS + lane; }
     // A contributed part: the fp32 sums as they are.
     __device__ __forceinline__ void contribute(float4* slot, int quarter) const {
 #pragma unroll 1
         for (int c = part; c < chunks; c += kGroups) {
-            uint32_t r[8];
-            tmem_ld_16x256b_pair(tmem + 8 * c, r);
-            tmem_ld_wait();
+            float v[8 * MATS];
+            tmem_ld_16x256b(tmem + 8 * MATS * c, v);
+            tmem_ld_wait_for(v);
             float4* p = slot + slot_index(quarter, c);
-            __stcg(p, make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3])));
-            __stcg(p + 32, make_float4(__uint_as_float(r[4]), __uint_as_float(r[5]), __uint_as_float(r[6]), __uint_as_float(r[7])));
+#pragma unroll
+            for (int i = 0; i < 2 * MATS; ++i) __stcg(p + 32 * i, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
         }
     }
     // The owner of a cut tile: its own sums, then the others' in CTA order (`slots`: the first one's slot, the next ones
-    // `stride` float4 further each), rounded once.  Two chunks of two contributors are asked for together, so the trips to the
-    // L2 are shared by 32 values per lane.
+    // `stride` float4 further each), rounded once.  The parts come one chunk of two contributors at a time, the next ones being on their way
+    // while a chunk is added up, rounded and stored.
     __device__ __forceinline__ void finish(const float4* slots, size_t stride, int others, int quarter, __nv_bfloat16* y, int M, int N, int n0,
                                            int token0) const {
+        float4 x[2][2 * MATS];
+        auto ask = [&](int c, int o) {
+            const float4* p = slots + o * stride + slot_index(quarter, c);
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+                if (o + b < others)
+#pragma unroll
+                    for (int i = 0; i < 2 * MATS; ++i) x[b][i] = load_behind_wait(p + b * stride + 32 * i);
+        };
+        if (part < chunks) ask(part, 0);
 #pragma unroll 1
-        for (int c = part; c < chunks; c += 2 * kGroups) {
-            const bool second = c + kGroups < chunks;
-            float v[2][8];
-            float4 x[2][2][2];
-            auto load = [&](int o) {
-#pragma unroll
-                for (int b = 0; b < 2; ++b)
-#pragma unroll
-                    for (int k = 0; k < 2; ++k)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h)
-                            if (o + b < others && (k == 0 || second))
-                                x[b][k][h] = load_behind_wait(slots + (o + b) * stride + slot_index(quarter, c + k * kGroups) + 32 * h);
-            };
-            load(0);
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                if (k == 1 && !second) break;
-                uint32_t r[8];
-                tmem_ld_16x256b_pair(tmem + 8 * (c + k * kGroups), r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v[k][j] = __uint_as_float(r[j]);
-            }
+        for (int c = part; c < chunks; c += kGroups) {
+            float v[8 * MATS];
+            tmem_ld_16x256b(tmem + 8 * MATS * c, v);
+            tmem_ld_wait_for(v);
+#pragma unroll 1
             for (int o = 0; o < others; o += 2) {
 #pragma unroll
                 for (int b = 0; b < 2; ++b)
+                    if (o + b < others)
 #pragma unroll
-                    for (int k = 0; k < 2; ++k)
-                        if (o + b < others && (k == 0 || second))
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                v[k][4 * h] += x[b][k][h].x; v[k][4 * h + 1] += x[b][k][h].y;
-                                v[k][4 * h + 2] += x[b][k][h].z; v[k][4 * h + 3] += x[b][k][h].w;
-                            }
-                if (o + 2 < others) load(o + 2);
+                        for (int i = 0; i < 2 * MATS; ++i) {
+                            v[4 * i] += x[b][i].x; v[4 * i + 1] += x[b][i].y;
+                            v[4 * i + 2] += x[b][i].z; v[4 * i + 3] += x[b][i].w;
+                        }
+                if (o + 2 < others) ask(c, o + 2);
+                else if (c + kGroups < chunks) ask(c + kGroups, 0);
             }
-            store(v[0], y, M, N, n0, token0 + 8 * c);
-            if (second) store(v[1], y, M, N, n0, token0 + 8 * (c + kGroups));
+            uint32_t m[MATS][4];
+            round(v, m);
+            store(m, y, M, N, n0, token0 + 8 * MATS * c);
         }
     }
 };
@@ -499,8 +506,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap act_map, const uint8_t* __restri
             // segment (those of the group's job before it, in segment last_seg) that waits for that accumulator.
             uint32_t* flags = reinterpret_cast<uint32_t*>(workspace + kGemmFlagOffset) + (warp - kFirstDequant);
             int duty = 0, last_seg = 0;
-            DrainShare share;
-            share.part = group; share.lane = lane; share.chunks = bt / 8;
+            constexpr int kDrainMats = BT > 32 ? 2 : 1;
+            DrainShare<kDrainMats> share;
+            share.part = group; share.lane = lane; share.chunks = bt / (8 * kDrainMats);
             // arrivals on the barriers of the CTA that issues the MMAs
             const auto arrive_issuer = [&](uint64_t* bar) {
                 if constexpr (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(bar), 0));
