@@ -127,3 +127,24 @@ def test_blob_is_tile_major_and_contiguous_per_strip():
     diff = np.nonzero(base != other)[0]
     lo = 256 + (1 * 3 + 1) * 4256
     assert len(diff) == 1 and lo <= diff[0] < lo + 4096
+
+
+@pytest.mark.parametrize("bits,K,N,group,shift", [(4, 2048, 8264, 128, 0), (4, 2048, 8264, 32, 0), (4, 2048, 8264, 128, 8), (8, 1024, 8264, 128, 0), (8, 1024, 8264, 128, 4)])
+def test_large_blobs_are_the_same_bytes_as_their_parts(bits, K, N, group, shift):
+    """From 8 MB on tiles go past the caches, where the blob is 16-byte aligned: columns packed as two smaller blobs and joined give the same."""
+    p = wl.make_w4(1, K, N, seed=K + N, group_size=group) if bits == 4 else wl.make_w8(1, K, N, seed=K + N)
+    size = tf.tf_packed_size(bits, K, N, group)
+    assert size >= 8 << 20
+    raw = np.full(size + 64, 0xA5, dtype=np.uint8)
+    start = -raw.ctypes.data % 16 + shift
+    out = raw[start:start + size]
+
+    def pack(c0, c1, into=None):
+        cut = lambda a, per: np.ascontiguousarray(a[:, c0 // per:c1 // per])  # noqa: E731
+        if bits == 4:
+            return tf.tf_pack_awq(cut(p.qweight, 8), cut(p.scales_f16, 1), cut(p.qzeros, 8), K, c1 - c0, group, out=into)
+        return tf.tf_pack_w8(cut(p.w_i8, 1), cut(p.scales_f16, 1), K, c1 - c0, group, out=into)
+
+    pack(0, N, out)
+    assert np.array_equal(out, tf.tf_pack_concat([pack(0, 4096), pack(4096, N)]))
+    assert (raw[:start] == 0xA5).all() and (raw[start + size:] == 0xA5).all()
