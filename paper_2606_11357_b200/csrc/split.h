@@ -47,11 +47,11 @@ struct Ranges {
 // leave SMs idle.  Split of the (tile, k-tile) units over `grid` CTAs: the owner of a cut tile adds up the others' parts
 // at the end of its range.  The candidates are one CTA per SM, in equal ranges, and, where there are fewer tiles than SMs, every whole
 // number of CTAs per tile; the one with the smallest estimate is taken.  In ns, for a call in a chain: a k-tile 360 + 0.9 bt
-// (dequantization up to about 128 tokens, MMAs above); the drain of the last tile 9 bt, of every other tile of a CTA 15 bt above 128 tokens
-// (one accumulator: nothing runs under it); a cut 1000, storing and reading the parts 9.5 bt + 2 bt for each of the others, and 350 for every trip to
-// the L2 that brings them (two CTAs' parts at a time, 64 tokens at a time); 1200 where more than half of the SMs are taken, as the
-// start of the next call of a chain then no longer hides behind this one.  Fitted to 2900 timings (4-bit and int8, groups of 32 and 128,
-// 20 to 2048 tokens, 0.5 to 67 M weights): 6 % off on average; the choice costs 0.9 % over the best candidate.
+// (dequantization up to about 128 tokens, MMAs above); the drain of the last tile 9 bt, of every other tile of a CTA 12 bt above 128 tokens
+// (one accumulator: nothing runs under it) and 600 below; a cut 1000, storing and reading the parts 9 bt + 2.5 bt for each of the others, and 350 for
+// every trip to the L2 that brings them (two CTAs' parts at a time, 64 tokens at a time); 1100 where more than half of the SMs are taken, as
+// the start of the next call of a chain then no longer hides behind this one.  Fitted to 4700 timings (4-bit and int8, 20 to 3100 tokens,
+// 0.5 to 59 M weights): 6 % off on average; over 400 sizes the choice costs 0.8 % over the best candidate.
 struct GemmSplit {
     int grid, rows;            // CTAs; rows of the grid: one, or one per tile
     bool whole_tiles;
@@ -62,14 +62,14 @@ inline GemmSplit split_gemm(int tiles, int ktiles, int bt, int sm_count) {
     const long long units = (long long)tiles * ktiles;
     const int t_unit = 360 + 9 * bt / 10;
     const auto range = [&](int grid, long long len) {        // a CTA's range of k-tiles, with the drains of all its tiles
-        return len * t_unit + 9 * bt + (bt > 128 ? (len - 1) / ktiles * 15 * bt : 0) + (2 * grid > sm_count ? 1200 : 0);
+        return len * t_unit + 9 * bt + (len - 1) / ktiles * (bt > 128 ? 12 * bt : 600) + (2 * grid > sm_count ? 1100 : 0);
     };
     GemmSplit best;
     best.grid = tiles < sm_count ? tiles : sm_count;
     best.whole_tiles = true;
     best.cost = range(best.grid, (long long)((tiles + best.grid - 1) / best.grid) * ktiles);
     auto consider = [&](int grid, long long others) {        // others: CTAs besides the owner that hold a part of a tile
-        const long long cost = range(grid, (units + grid - 1) / grid) + 1000 + 350 * ((others + 1) / 2) * ((bt + 63) / 64) + 19 * bt / 2 + 2 * others * bt;
+        const long long cost = range(grid, (units + grid - 1) / grid) + 1000 + 350 * ((others + 1) / 2) * ((bt + 63) / 64) + 9 * bt + 5 * others * bt / 2;
         if (cost < best.cost) { best.cost = cost; best.grid = grid; best.whole_tiles = false; }
     };
     for (int per_tile = 2; per_tile * tiles <= sm_count && per_tile <= ktiles; ++per_tile) consider(per_tile * tiles, per_tile - 1);
