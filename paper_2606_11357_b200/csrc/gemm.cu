@@ -27,12 +27,10 @@
 // Work split: whole tiles, or the sequence of (output tile, k-tile) units cut into equal contiguous ranges, one per CTA
 // (split_gemm).  A CTA that computes part of a tile whose last k-tile is another CTA's does that first and writes its fp32 sums
 // to the workspace; the owner of the last k-tile adds them to its own in CTA order (deterministic) and stores y.
-// What bounds it: with 256 tokens the tensor pipe, 73 % active over a launch (inside a tile a k-tile takes 1060 cycles, 1024 of them
-// MMA; start, drains and cuts bring it to about 1400), at a clock that the power limit holds down in a loop (1.4 to 1.6 GHz); up
-// to 128 tokens the issue slots of the dequant warps and the waits of the warp that issues the MMAs (0.43 to 0.6 us per k-tile),
-// for short calls the 4 to 5 us around them.  us per call in a chain: 32x4096x18944 17.9, 96x2944x11016 13.9, 297x2944x11016 26.1,
-// int8 1024x4096x4096 28.2, 512x4096x4096 20.5.  (With eight dequant warps on one k-tile at a time, a packed ring of 26 KB and partial
-// sums through an arrival counter a k-tile took 0.61 to 0.83 us and these calls 24.1, 18.9, 33.5, 32.9 and 31.1.)
+// What bounds it: with 256 tokens the tensor pipe (inside a tile a k-tile takes 1100 cycles in pairs of CTAs, 1024 of them MMA; between two
+// tiles of a CTA the MMAs wait 6400 cycles for the one accumulator), at a clock that the power limit holds down in a loop (1.3 to 1.5 GHz); up
+// to 128 tokens the issue slots of the dequant warps, 70 % used by 509 instructions per warp and k-tile (0.4 us), for short calls the 4 to 5 us
+// around them.  us per call in a chain: 24x4096x14336 15.1, 77x2944x11016 (group 32) 13.4, 128x8192x8192 21.0, int8 1024x4096x4096 31.9.
 // Pairs of CTAs (PAIR): two CTAs of a cluster, on neighbouring SMs, share an output tile of 256 columns x bt tokens.  One MMA of 256 rows
 // (cta_group::2) works on both halves, so each SM loads and holds only half of the activations.  A CTA on its own is bound by what its SM can
 // take from the L2: 64 KB of activations and 8.5 KB of weights per k-tile of 256 tokens, 62 bytes per cycle at 1195 cycles; a pair takes 41 KB and
