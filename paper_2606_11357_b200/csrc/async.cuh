@@ -165,11 +165,12 @@ __device__ __forceinline__ uint32_t cta_rank_in_cluster() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// Arrival on an mbarrier of any CTA of the cluster, and the wait for such arrivals.  For what lies in tensor memory, which tcgen05.wait and
-// tcgen05.fence order: the arrival is a release for the arriving CTA only.  (As a release for the cluster it waits for everything that the thread has on its way:
-// 2700 cycles in the GEMM's dequantization warps, where this takes 50 to 100.)
+// Arrival on an mbarrier of any CTA of the cluster, and the wait for such arrivals.  For what lies in tensor memory: tcgen05.wait has it done,
+// tcgen05.fence::before_thread_sync puts it ahead of the arrival and ::after_thread_sync behind the wait, and for that order the arrival itself may be
+// relaxed, but its scope has to hold the waiting thread, which the default (the arriving CTA) does not.  It orders nothing else.  (As a release for the
+// cluster it waits for everything that the thread has on its way: 2700 cycles in the GEMM's dequantization warps, where this takes 50 to 100.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
     uint32_t done;
