@@ -46,6 +46,7 @@
 #include "async.cuh"
 #include "common.cuh"
 #include "kernels.h"
+#include "rings.h"
 #include "tensormap.h"
 
 namespace tf {
@@ -54,51 +55,9 @@ namespace {
 
 constexpr int kGemmThreads = 640;
 constexpr int kBN = 128;                  // weight columns per CTA tile (two packed strips)
-constexpr int kBK = 64;                   // k of one 128-byte swizzled activation row
-constexpr int kGroups = 4;                // dequantization groups of four warps
 constexpr int kFirstDequant = 4;
 constexpr int kTmemAccCols = 256;
 constexpr int kTmemCols = 512;
-constexpr int kMaxActStages = 8;
-constexpr int kMaxWpStages = 8;
-
-// Packed-weight ring: one stage = a chunk of one or two k-tiles of the two strips.  A chunk goes to one group per k-tile, and
-// the ring is a whole number of rounds of the groups, so a stage always meets the same groups and the parity of its barrier
-// cannot alias.  Narrow token tiles consume weights fast and want 70 to 140 KB of them in flight (with 26 KB a 32-token tile
-// could not take a k-tile faster than one per 0.34 us: the latency of HBM), 4-bit ones in chunks of two: the thread that
-// issues the copies pays about 100 cycles for each.
-__host__ __device__ constexpr int chunk_tiles(int bits, int bt) { return bt > 128 || bits == 8 ? 1 : 2; }
-__host__ __device__ constexpr int wp_stage_bytes(int bits, int bt, int G) { return 2 * chunk_tiles(bits, bt) * tile_bytes(bits, G); }
-// Activations.  Up to 128 tokens a k-tile of them is one stage that goes with an operand stage: one barrier says that both
-// are there and one that both are free, so the warp that issues the MMAs, whose waits and issue set the pace of narrow tiles,
-// pays for one of each per k-tile.  A k-tile of 256 tokens is 64 KB; there the ring is of half k-tiles, with barriers of its own.
-__host__ __device__ constexpr bool tied(int bt) { return bt <= 128; }
-__host__ __device__ constexpr int act_stage_k(int bt) { return tied(bt) ? kTileK : kBK; }
-constexpr int kGemmSmemMax = 227 * 1024;  // dynamic shared memory one CTA may ask for
-constexpr int kDrainWarpBytes = 1024;     // per dequant warp: 16 tokens x 32 columns of bf16, for the drain of an accumulator
-constexpr int kGemmBarrierBytes = 1024;
-constexpr int kGemmSmemFixed = 1024 /*alignment slack*/ + 4 * kGroups * kDrainWarpBytes + kGemmBarrierBytes;
-// The rings share what the fixed part leaves: the activations (of the call's own bt columns) come first where they are tied;
-// otherwise the weights take one round of the groups and the activations the rest.
-struct GemmRings {
-    int act_stage_bytes, act_stages, wp_stages, smem_bytes;
-};
-inline GemmRings gemm_rings(int bits, int BT, int act_rows, int G) {
-    GemmRings r;
-    const int left = kGemmSmemMax - kGemmSmemFixed, wp = wp_stage_bytes(bits, BT, G), round = kGroups / chunk_tiles(bits, BT);
-    r.act_stage_bytes = act_rows * act_stage_k(BT) * 2;
-    if (tied(BT)) {
-        r.act_stages = kGroups;
-        r.wp_stages = (left - r.act_stages * r.act_stage_bytes) / wp / round * round;
-        if (r.wp_stages > kMaxWpStages) r.wp_stages = kMaxWpStages;
-    } else {
-        r.wp_stages = round;
-        r.act_stages = (left - r.wp_stages * wp) / r.act_stage_bytes;
-        if (r.act_stages > kMaxActStages) r.act_stages = kMaxActStages;
-    }
-    r.smem_bytes = kGemmSmemFixed + r.act_stages * r.act_stage_bytes + r.wp_stages * wp;
-    return r;
-}
 
 // workspace: [0,16) status | [kGemmFlagOffset, + 64 * CTAs) "this dequant warp's part of its CTA's slot is filled" | (the GEMV's
 // partial-sum slots, not touched here) | one slot of BT tokens x 128 columns of fp32 sums per CTA (the part of a tile it contributes)
@@ -155,7 +114,7 @@ template <int MATS>
 struct DrainShare {
     uint32_t tmem;             // accumulator, this lane quarter
     int part, lane, chunks;    // chunks = bt / (8 MATS)
-    uint8_t* tbuf;             // 512 MATS bytes of this warp
+    uint8_t* tbuf;             // kDrainWarpBytes of this warp
 
     // A chunk rounded: matrix i of its eight columns c in m[c][i].
     __device__ __forceinline__ static void round(const float (&v)[8 * MATS], uint32_t (&m)[MATS][4]) {
@@ -168,21 +127,20 @@ struct DrainShare {
             }
     }
     // ... and stored.  y wants a token's columns side by side: the matrices are transposed by stmatrix and stored as 16 bytes per lane,
-    // 8 columns of one token.
+    // 8 columns of one token, eight tokens after the other through the same 512 bytes (why no more: kDrainWarpBytes).
     __device__ __forceinline__ void store(const uint32_t (&m)[MATS][4], __nv_bfloat16* y, int M, int N, int n0, int token0) const {
         const int n8 = n0 + 8 * (lane & 3), tl = lane >> 2;
         const uint32_t put = smem_u32(tbuf) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane & 7) >> 1)) & 3) * 16;
-#pragma unroll
-        for (int c = 0; c < MATS; ++c) stmatrix_x4_trans(put + 512 * c, m[c]);
-        __syncwarp();
-        const uint8_t* get = tbuf + tl * 64 + (((lane & 3) ^ (tl >> 1)) & 3) * 16;
+        const uint4* get = reinterpret_cast<const uint4*>(tbuf + tl * 64 + (((lane & 3) ^ (tl >> 1)) & 3) * 16);
         __nv_bfloat16* to = y + (size_t)(token0 + tl) * N + n8;
 #pragma unroll
         for (int c = 0; c < MATS; ++c) {
-            const uint4 d = *reinterpret_cast<const uint4*>(get + 512 * c);
+            stmatrix_x4_trans(put, m[c]);
+            __syncwarp();
+            const uint4 d = *get;
             if (token0 + tl + 8 * c < M && n8 < N) *reinterpret_cast<uint4*>(to + (size_t)(8 * c) * N) = d;
+            __syncwarp();
         }
-        __syncwarp();
     }
     // A whole tile.
     __device__ __forceinline__ void whole(__nv_bfloat16* y, int M, int N, int n0, int token0) const {
