@@ -53,9 +53,10 @@ void write_header(void* out, int bits, int K, int N, int g, size_t total) {
 constexpr int kW4RowBytes = tf::kTileN / 2;          // one k of a 4-bit tile: eight words
 // The next strip's part of a row is asked for while this one's is worked on: a tile reads 128 rows that are kilobytes apart, more than the
 // processor follows by itself, and waited for each of them (4096x14336 4-bit, buffers that are in no cache, 16 cores: 1350 us without, 1110
-// with; two lines ahead is no better).  Behind the end of the matrix it asks for nothing.  int8 only for large blobs: smaller ones mostly lie in
-// caches, where 128 requests per tile only cost (us of one core, buffers reused, asked ahead / not: 512x512 15.5 / 14.1, 640x2128 87.9 / 86.7;
-// buffers that are in no cache, 4096x11008: 3085 / 3320 with 8 cores, 977 / 997 on a machine with more).
+// with; two lines ahead is no better).  The last strip asks for nothing: what lies behind it is another row, or behind the matrix.
+// int8 only for large blobs: smaller ones mostly lie in caches, where 128 requests per tile only cost (us of one core, buffers reused, asked
+// ahead / not: 512x512 15.5 / 14.1, 640x2128 87.9 / 86.7; buffers that are in no cache, 4096x11008: 3085 / 3320 with 8 cores, 977 / 997 on a
+// machine with more).
 constexpr size_t kLine = 64;
 constexpr size_t kLargeBlob = 8 << 20;       // of a size that no cache holds until it is read
 
@@ -275,7 +276,7 @@ extern "C" __attribute__((visibility("default"))) tf_status tf_pack_awq(const ui
         uint8_t* tile = stream ? buffer : dst;
         const uint8_t* src = q + (size_t)k0 * row_bytes + n0 / 2;
         if (n0 + tf::kTileN <= N) {
-            weights_w4(src, row_bytes, tile, S % 2 == 0);       // a line of a row is two strips'
+            weights_w4(src, row_bytes, tile, S % 2 == 0 && S + 2 < strips);       // two strips' parts of a row make a line (of rows that begin with one)
         } else {
             // padded columns: q = z = 0, s = 0  ->  dequantizes to exactly 0
             uint8_t part[tf::kTileK * kW4RowBytes];
@@ -310,7 +311,7 @@ extern "C" __attribute__((visibility("default"))) tf_status tf_pack_w8(const int
         uint8_t* tile = stream ? buffer : dst;
         const uint8_t* src = q + (size_t)k0 * N + n0;
         if (n0 + tf::kTileN <= N) {
-            if (large) weights_w8<true>(src, (size_t)N, tile);
+            if (large && S + 1 < strips) weights_w8<true>(src, (size_t)N, tile);
             else weights_w8<false>(src, (size_t)N, tile);
         } else {
             uint8_t part[tf::kTileK * tf::kTileN];

@@ -55,3 +55,10 @@ def program(tmp_path_factory):
 def test_int8_asks_ahead_for_large_blobs_only(program):
     assert program(8, 512, 512)[0] == 0 and program(8, 2048, 2048)[0] == 0
     assert program(8, 1024, 8256)[0] > 0
+
+
+@pytest.mark.parametrize("bits,K,N", [(4, 256, 64), (4, 256, 128), (4, 256, 192), (4, 256, 200), (4, 256, 520), (4, 1024, 16384 + 64), (8, 1024, 8192), (8, 1024, 8264)])
+def test_nothing_is_asked_for_behind_the_last_strip(program, bits, K, N):
+    count, outside, wrapped = program(bits, K, N)
+    assert (outside, wrapped) == (0, 0)
+    assert count > 0 or N <= 128
