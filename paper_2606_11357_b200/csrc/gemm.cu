@@ -30,12 +30,13 @@
 // What bounds it: with 256 tokens the tensor pipe (inside a tile a k-tile takes 1100 cycles in pairs of CTAs, 1024 of them MMA; between two
 // tiles of a CTA the MMAs wait 6400 cycles for the one accumulator), at a clock that the power limit holds down in a loop (1.3 to 1.5 GHz); up
 // to 128 tokens the issue slots of the dequant warps, 70 % used by 509 instructions per warp and k-tile (0.4 us), for short calls the 4 to 5 us
-// around them.  us per call in a chain: 24x4096x14336 15.1, 77x2944x11016 (group 32) 13.4, 128x8192x8192 21.0, int8 1024x4096x4096 31.9.
+// around them.  us per call in a chain: 24x4096x14336 15.3, 77x2944x11016 (group 32) 13.4, 128x8192x8192 21.3, int8 80x4096x14336 19.1.
 // Pairs of CTAs (PAIR): two CTAs of a cluster, on neighbouring SMs, share an output tile of 256 columns x bt tokens.  One MMA of 256 rows
 // (cta_group::2) works on both halves, so each SM loads and holds only half of the activations.  A CTA on its own is bound by what its SM can
 // take from the L2: 64 KB of activations and 8.5 KB of weights per k-tile of 256 tokens, 62 bytes per cycle at 1195 cycles; a pair takes 41 KB and
-// 1100 cycles, and moves fewer bytes, which under the power limit is worth as much: us, 2048x4096x14336 203.9 -> 193.6, 512x32768x4096
-// 119.6 -> 116.5, 1024x4096x8584 59.6 -> 53.9.  Each CTA unpacks and drains its own 128 columns; CTA 0 issues the MMAs, and the barriers that its MMA
+// 1100 cycles, and moves fewer bytes, which under the power limit is worth as much: us of the kernel as it is, alone -> in pairs, inputs
+// changing, 2048x4096x14336 212.9 -> 196.4, 512x32768x4096 125.7 -> 115.4, int8 1024x4096x4096 34.1 -> 33.1; in a chain 1024x4096x8584 56.2 -> 53.1,
+// 600x8192x8200 71.0 -> 66.9.  Each CTA unpacks and drains its own 128 columns; CTA 0 issues the MMAs, and the barriers that its MMA
 // warp waits on are arrived at by both (choose_gemm_tiling says when).
 // Every mbarrier wait is bounded; on a timeout all roles leave, TMEM is freed, the status word is set.
 #include <cuda.h>
@@ -109,7 +110,8 @@ static_assert(offsetof(GemmBarriers, wait_kcycles) == offsetof(GemmBarriers, abo
 // tokens each: 16, or 8 where that is what gives every group of warps a chunk (32 tokens).  A chunk is read in the fragment layout of 8 x 8
 // matrices (see tmem_ld_16x256b), the next one being on its way out of tensor memory meanwhile.  No MMA runs on a tile of 256 tokens until
 // it is empty, so what counts is the chain of latencies of a chunk, and how few chunks there are (with 8 tokens a tile of 256 took 3700
-// cycles, with 16 2900; a part of a cut one is bound by the L2, 128 KB of every CTA's in 5000 cycles).
+// cycles, with 16 2900, measured with 1 KB per warp, so that its 16 tokens were transposed at once; a part of a cut one is bound by the L2,
+// 128 KB of every CTA's in 5000 cycles).
 template <int MATS>
 struct DrainShare {
     uint32_t tmem;             // accumulator, this lane quarter

@@ -4,7 +4,7 @@
 // What bounds it: memory.  The matrix is read and written once, and the shuffle between is a transposition of nibbles
 // (4-bit) or bytes (int8) inside small blocks that 16-byte vectors do in a few operations per block.  Done code by code
 // (the first form of this file) 4096 x 14336 4-bit weights took 59 ms, bound by about 15 scalar operations per code;
-// now 0.7 ms with 16 cores (90 GB/s read and written).
+// now 0.6 to 0.7 ms with 16 cores (90 to 100 GB/s read and written).
 #include <string.h>
 
 #include <thread>
@@ -140,7 +140,7 @@ inline void weights_w8(const uint8_t* src, size_t row_bytes, uint8_t* tile) {
 }
 
 // A finished tile -> the blob, past the caches: a store that goes through them first fetches the line that it overwrites.  For large blobs,
-// which no cache holds until they are read: 4096x14336 4-bit 1110 -> 1060 us with buffers that are in no cache, 930 to 1390 -> 660 where two
+// which no cache holds until they are read: 4096x14336 4-bit 1110 -> 1060 us with buffers that are in no cache, 930 to 1390 -> 590 to 710 where two
 // pairs of buffers take turns; one pair alone, packed again and again, is slower (0.6 -> 0.8 ms).
 inline void put_tile(uint8_t* dst, const uint8_t* tile, size_t bytes) {
 #ifdef __SSE2__

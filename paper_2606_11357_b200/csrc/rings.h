@@ -11,7 +11,7 @@ constexpr int kMaxWpStages = 8;
 
 // Packed-weight ring: one stage = a chunk of one or two k-tiles of the two strips.  A chunk goes to one group per k-tile, and
 // the ring is a whole number of rounds of the groups, so a stage always meets the same groups and the parity of its barrier
-// cannot alias.  Narrow token tiles consume weights fast and want 70 to 140 KB of them in flight (with 26 KB a 32-token tile
+// cannot alias.  Narrow token tiles consume weights fast and want 66 to 140 KB of them in flight (with 26 KB a 32-token tile
 // could not take a k-tile faster than one per 0.34 us: the latency of HBM), 4-bit ones in chunks of two: the thread that
 // issues the copies pays about 100 cycles for each.
 TF_HD constexpr int chunk_tiles(int bits, int bt) { return bt > 128 || bits == 8 ? 1 : 2; }

@@ -51,7 +51,9 @@ struct Ranges {
 // (one accumulator: nothing runs under it) and 600 below; a cut 1000, storing and reading the parts 9 bt + 2.5 bt for each of the others, and 350 for
 // every trip to the L2 that brings them (two CTAs' parts at a time, 64 tokens at a time); 1100 where more than half of the SMs are taken, as
 // the start of the next call of a chain then no longer hides behind this one.  Fitted to 4700 timings (4-bit and int8, 20 to 3100 tokens,
-// 0.5 to 59 M weights): 6 % off on average; over 400 sizes the choice costs 0.8 % over the best candidate.
+// 0.5 to 59 M weights), for the differences between candidates: over 400 sizes the choice costs 0.8 % over the best one.  It is no time of a call:
+// what every candidate pays is left out, and under the power limit the clock is lower than in the fit.  Of 76 sizes the estimate is 27 % below the time
+// of a chained call up to 10 us, 19 % from 10 to 30, 21 to 22 % above (2 to 50 %; 2048x4096x14336 142 and 168 us, 1024x4096x8584 44 and 53 to 67).
 struct GemmSplit {
     int grid, rows;            // CTAs; rows of the grid: one, or one per tile
     bool whole_tiles;
